@@ -547,6 +547,23 @@ int launch_pairs16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int8_
                    const Pair16Job* d_jobs, uint32_t n_jobs, uint32_t max_n, Scores out);
 int pairs16_wide_rows();
 
+// Explicit pairs as wavefronts of small lane groups (k_pairwave.cu): class of a
+// pair by its query length (ascending cost; group size and rows per block),
+// and one launch over pairs sorted by (class, window length).
+constexpr int WAVE_CLASSES = 11;
+constexpr int WAVE_NONE = 15;      // sort class of pairs that take another path
+__host__ __device__ inline int pair_wave_class(uint64_t m) {
+  if (m <= 128) return m <= 64 ? 0 : m <= 96 ? 1 : 2;
+  if (m <= 256) return m <= 192 ? 3 : 4;
+  if (m <= 512) return m <= 384 ? 5 : 6;
+  if (m <= 1024) return m <= 768 ? 7 : 8;
+  // several bands of 768 or 1,024 rows, whichever computes fewer rows
+  return (m + 767) / 768 * 12 < (m + 1023) / 1024 * 16 ? 9 : 10;
+}
+int launch_pair_wave(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int8_t* d_matrix, int A,
+                     int o, int e, int mode, uint32_t fe, int smax, int smin, const dsa_pair* d_pairs,
+                     const uint32_t* d_order, const uint64_t* class_n, uint32_t max_n, Scores out);
+
 // Device planning of explicit pairs (k_pairplan.cu).
 struct PairPlanParams {
   uint32_t n_queries, n_targets;
@@ -554,6 +571,8 @@ struct PairPlanParams {
   int32_t o, e;
   bool local16;         // local mode with the saturation flag: every size fits
   bool packed_ok;       // the packed int16 form is allowed
+  bool wave;            // packed pairs take the wavefront kernel
+  int32_t smax, smin;
 };
 struct PairPlanStats {   // field order is used by the kernels' atomics
   uint64_t cells;        // cells of all valid pairs
@@ -563,7 +582,10 @@ struct PairPlanStats {   // field order is used by the kernels' atomics
   uint64_t n_jobs;       // packed jobs (two pairs of equal query length each)
   uint32_t max_t_len;    // longest window of a valid pair
   uint32_t pad;
+  uint64_t cls[16];      // wave: packed pairs of each class
 };
+// A valid pair of m x n takes the packed kernel the call chose.
+bool pair_packed(const PairPlanParams& P, uint64_t m, uint64_t n);
 // Range check, class, sort key ((m << 32) | t_len) and value (pair index) of
 // every packed pair; hist[m] = packed pairs of query length m, jcnt[m] = their
 // jobs; L = longest query + 2 entries (the last stays 0).

@@ -82,11 +82,15 @@ struct PairPass {
   const dsa_pair* d_pairs = nullptr;  // device copy (the caller's own when on the device)
   DevBuf d_pairs_buf, d_key, d_idx, d_hist, d_jcnt, d_stats;
   PairPlanStats pst{};
+  PairPlanParams plan{};
   uint64_t L = 0;                     // query lengths 0 .. L-1 are counted
   std::vector<dsa_pair> hp;           // host copy, made only when the host planner needs it
   bool hp_ready = false;
   int need_hp(dsa_ctx* ctx);
 };
+// The call's short pairs take the wavefront kernel (k_pairwave.cu).
+bool pairs_take_wave(const int8_t* matrix, int A, int mode, int o, int e, const Validated& v,
+                     uint64_t n_pairs, bool local16, bool packed_ok);
 // Upload (unless on the device), range-check and classify the pairs.
 int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairPlanParams& P,
                    PairPass& pp);

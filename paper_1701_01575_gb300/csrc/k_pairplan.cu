@@ -5,7 +5,7 @@
 // packed int16 pairs kernel are all computed on the device, so the host
 // touches no per-pair data.  The host planner in api.cu stays the path for
 // calls that hold long or int32 pairs; both produce the same job list.
-#include "dsa_internal.cuh"
+#include "pairwave.cuh"
 
 namespace dsa {
 namespace {
@@ -25,9 +25,21 @@ __device__ __forceinline__ uint32_t warp_max(uint32_t v) {
   return v;
 }
 
+// A valid pair of m x n takes the packed kernel the call chose: the wavefront
+// form admits every pair whose values provably fit (or, in local mode, can be
+// flagged), the two-pairs-per-thread form a narrower range.
+__host__ __device__ inline bool takes_packed(const PairPlanParams& P, uint64_t m, uint64_t n) {
+  if (!P.packed_ok || m < 1 || n < 1 || m * n >= LONG_PAIR_CELLS) return false;
+  if (P.local16) return true;
+  if (P.wave) return pair_wave_range_ok((int64_t)m, (int64_t)n, P.o, P.e, P.smax, P.smin);
+  return (int64_t)(m + n) * P.w16 + P.o < 12000 && P.o + P.e < 4096;
+}
+
 // One pass over the pairs: range check (smallest bad index), the class of
 // every pair, the sort key (m << 32 | t_len) of every packed pair, the number
-// of packed pairs of every query length, and the call's totals.
+// of packed pairs of every query length, and the call's totals.  Wavefront
+// form: key (class << 32 | t_len) of every pair (WAVE_NONE: another path) and
+// the number of packed pairs of every class.
 __global__ void __launch_bounds__(PLAN_T) k_pair_classify(
     const dsa_pair* __restrict__ pairs, uint64_t n, const uint32_t* __restrict__ q_len,
     const uint32_t* __restrict__ db_len, PairPlanParams P, uint64_t* __restrict__ key,
@@ -54,15 +66,17 @@ __global__ void __launch_bounds__(PLAN_T) k_pair_classify(
         const uint64_t c = m * p.t_len;
         cells += c;
         max_t = max(max_t, p.t_len);
-        const bool fits16 =
-            P.local16 || ((int64_t)(m + p.t_len) * P.w16 + P.o < 12000 && P.o + P.e < 4096);
-        if (P.packed_ok && fits16 && m >= 1 && c < LONG_PAIR_CELLS) {
-          key[k] = (m << 32) | p.t_len;
+        if (takes_packed(P, m, p.t_len)) {
+          hm = P.wave ? (uint32_t)pair_wave_class(m) : (uint32_t)m;
+          key[k] = ((uint64_t)hm << 32) | p.t_len;
           idx[k] = (uint32_t)k;
           c16 += c;
-          hm = (uint32_t)m;
         } else {
           ++n_other;
+          if (P.wave) {
+            key[k] = ((uint64_t)WAVE_NONE << 32) | p.t_len;
+            idx[k] = (uint32_t)k;
+          }
         }
       }
     }
@@ -233,15 +247,18 @@ int bits_of(uint64_t v) {
 
 }  // namespace
 
+bool pair_packed(const PairPlanParams& P, uint64_t m, uint64_t n) { return takes_packed(P, m, n); }
+
 int launch_pair_classify(dsa_ctx* ctx, const dsa_pair* d_pairs, uint64_t n, const dsa_db* qs,
                          const dsa_db* db, const PairPlanParams& P, uint64_t* d_key,
                          uint32_t* d_idx, uint64_t* d_hist, uint64_t L, uint64_t* d_jcnt,
                          PairPlanStats* d_stats) {
   if (n) {
-    k_pair_classify<<<plan_grid(ctx, n), PLAN_T, 0, ctx->stream>>>(d_pairs, n, qs->d_len, db->d_len,
-                                                                   P, d_key, d_idx, d_hist, d_stats);
+    k_pair_classify<<<plan_grid(ctx, n), PLAN_T, 0, ctx->stream>>>(
+        d_pairs, n, qs->d_len, db->d_len, P, d_key, d_idx, P.wave ? d_stats->cls : d_hist, d_stats);
     DSA_TRY(launched(ctx, "pair classify"));
   }
+  if (P.wave) return DSA_OK;
   k_pair_jobs_per_len<<<plan_grid(ctx, L), PLAN_T, 0, ctx->stream>>>(d_hist, L, d_jcnt, d_stats);
   return launched(ctx, "pair jobs per length");
 }

@@ -1,0 +1,406 @@
+// Explicit pairs as small wavefronts, packed int16x2: a group of G lanes (2
+// to 32, a power of two) aligns one pair (Sec. II.B.1; any of the three
+// algorithms of Sec. II.C.2).  Shared by the planned kernel (k_pairwave.cu)
+// and the allocation-free entry point (k_noalloc.cu).
+//
+// Layout.  The query's rows are cut into blocks of R rows; lane k of the group
+// owns blocks 2k (low 16-bit halves) and 2k + 1 (high halves).  At step s the
+// low half works on target column s - 2k and the high half on the column
+// before it, so a block's top row is the bottom row that the block above
+// computed one step earlier: one shuffle each for H and F, joined with the
+// lane's own low half by a byte permute.  A pair therefore keeps G lanes busy
+// from its first column on, where one thread per pair leaves most of the chip
+// idle unless there are hundreds of thousands of pairs, and takes as long as
+// its longest pair.  2 G R rows make a band; further bands are chained through
+// one boundary row.
+//
+// Substitution scores come from a profile of the lane's own 2R rows in shared
+// memory, a byte per (residue, row): two loads per step give all rows of both
+// blocks (the halves are on different columns, so on different residues), and
+// one byte permute per packed cell joins and sign-extends them.  Planes of 16
+// bytes per lane keep a quarter-warp's loads in different banks whatever
+// residues they hold.  No lane reads another lane's profile.
+//
+// Anchoring.  The query is shifted down by (R - m mod R) mod R padding rows,
+// so that row m is the last row of one block; padding rows reproduce row 0.
+// Columns before the window (lanes start one after another) and past its end
+// hold the padding residue: before the window a block's column-0 state is a
+// fixed point of the update with it, so no step needs a bounds test.
+//
+// Cell update, local (offset binary, Ho = H - o, as in the inter-sequence
+// kernel):  E = max(E - e, Ho_left);  t = max(Ho_diag + (S + o), E);
+//   H = max(t, F, 0);  Ho = H - o;  F' = max(F - e, Ho).
+// Cell update, global and semi-global: every value is kept with e (i + j)
+// added, so extending a gap adds nothing, and E and F of the next cell are one
+// operation each; with G = value + e (i + j) and P = S + 2e + K >= 0:
+//   x = Gk_diag + P;  G = max(x, E, F);  Gk = G - K;
+//   E' = max(Gk + (K + e - o), E);  F' = max(Gk + (K + e - o), F)
+// The two sums are plain 32-bit additions: no half leaves [0, 2^16), so
+// nothing carries from one into the other.  Three of the five operations are
+// maxima on the half-rate pipe, against four of five before.
+//
+// Range.  Local: the saturation rule of the other packed kernels (a best above
+// 32767 - max S is rerun in int32 by the caller).  Global and semi-global:
+// values with e (i + j) added lie between -3o (less e for each column a lane
+// starts before the window) and max(S, 0) min(m, n) + e (m + n + margin);
+// pair_wave_range_ok() admits only pairs whose values fit 16 bits, so nothing
+// is ever rerun.
+#pragma once
+#include "dsa_internal.cuh"
+#include "dpx.cuh"
+
+namespace dsa {
+
+constexpr int WAVE_WARPS = 4;             // warps per CTA, each on its own
+constexpr int WAVE_SM_PITCH = 36;         // bytes per row of the score table (spreads the banks)
+constexpr int WAVE_PLANE = 32 * 16;       // profile bytes per residue and half
+constexpr int WAVE_RESIDUE = 2 * WAVE_PLANE;
+
+struct WaveParams {
+  int A, o, e, mode;
+  uint32_t fe;
+  int K, bias;      // global / semi-global: see above
+};
+
+// K of the global / semi-global update: every table byte is at least 0.
+__host__ __device__ inline int pair_wave_K(int o, int e, int smin) {
+  int k = -(smin + 2 * e);
+  if (o - 2 * e > k) k = o - 2 * e;
+  return k > 0 ? k : 0;
+}
+// The stored value of 0 at cell (0, 0): values fall by 3o below the boundary's
+// and by e for each of the up to 63 columns a lane starts before the window.
+__host__ __device__ inline int pair_wave_bias(int o, int e, int K) { return 4 * o + 64 * e + K + 64; }
+// The byte tables hold every score of this scoring.
+__host__ __device__ inline bool pair_wave_tables_ok(bool local, int o, int e, int smax, int smin) {
+  if (local) return o >= 1 && o + smax <= 127 && o + smin >= -128;
+  const int K = pair_wave_K(o, e, smin);
+  return (smax > 0 ? smax : 0) + 2 * e + K <= 127;
+}
+// A pair of m x n fits the packed global / semi-global range.
+__host__ __device__ inline bool pair_wave_range_ok(int64_t m, int64_t n, int o, int e, int smax,
+                                                   int smin) {
+  const int K = pair_wave_K(o, e, smin);
+  const int64_t up = (int64_t)(smax > 0 ? smax : 0) * (m < n ? m : n) + (int64_t)e * (m + n + 256);
+  return up + pair_wave_bias(o, e, K) + 512 < 65536;
+}
+
+// Shared-memory bytes of a CTA: the score table, then per warp the profile
+// and (local) the parked columns.
+__host__ __device__ inline uint32_t pair_wave_table_bytes(int A) {
+  return ((uint32_t)(A + 2) * WAVE_SM_PITCH + 127u) / 128u * 128u;
+}
+__host__ __device__ inline uint32_t pair_wave_warp_bytes(int A, bool local) {
+  return (uint32_t)(A + 1) * WAVE_RESIDUE + (local ? 2u * 16u * 32u * 2u : 0u);
+}
+
+#ifdef __CUDACC__
+
+// Score table rows by query residue (row A: padding rows above the query, row
+// A + 1: rows below it), bytes by target residue (entry A: the padding
+// residue).  S(q, a) is the caller's matrix.
+template <bool LOCAL, class Fn>
+__device__ __forceinline__ void pair_wave_table(const WaveParams& W, uint8_t* tab, Fn S) {
+  const bool sg = W.mode == DSA_SEMIGLOBAL;
+  const bool qb = sg && (W.fe & DSA_FREE_Q_BEGIN), tb = sg && (W.fe & DSA_FREE_T_BEGIN);
+  const int z = 2 * W.e + W.K;   // S = 0
+  for (int x = threadIdx.x; x < (W.A + 2) * (WAVE_SM_PITCH); x += blockDim.x) {
+    const int q = x / WAVE_SM_PITCH, a = x % WAVE_SM_PITCH;
+    int v = LOCAL ? -128 : 0;
+    if (q < W.A && a < W.A) v = LOCAL ? S(q, a) + W.o : S(q, a) + z;
+    else if (!LOCAL && q < W.A && a == W.A) v = qb ? z : z - W.o;
+    else if (!LOCAL && q == W.A) v = (a == W.A || tb) ? z : z - W.o;
+    tab[x] = (uint8_t)(int8_t)v;
+  }
+}
+
+// One warp, 32 / G pairs (group g = lane / G; m = n = 0: no pair).  q, t, m, n,
+// scr (the group's boundary row, for queries of more than one band) and the
+// outputs are the group's; the result is valid on the group's first lane:
+// local: score and 1-based end cell (0 when nothing scores); others: score and
+// end cell (i, j) with i in 0..m, j in 0..n.
+template <bool LOCAL, int R>
+__device__ __forceinline__ void pair_wave_run(const WaveParams& W, const uint8_t* tab, uint8_t* prof,
+                                              uint16_t* park, int G, const uint8_t* q,
+                                              const uint8_t* t, int m, int n, uint32_t* scr,
+                                              int& out_s, int& out_i, int& out_j) {
+  static_assert(R % 4 == 0 && R <= 16, "rows per block");
+  constexpr unsigned FULL = 0xFFFFFFFFu;
+  constexpr uint32_t BIAS2 = 0x80008000u;
+  const int lane = threadIdx.x & 31, k = lane & (G - 1);
+  const int o = W.o, e = W.e, A = W.A;
+  const bool sg = W.mode == DSA_SEMIGLOBAL;
+  const bool qb_free = sg && (W.fe & DSA_FREE_Q_BEGIN), qe_free = sg && (W.fe & DSA_FREE_Q_END);
+  const bool tb_free = sg && (W.fe & DSA_FREE_T_BEGIN), te_free = sg && (W.fe & DSA_FREE_T_END);
+  const uint32_t neg_e2 = pack2(-e, -e), o2 = pack2(o, 0) + ((uint32_t)o << 16);
+  const uint32_t K2 = (uint32_t)W.K * 0x10001u;
+  const uint32_t c2 = pack2(W.K + e - o, W.K + e - o);
+  const uint32_t mo2 = pack2(-o, -o) ^ BIAS2;   // local: H = 0 as H - o
+  const int pad = (R - m % R) % R, mp = m + pad;
+  const int band = 2 * G * R;
+  const int nb = (mp + band - 1) / band;
+  int nbmax = nb, nmax = n;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    nbmax = max(nbmax, __shfl_xor_sync(FULL, nbmax, s));
+    nmax = max(nmax, __shfl_xor_sync(FULL, nmax, s));
+  }
+  // value of H at column 0, row i' (padded rows, 1-based; row 0 and padding
+  // rows: 0), and of F entering row i' + 1 there, with e (i' + j) added
+  auto hv = [&](int i, int j) {
+    const int h = (i <= pad || qb_free) ? 0 : -(o + (i - pad - 1) * e);
+    return W.bias + h + e * (i + j) - W.K;
+  };
+  auto fv = [&](int i, int j) {
+    const int f = (i <= pad || qb_free) ? -o : -(o + (i - pad) * e);
+    return W.bias + f + e * (i + 1 + j);
+  };
+  auto row0 = [&](int j) { return (j == 0 || tb_free) ? 0 : -(o + (j - 1) * e); };
+
+  // local: running best per half.  others: column n's best (free query end),
+  // H[m][n] and row m's best column, held by the lane that has them
+  int best_lo = 0, best_hi = 0, bj_lo = 0, bj_hi = 0, bi_lo = 0, bi_hi = 0;
+  int cb = qe_free ? row0(n) : INT32_MIN, ci = 0, hmn = INT32_MIN, rj = 0;
+  int rbest = INT32_MIN;
+  uint8_t* const plo = prof + lane * 16;
+  const int jl0 = -2 * k;   // the low half's column before step 1
+
+  for (int b = 0; b < nbmax; ++b) {
+    const int base = b * band + 2 * k * R;   // rows above the low block
+    // ---- the lane's profile ----
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const uint32_t* row[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = base + x * R + r - pad;   // 0-based query row
+        const int c = i < 0 ? A : (i < m ? (int)q[i] : A + 1);
+        row[r] = reinterpret_cast<const uint32_t*>(tab + c * WAVE_SM_PITCH);
+      }
+      for (int a = 0; a <= A; a += 4) {
+        uint32_t w[4][4];
+#pragma unroll
+        for (int g = 0; g < R / 4; ++g) {   // 4 rows x 4 residues, transposed
+          const uint32_t w0 = row[4 * g][a / 4], w1 = row[4 * g + 1][a / 4];
+          const uint32_t w2 = row[4 * g + 2][a / 4], w3 = row[4 * g + 3][a / 4];
+          const uint32_t p0 = prmt(w0, w1, 0x5140), p1 = prmt(w0, w1, 0x7362);
+          const uint32_t p2 = prmt(w2, w3, 0x5140), p3 = prmt(w2, w3, 0x7362);
+          w[0][g] = prmt(p0, p2, 0x5410);
+          w[1][g] = prmt(p0, p2, 0x7632);
+          w[2][g] = prmt(p1, p3, 0x5410);
+          w[3][g] = prmt(p1, p3, 0x7632);
+        }
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          if (a + y <= A) {
+            uint8_t* dst = plo + (a + y) * WAVE_RESIDUE + x * WAVE_PLANE;
+            if (R == 8)
+              *reinterpret_cast<uint2*>(dst) = make_uint2(w[y][0], w[y][1]);
+            else
+              *reinterpret_cast<uint4*>(dst) =
+                  make_uint4(w[y][0], w[y][1], w[y][2], R == 16 ? w[y][3] : 0u);
+          }
+      }
+    }
+    // ---- column-0 state ----
+    uint32_t Ho[R], E[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (LOCAL) {
+        Ho[r] = mo2;
+        E[r] = pack2(NEG16, NEG16) ^ BIAS2;
+      } else {
+        Ho[r] = pack2(hv(base + r + 1, jl0), hv(base + R + r + 1, jl0 - 1));
+        E[r] = add2(Ho[r], c2);   // E of column 1 opens from column 0
+      }
+    }
+    uint32_t diag = LOCAL ? mo2 : pack2(hv(base, jl0), hv(base + R, jl0 - 1));
+    uint32_t sendH = Ho[R - 1];
+    uint32_t sendF = LOCAL ? mo2 : pack2(fv(base + R, jl0), fv(base + 2 * R, jl0 - 1));
+    // row m's best so far as a threshold that moves with e j (a half that does
+    // not hold row m: never passed); the candidate (m, 0) starts it
+    uint32_t rthr = 0xFFFFFFFFu, rinc = 0;
+    const bool own_lo = !LOCAL && m > 0 && base + R == mp;
+    const bool own_hi = !LOCAL && m > 0 && base + 2 * R == mp;
+    if (te_free && own_lo) { rthr = 0xFFFF0000u | (uint32_t)hv(mp, jl0); rinc = (uint32_t)e; }
+    if (te_free && own_hi) { rthr = 0x0000FFFFu | (uint32_t)hv(mp, jl0 - 1) << 16; rinc = (uint32_t)e << 16; }
+    uint32_t thr2 = 0xFFFFFFFFu;
+    auto set_thr = [&]() {
+      if (LOCAL && b < nb) thr2 = pack2(max(best_lo - 1, 0), max(best_hi - 1, 0)) ^ BIAS2;
+    };
+    set_thr();
+    int pend = 0;
+    // lane 0's input row: row 0, or the band above
+    uint32_t inw = 0;
+    const bool keep = b + 1 < nb && k == G - 1;   // this band's bottom row is read again
+    uint32_t topc = 0;                            // row 0 at column j: G - K
+    if (!LOCAL) topc = (uint32_t)(W.bias - W.K + (tb_free ? e : e - o));
+    if (b > 0 && k == 0 && n > 0) inw = scr[0];
+    // residues one column ahead
+    auto code = [&](int j) -> uint32_t {
+      return (uint32_t)(j - 1) < (uint32_t)n ? (uint32_t)t[j - 1] * WAVE_RESIDUE
+                                              : (uint32_t)A * WAVE_RESIDUE;
+    };
+    uint32_t a_hi = (uint32_t)A * WAVE_RESIDUE, a_lo = code(jl0 + 1);
+    const int steps = nmax + 2 * G - 1;
+    int j = jl0;
+    for (int s = 1; s <= steps; ++s) {
+      ++j;   // the low half's column; the high half's is j - 1
+      const uint32_t a_next = code(j + 1);
+      uint32_t upH = __shfl_up_sync(FULL, sendH, 1);
+      uint32_t upF = __shfl_up_sync(FULL, sendF, 1);
+      if (k == 0) {
+        if (b == 0) {
+          upH = LOCAL ? mo2 : topc << 16;
+          upF = LOCAL ? mo2 : (topc + (uint32_t)(W.K + e - o)) << 16;
+          if (!LOCAL && tb_free) topc += (uint32_t)e;
+        } else {
+          upH = inw << 16;
+          upF = inw & 0xFFFF0000u;
+          if (s < n) inw = scr[s];
+        }
+      }
+      const uint32_t topH = prmt(upH, sendH, 0x5432);
+      uint32_t F = prmt(upF, sendF, 0x5432);
+      uint32_t pl[4], ph[4];
+      if (R == 8) {
+        const uint2 v = *reinterpret_cast<const uint2*>(plo + a_lo);
+        const uint2 u = *reinterpret_cast<const uint2*>(plo + WAVE_PLANE + a_hi);
+        pl[0] = v.x; pl[1] = v.y; ph[0] = u.x; ph[1] = u.y;
+      } else {
+        const uint4 v = *reinterpret_cast<const uint4*>(plo + a_lo);
+        const uint4 u = *reinterpret_cast<const uint4*>(plo + WAVE_PLANE + a_hi);
+        pl[0] = v.x; pl[1] = v.y; pl[2] = v.z; pl[3] = v.w;
+        ph[0] = u.x; ph[1] = u.y; ph[2] = u.z; ph[3] = u.w;
+      }
+      a_hi = a_lo;
+      a_lo = a_next;
+      uint32_t d = diag;
+      diag = topH;
+      uint32_t cm = BIAS2, hprev = BIAS2;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const uint32_t bsel = r & 3;
+        const uint32_t sp = prmt(pl[r / 4], ph[r / 4],
+                                 bsel | (8 + bsel) << 4 | (4 + bsel) << 8 | (12 + bsel) << 12);
+        const uint32_t old = Ho[r];
+        if (LOCAL) {
+          E[r] = addmax2u(E[r], neg_e2, old);
+          const uint32_t x = addmax2u(d, sp, E[r]);
+          const uint32_t h = max3_2u(x, F, BIAS2);
+          Ho[r] = h - o2;
+          F = addmax2u(F, neg_e2, Ho[r]);
+          if (r & 1) cm = max3_2u(cm, hprev, h);
+          else hprev = h;
+        } else {
+          const uint32_t h = max3_2u(d + sp, E[r], F);
+          const uint32_t hk = h - K2;
+          Ho[r] = hk;
+          E[r] = addmax2u(hk, c2, E[r]);
+          F = addmax2u(hk, c2, F);
+        }
+        d = old;
+      }
+      sendH = Ho[R - 1];
+      sendF = F;
+      if (keep && (uint32_t)(j - 2) < (uint32_t)n) scr[j - 2] = prmt(sendH, sendF, 0x7632);
+      if (LOCAL) {
+        if (__vmaxu2(cm, thr2) != thr2) {
+          const int cl = lo16(cm ^ BIAS2), ch = hi16(cm ^ BIAS2);
+          if (cl > best_lo - (j < bj_lo ? 1 : 0)) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) park[r * 32 + lane] = (uint16_t)(Ho[r] ^ BIAS2);
+            best_lo = cl; bj_lo = j; pend |= 1;
+          }
+          if (ch > best_hi - (j - 1 < bj_hi ? 1 : 0)) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) park[(16 + r) * 32 + lane] = (uint16_t)((Ho[r] ^ BIAS2) >> 16);
+            best_hi = ch; bj_hi = j - 1; pend |= 2;
+          }
+          set_thr();
+        }
+      } else {
+        if (te_free) {
+          rthr += rinc;
+          if (__vmaxu2(sendH, rthr) != rthr) {
+            const int jj = own_lo ? j : j - 1;
+            if (jj >= 1 && jj <= n) {
+              rthr = own_lo ? (rthr & 0xFFFF0000u) | (sendH & 0xFFFFu)
+                            : (rthr & 0x0000FFFFu) | (sendH & 0xFFFF0000u);
+              rj = jj;
+              rbest = (int)(own_lo ? sendH & 0xFFFFu : sendH >> 16) + W.K - W.bias - e * (mp + jj);
+            }
+          }
+        }
+        if ((uint32_t)(j - n) <= 1u) {   // column n, low half then high half
+          const int x = j - n, sh = 16 * x;
+          if (x ? own_hi : own_lo)
+            hmn = (int)((sendH >> sh) & 0xFFFFu) + W.K - W.bias - e * (mp + n);
+          if (qe_free) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              const int i = base + x * R + r + 1;
+              const int v = (int)((Ho[r] >> sh) & 0xFFFFu) + W.K - W.bias - e * (i + n);
+              if (i > pad && i <= mp && v > cb) { cb = v; ci = i - pad; }
+            }
+          }
+        }
+      }
+    }
+    if (!LOCAL && te_free && (own_lo || own_hi) && rj == 0)
+      rbest = qb_free ? 0 : -(o + (m - 1) * e);   // (m, 0) was never passed
+    if (LOCAL) {   // rows of the parked columns
+      if (pend & 1) {
+        const uint16_t want = (uint16_t)(best_lo - o);
+        int rr = 0;
+        for (int r = R - 1; r >= 0; --r)
+          if (park[r * 32 + lane] == want) rr = r;
+        bi_lo = base + rr + 1 - pad;
+      }
+      if (pend & 2) {
+        const uint16_t want = (uint16_t)(best_hi - o);
+        int rr = 0;
+        for (int r = R - 1; r >= 0; --r)
+          if (park[(16 + r) * 32 + lane] == want) rr = r;
+        bi_hi = base + R + rr + 1 - pad;
+      }
+    }
+    __syncwarp();
+  }
+  if (LOCAL) {
+    if (best_hi > best_lo || (best_hi == best_lo && best_hi > 0 &&
+                              (bj_hi < bj_lo || (bj_hi == bj_lo && bi_hi < bi_lo)))) {
+      best_lo = best_hi; bj_lo = bj_hi; bi_lo = bi_hi;
+    }
+    for (int w = G / 2; w > 0; w >>= 1) {
+      const int s2 = __shfl_xor_sync(FULL, best_lo, w);
+      const int j2 = __shfl_xor_sync(FULL, bj_lo, w);
+      const int i2 = __shfl_xor_sync(FULL, bi_lo, w);
+      if (s2 > best_lo || (s2 == best_lo && s2 > 0 && (j2 < bj_lo || (j2 == bj_lo && i2 < bi_lo)))) {
+        best_lo = s2; bj_lo = j2; bi_lo = i2;
+      }
+    }
+    out_s = best_lo;
+    out_i = best_lo > 0 ? bi_lo : 0;
+    out_j = best_lo > 0 ? bj_lo : 0;
+  } else {
+    for (int w = G / 2; w > 0; w >>= 1) {
+      const int s2 = __shfl_xor_sync(FULL, cb, w), i2 = __shfl_xor_sync(FULL, ci, w);
+      if (s2 > cb || (s2 == cb && i2 < ci)) { cb = s2; ci = i2; }
+      // one lane holds row m
+      hmn = max(hmn, __shfl_xor_sync(FULL, hmn, w));
+      const int r2 = __shfl_xor_sync(FULL, rbest, w), rj2 = __shfl_xor_sync(FULL, rj, w);
+      if (r2 > rbest) { rbest = r2; rj = rj2; }
+    }
+    int bs = hmn, bi = m, bj = n;   // (m, n); then column n, then row m
+    if (qe_free && (cb > bs || (cb == bs && ci < bi))) { bs = cb; bi = ci; }
+    if (te_free && (rbest > bs || (rbest == bs && rj < bj))) { bs = rbest; bi = m; bj = rj; }
+    out_s = bs;
+    out_i = bi;
+    out_j = bj;
+  }
+}
+
+#endif  // __CUDACC__
+
+}  // namespace dsa

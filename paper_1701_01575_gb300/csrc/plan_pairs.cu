@@ -7,6 +7,7 @@
 // the rest on the exact int32 kernel, and local packed pairs that saturate
 // are rerun exactly in int32.
 #include "host_util.cuh"
+#include "pairwave.cuh"
 
 #include <algorithm>
 #include <numeric>
@@ -16,6 +17,13 @@
 #include <string>
 
 namespace dsa {
+
+// Pairs of a byte-permute scoring (DNA) that still take the wavefront form.
+// Reads of 150 bp in 500 bp windows, wavefront against per-thread form (ms):
+// semi-global 1,000 pairs 0.15 / 1.12, 60,000 1.28 / 1.63, 120,000 2.52 /
+// 2.57, 200,000 4.17 / 3.97; local 60,000 1.64 / 1.79, 120,000 3.25 / 2.92.
+// Reads of 150 and 250 bp mixed break even near 300,000 and 150,000.
+constexpr uint64_t WAVE_MAX_SHORT_PAIRS = 160000, WAVE_MAX_SHORT_PAIRS_LOCAL = 100000;
 
 int PairPass::need_hp(dsa_ctx* ctx) {
   if (hp_ready) return DSA_OK;
@@ -32,11 +40,27 @@ int PairPass::need_hp(dsa_ctx* ctx) {
   return DSA_OK;
 }
 
+// Which packed kernel a call's short pairs take.  The wavefront form keeps 4
+// to 32 lanes on a pair, the other one thread on two pairs (equal lengths,
+// byte-permute scores), which needs hundreds of thousands of pairs to fill
+// the chip but then spends nothing on hand-overs between lanes.
+bool pairs_take_wave(const int8_t* matrix, int A, int mode, int o, int e, const Validated& v,
+                     uint64_t n_pairs, bool local16, bool packed_ok) {
+  if (!packed_ok || (mode == DSA_LOCAL && !local16) || n_pairs > UINT32_MAX) return false;
+  if (!pair_wave_tables_ok(mode == DSA_LOCAL, o, e, v.smax, v.smin)) return false;
+  if (A > 4 || !s_plus_o_fits_int8(matrix, A, o)) return true;
+  // DSA_PAIRS_ROWS fixes a variant of the per-thread form, and re-tuning times it
+  const char* tune = getenv("DSA_AUTOTUNE");
+  if (getenv("DSA_PAIRS_ROWS") || (tune && std::string(tune) == "retune")) return false;
+  return n_pairs < (mode == DSA_LOCAL ? WAVE_MAX_SHORT_PAIRS_LOCAL : WAVE_MAX_SHORT_PAIRS);
+}
+
 int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairPlanParams& P,
                    PairPass& pp) {
   const uint64_t n_pairs = pp.n_pairs;
   pp.L = (uint64_t)qs->max_len + 2;
   const uint64_t L = pp.L;
+  pp.plan = P;
   if (pp.flags & DSA_PAIRS_ON_DEVICE) {
     pp.d_pairs = pp.pairs;
   } else {
@@ -76,7 +100,9 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
   uint64_t scr = 0, cells = 0, lcells = 0, p16cells = 0;
   uint64_t bnd = 0, prog = 0, cand = 0;
   const int band = long_band_rows(), ckpt = long_ckpt_rows();
-  // every pair packed: the device planner lays out the jobs
+  // every pair packed: the device planner lays out the jobs (the wavefront
+  // form's pairs are always planned on the device)
+  const bool wave = pp.plan.wave;
   const bool dev_plan = n_pairs > 0 && pp.pst.n_other == 0;
   // host planner: classify on host threads: packed pairs (filled in place,
   // pair order kept); long and int32 pairs are few and follow serially
@@ -97,8 +123,7 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
         const uint64_t m = qs->h_len[p.query_id];
         const uint64_t c = m * p.t_len;
         cl += c;
-        const bool fits16 = local16 || ((int64_t)(m + p.t_len) * w16 + o < 12000 && o + e < 4096);
-        if (packed_ok && fits16 && m >= 1 && p.t_len >= 1 && c < LONG_PAIR_CELLS) {
+        if (pair_packed(pp.plan, m, p.t_len)) {
           cls[k] = C_P16;
           ++n;
           c16 += c;
@@ -115,8 +140,8 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
       cells += cells_t[t];
       p16cells += c16_t[t];
     }
-    p16.resize(n16[T]);
-    parallel_for(n_pairs, T, [&](unsigned t, size_t b, size_t x1) {
+    if (!wave) p16.resize(n16[T]);
+    if (!wave) parallel_for(n_pairs, T, [&](unsigned t, size_t b, size_t x1) {
       uint64_t pos = n16[t];
       for (size_t k = b; k < x1; ++k)
         if (cls[k] == C_P16) p16[pos++] = k;
@@ -272,10 +297,27 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
     res->phase_cells[PH_INTRA] = lcells;
     res->phase_cells[PH_INT32] = cells - lcells;
   }
-  if (dev_plan || !p16.empty()) {
+  const uint64_t n_wave = wave ? n_pairs - pp.pst.n_other : 0;
+  if (n_wave || (!wave && dev_plan) || !p16.empty()) {
     DevBuf d_pj;
     uint32_t n_pj = 0, max_n = 1;
-    if (dev_plan) {
+    if (wave) {
+      // stable sort by (class, window length); pairs of other paths last
+      DevBuf d_key2, d_idx2;
+      if ((rc = d_key2.alloc(ctx, n_pairs * sizeof(uint64_t))) ||
+          (rc = d_idx2.alloc(ctx, n_pairs * sizeof(uint32_t))))
+        return (rc);
+      uint64_t* kk = pp.d_key.as<uint64_t>();
+      uint32_t* vv = pp.d_idx.as<uint32_t>();
+      if ((rc = launch_pair_sort(ctx, kk, vv, d_key2.as<uint64_t>(), d_idx2.as<uint32_t>(), n_pairs,
+                                 WAVE_NONE, pp.pst.max_t_len)))
+        return (rc);
+      phase_begin(res, PH_INTER);
+      if ((rc = launch_pair_wave(ctx, db, qs, d_mat, A, o, e, mode, fe, v.smax, v.smin, d_pairs, vv,
+                                 pp.pst.cls, pp.pst.max_t_len, sc)))
+        return (rc);
+      phase_end(res, PH_INTER);
+    } else if (dev_plan) {
       // device planner: stable sort by (query length, window length), jobs
       // from the runs of equal query length
       DevBuf d_key2, d_idx2;
@@ -354,8 +396,8 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
       n_pj = (uint32_t)pj.size();
       max_n = max_n16;
     }
-    bool bytes = A <= 4;   // byte-permute substitution form
-    for (int x = 0; x < A * A; ++x) bytes = bytes && matrix[x] + o >= -128 && matrix[x] + o <= 127;
+    if (!wave) {
+    const bool bytes = A <= 4 && s_plus_o_fits_int8(matrix, A, o);   // byte-permute substitution form
     auto launch = [&](int rows) {
       return launch_pairs16(ctx, db, qs, d_mat, A, o, e, mode, fe, v.smax, bytes, rows,
                             d_pj.as<Pair16Job>(), n_pj, max_n, sc);
@@ -405,6 +447,7 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
     phase_begin(res, PH_INTER);
     if ((rc = launch(rows))) return (rc);
     phase_end(res, PH_INTER);
+    }
     res->phase_cells[PH_INTER] = p16cells;
     res->phase_cells[PH_INT32] -= p16cells;
     if (mode == DSA_LOCAL) {
