@@ -310,7 +310,7 @@ int dsa_server_destroy(dsa_server* srv);
  * = codes[offsets[k] .. offsets[k+1])), `n_pairs` dsa_pair records, the
  * A x A int8 matrix, and three int32 output arrays of `n_pairs` entries
  * (score, q_end, t_end, as dsa_align reports them for explicit pairs).  The
- * call works on the current CUDA device and enqueues one kernel on
+ * call works on the current CUDA device and enqueues its kernels on
  * `cuda_stream` (NULL = the legacy default stream); it does not synchronize.
  *
  * Scratch: the query strips' boundary rows live in a fixed 32 MiB array
