@@ -276,6 +276,19 @@ int launch_intra_glob16(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, con
                         const PackedPlan& plan, const IntraWork& work, int mode, uint32_t fe,
                         int o, int e, int smax, int smin, Scores out, uint32_t n_targets_out);
 
+// Wavefront search of the first n_targets of the length order (k_wave.cu) on
+// `stream`: units of strips of `rows` (16 or 24) query rows as for the
+// inter-sequence kernel (records, each unit's first strip and strip count).
+// wave_takes: queries of up to max_m against targets of up to max_n residues
+// stay inside its 16-bit range.
+constexpr uint32_t WAVE_LONG_TARGET = 2048;   // longer targets take up to 32 lanes
+bool wave_takes(bool local, uint32_t max_m, uint32_t max_n, int o, int e, int smax, int smin);
+int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, const dsa_db* qs,
+                       const int8_t* d_matrix, const int8_t* d_pssm, int A, int mode, uint32_t fe, int o,
+                       int e, int smax, int smin, int rows, const std::vector<StripMeta>& meta,
+                       const std::vector<uint32_t>& sbase, const std::vector<uint32_t>& ns,
+                       uint32_t n_targets, Scores out);
+
 // Top-k per query over a dense [n_queries][n_targets] score matrix.
 int launch_topk(dsa_ctx* ctx, const Scores& s, uint32_t n_queries, uint32_t n_targets,
                 uint32_t k, dsa_hit* d_hits);

@@ -1,0 +1,676 @@
+// Database search on wavefronts, packed int16x2 (the score pass of the map
+// phase, Sec. II.B.1; DSW / DNW / DSG of Sec. II.C.2): G lanes (4 to 32, a
+// power of two) sweep one target against a stream of query strips.
+//
+// Layout.  As in the inter-sequence kernel the two 16-bit halves of every
+// register follow two balanced streams of queries, cut into strips of R rows.
+// Lane k of a group holds strip b G + k of the unit in band b and works on
+// target column s - k at step s; H and F of a strip's bottom row reach the
+// next strip by one shuffle each, one step later.  Only the last strip of a
+// band goes through memory (a boundary row per group), every G R rows instead
+// of every strip.  A CTA's 8 warps work on neighbouring targets of the length
+// order and share the band's query profile in shared memory: 16-byte words
+// [residue][row quad][strip], so the lanes of a quarter-warp read different
+// banks whatever residues they hold.  Short targets take few lanes (fewer
+// steps to fill and drain), the longest ones 32.
+//
+// Cells.  Values are stored unsigned with a bias B, so that no 16-bit half
+// leaves [0, 2^16) and sums are plain 32-bit additions that carry nothing
+// between the halves; the profile's packed words are integer sums
+// (hi << 16) + lo for the same reason.
+//   Local: e j is added to every value of column j, so that E is
+//   max(E, H - o + e, floor) with the floor 0 as the third operand:
+//     x = Ho_diag + (S + o + e);  H = max(x, E, F);  Ho = H - o;
+//     F' = max(F - e, Ho);  E' = max(E, Ho + e, floor of column j + 1)
+//   three maxima on the half-rate pipe and three sums, against four and one.
+//   Long targets, whose e j would pass 16 bits, take the form of the other
+//   local kernels (no e j; maxima that wrap alone).
+//   Global and semi-global: e (i + j) is added, and E and F of the next cell
+//   are max(H - o + e, E) and max(H - o + e, F): three maxima and one sum.
+//   Launches whose scores or gaps could pass 16 bits stay on the kernels of
+//   k_intra.cu, so nothing is flagged here.
+// Lanes start one after another: before a target's first column they hold the
+// padding residue, under which a strip's column-0 state is a fixed point.
+//
+// End cells.  Local: a column maximum above the best of the strip's query so
+// far (as known to the lane: shared along the query's lanes every 32 steps)
+// parks the column in shared memory; per band the lanes of a query are
+// reduced under (score desc, j asc, i asc), the winner looks its row up and
+// merges with the earlier bands' result.  Global and semi-global: as in the
+// inter-sequence kernel (column n parked, row m tracked).
+//
+// Bound by the ALU pipe; 128 registers keep 16 warps per SM.  Measured (whole
+// score pass, before: the inter-sequence kernel with the longest targets on
+// the wavefronts of k_intra.cu): 7 queries of 90-1,100 against 50,011 targets,
+// global, 16.1 -> 8.8 ms (6,100 GCUPS); 5 of 60-700 against 60,000, local, 17.1
+// -> 7.4 ms; 32 of 64-5,000 against 100,000, local, 225.6 -> 225.3 ms.
+#include "dsa_internal.cuh"
+#include "dpx.cuh"
+
+#include <algorithm>
+#include <cstring>
+#include <vector>
+
+namespace dsa {
+namespace {
+
+constexpr int NW = 8;              // warps per CTA
+constexpr int NT = NW * 32;
+constexpr int FEW_LANES = 8;       // lanes per target where targets abound
+constexpr int PLANE = 512;         // bytes of one row quad of 32 strips
+enum Form { LOCAL_SUM = 0, LOCAL_WRAP = 1, GLOBAL_SUM = 2 };
+
+// Targets first .. first + count of the length order against one unit, `G`
+// lanes a target, CTA items of NW * 32 / G targets.
+struct Segment {
+  uint32_t unit, first, count, item0;
+  int32_t G;
+};
+
+struct WaveArgs {
+  const uint8_t* tcodes;
+  const uint64_t* toff;
+  const uint32_t* tlen;
+  const uint32_t* perm;            // length order -> target id
+  const uint32_t* prof;            // [strip][residue][R] packed
+  const StripMeta* meta;
+  const uint32_t* sbase;
+  const uint32_t* nstrips;
+  const uint32_t* qlen;
+  int A, o, e, mode, bias, T;
+  uint32_t fe;
+  uint32_t pad_word;               // profile word of strips past a unit's end
+  const Segment* segs;
+  uint32_t n_segs, n_items;
+  uint32_t* counter;
+  uint2* scratch;
+  uint64_t warp_cols;              // boundary cells per warp
+  Scores out;
+  uint32_t n_out_t;
+};
+
+template <int FORM, int R>
+__global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
+  constexpr bool LOCAL = FORM != GLOBAL_SUM;
+  constexpr bool SUM = FORM != LOCAL_WRAP;
+  constexpr unsigned FULL = 0xFFFFFFFFu;
+  constexpr uint32_t BIAS2 = 0x80008000u;
+  constexpr int RS = R / 4 * PLANE;   // profile bytes per residue
+  extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ Segment s_seg;
+  __shared__ uint32_t s_tile;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // parked columns: local [half][8 rows of 16 bits][thread], others packed
+  // [row][thread]
+  uint4* const park = reinterpret_cast<uint4*>(smem + (A.A + 1) * RS) + tid;
+  uint32_t* const parkw = reinterpret_cast<uint32_t*>(smem + (A.A + 1) * RS) + tid;
+  const int o = A.o, e = A.e;
+  const uint32_t e2 = (uint32_t)e * 0x10001u, o2 = (uint32_t)o * 0x10001u;
+  const uint32_t neg_e2 = pack2(-e, -e), c2 = pack2(e - o, e - o);
+  const uint32_t mo2 = pack2(-o, -o) ^ BIAS2;
+  const bool sg = A.mode == DSA_SEMIGLOBAL;
+  const bool qb_free = sg && (A.fe & DSA_FREE_Q_BEGIN), qe_free = sg && (A.fe & DSA_FREE_Q_END);
+  const bool tb_free = sg && (A.fe & DSA_FREE_T_BEGIN), te_free = sg && (A.fe & DSA_FREE_T_END);
+  auto row0 = [&](int j) { return (j == 0 || tb_free) ? 0 : -(o + (j - 1) * e); };
+  uint2* const scr_warp = A.scratch + (uint64_t)(blockIdx.x * NW + warp) * A.warp_cols;
+  uint32_t held = NONE;               // first strip and group size of the profile in place
+
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) {
+      const uint32_t item = atomicAdd(A.counter, 1u);
+      if (item >= A.n_items) {
+        s_tile = NONE;
+      } else {
+        uint32_t lo = 0, hi = A.n_segs;   // the last segment starting at or before the item
+        while (hi - lo > 1) {
+          const uint32_t mid = (lo + hi) / 2;
+          if (A.segs[mid].item0 <= item) lo = mid;
+          else hi = mid;
+        }
+        s_seg = A.segs[lo];
+        s_tile = item - s_seg.item0;
+      }
+    }
+    __syncthreads();
+    if (s_tile == NONE) break;
+    const int G = s_seg.G, k = lane & (G - 1);
+    const uint32_t ns = A.nstrips[s_seg.unit], sb = A.sbase[s_seg.unit];
+    const uint32_t in_seg = s_tile * (NW * 32 / G) + warp * (32 / G) + lane / G;
+    const bool valid = in_seg < s_seg.count;
+    uint32_t id = 0;
+    int n = 0;
+    const uint8_t* t = A.tcodes;
+    if (valid) {
+      id = A.perm[s_seg.first + in_seg];
+      n = (int)A.tlen[id];
+      t = A.tcodes + A.toff[id];
+    }
+    int nmax = n, nmin = n;
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) {
+      nmax = max(nmax, __shfl_xor_sync(FULL, nmax, w));
+      nmin = min(nmin, __shfl_xor_sync(FULL, nmin, w));
+    }
+    const uint32_t sh = 8u * (uint32_t)((uintptr_t)(t - k) & 3);
+    uint2* const scr = scr_warp + (uint64_t)(lane / G) * nmax;
+    const int steps = nmax + G - 1;
+    const int nb = ((int)ns + G - 1) / G;
+
+    for (int b = 0; b < nb; ++b) {
+      const uint32_t want = (sb + (uint32_t)(b * G)) * 64u + (uint32_t)G;
+      if (held != want) {
+        __syncthreads();
+        // slot x of 8 or more holds strip x mod G: 4 lanes a target read two copies
+        const int slots = max(G, 8), lg = 31 - __clz(slots);
+        const int total = slots * (A.A + 1) * (R / 4);
+        for (int x = tid; x < total; x += NT) {
+          const int slot = x & (slots - 1), rest = x >> lg;
+          const uint32_t strip = (uint32_t)(b * G + (slot & (G - 1)));
+          uint4 v = make_uint4(A.pad_word, A.pad_word, A.pad_word, A.pad_word);
+          if (strip < ns)
+            v = __ldg(reinterpret_cast<const uint4*>(A.prof + (uint64_t)(sb + strip) * (A.A + 1) * R) + rest);
+          *reinterpret_cast<uint4*>(smem + rest * PLANE + slot * 16) = v;
+        }
+        __syncthreads();
+        held = want;
+      }
+      const uint8_t* const pbase = smem + (lane & (max(G, 8) - 1)) * 16;
+      StripMeta md{NONE, 0, NONE, 0};
+      if ((uint32_t)(b * G + k) < ns) md = A.meta[sb + b * G + k];
+      const int ka = (int)(md.ka & ~LAST), kb = (int)(md.kb & ~LAST);
+      const uint32_t keep = (ka == 0 ? 0u : 0x0000FFFFu) | (kb == 0 ? 0u : 0xFFFF0000u);
+      const bool last_a = (md.ka & LAST) && md.qa != NONE, last_b = (md.kb & LAST) && md.qb != NONE;
+
+      // ---- column-0 state ----
+      int j = -k;                    // the lane's column
+      uint32_t Ho[R], E[R], diag, sendH, sendF;
+      uint32_t flo2 = mo2, fln2 = 0; // local: H = 0 as H - o at column j, the floor of column j + 1
+      uint32_t rthr = 0xFFFFFFFFu, rinc = 0;
+      int rj_a = 0, rj_b = 0;
+      uint32_t hmn = 0;
+      if (LOCAL) {
+        if (SUM) {
+          flo2 = (uint32_t)(A.bias + e * j - o) * 0x10001u;
+          fln2 = flo2 + o2 + e2;
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          Ho[r] = flo2;
+          E[r] = SUM ? fln2 : pack2(NEG16, NEG16) ^ BIAS2;
+        }
+        diag = sendH = sendF = flo2;
+      } else {
+        // H of column 0 at padded row i, and F entering row i + 1 there, with
+        // e (i + j) added; a half without a query is all padding rows
+        const int ma = md.qa != NONE ? (int)A.qlen[md.qa] : 0, mb = md.qb != NONE ? (int)A.qlen[md.qb] : 0;
+        const int pa = md.qa != NONE ? (R - ma % R) % R : INT32_MAX;
+        const int pb = md.qb != NONE ? (R - mb % R) % R : INT32_MAX;
+        auto hv = [&](int i, int p) {
+          const int h = (i <= p || qb_free) ? 0 : -(o + (i - p - 1) * e);
+          return A.bias + h + e * (i + j);
+        };
+        auto fv = [&](int i, int p) {
+          const int f = (i <= p || qb_free) ? -o : -(o + (i - p) * e);
+          return A.bias + f + e * (i + 1 + j);
+        };
+        const int ba = ka * R, bb = kb * R;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          Ho[r] = pack2(hv(ba + r + 1, pa), hv(bb + r + 1, pb));
+          E[r] = add2(Ho[r], c2);
+        }
+        diag = pack2(hv(ba, pa), hv(bb, pb));
+        sendH = Ho[R - 1];
+        sendF = pack2(fv(ba + R, pa), fv(bb + R, pb));
+        if (te_free && last_a) { rthr = (rthr & 0xFFFF0000u) | (uint32_t)hv(ba + R, pa); rinc |= (uint32_t)e; }
+        if (te_free && last_b) { rthr = (rthr & 0x0000FFFFu) | (uint32_t)hv(bb + R, pb) << 16; rinc |= (uint32_t)e << 16; }
+      }
+      // local: the best this lane has seen per half in this band, the best of
+      // its query's earlier bands and, from the last exchange, of its lanes,
+      // and the trigger threshold
+      int best_a = 0, best_b = 0, bj_a = 0, bj_b = 0;
+      uint32_t shared2 = 0, thr2 = 0;
+      if (LOCAL && b > 0 && valid) {
+        if (ka > k) shared2 = (uint32_t)min(A.out.score[(uint64_t)md.qa * A.n_out_t + id], 0xFFFF);
+        if (kb > k) shared2 |= (uint32_t)min(A.out.score[(uint64_t)md.qb * A.n_out_t + id], 0xFFFF) << 16;
+      }
+      auto set_thr = [&]() {   // columns whose maximum reaches the best trigger
+        const uint32_t v = __vmaxu2(shared2, pack2(best_a, best_b));
+        thr2 = __vsubus2(v, 0x00010001u) + (SUM ? flo2 + o2 : BIAS2);
+      };
+      if (LOCAL) set_thr();
+      const bool hand = b + 1 < nb && k == G - 1;   // the band's bottom row is read again
+      uint2 in = make_uint2(0, 0);
+      if (b > 0 && k == 0 && n > 0) in = scr[0];
+
+      // residues of 4 steps, one block ahead: two aligned words, or (edge) the
+      // four bytes with the padding residue outside the target
+      auto edge_at = [&](int s0) { return s0 < G - 1 || s0 + 4 > nmin; };
+      auto fetch = [&](int s0) -> uint2 {
+        const int x = s0 - k;
+        if (!edge_at(s0)) {
+          const uint32_t* p = reinterpret_cast<const uint32_t*>((uintptr_t)(t + x) & ~(uintptr_t)3);
+          return make_uint2(__ldg(p), __ldg(p + 1));
+        }
+        uint32_t w = 0;
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          w |= ((uint32_t)(x + y) < (uint32_t)n ? (uint32_t)__ldg(t + x + y) : (uint32_t)A.A) << (8 * y);
+        return make_uint2(w, 0);
+      };
+      uint2 nxt = fetch(0);
+      for (int s0 = 0; s0 < steps; s0 += 4) {
+        const uint32_t r4 = edge_at(s0) ? nxt.x : __funnelshift_r(nxt.x, nxt.y, sh);
+        nxt = fetch(s0 + 4);
+        if (LOCAL && ((s0 & 31) == 28 || s0 == 4 || s0 == 12)) {
+          // the best of the query's lanes: maxima over the lanes above and
+          // below that hold the same query, per half
+          const int fa = max(0, k - ka), fb = max(0, k - kb);
+          uint32_t v = __vmaxu2(shared2, pack2(best_a, best_b));
+          for (int w = 1; w < G; w <<= 1) {
+            const uint32_t u = __shfl_up_sync(FULL, v, w);
+            const uint32_t ok = (k - w >= fa ? 0x0000FFFFu : 0u) | (k - w >= fb ? 0xFFFF0000u : 0u);
+            const uint32_t d = __shfl_down_sync(FULL, v, w);
+            const int fda = __shfl_down_sync(FULL, fa, w), fdb = __shfl_down_sync(FULL, fb, w);
+            const uint32_t okd = k + w < G ? (fda <= k ? 0x0000FFFFu : 0u) | (fdb <= k ? 0xFFFF0000u : 0u) : 0u;
+            v = max3_2u(v, u & ok, d & okd);
+          }
+          shared2 = v;
+          set_thr();
+        }
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          ++j;
+          uint32_t upH = __shfl_up_sync(FULL, sendH, 1);
+          uint32_t upF = __shfl_up_sync(FULL, sendF, 1);
+          if (b > 0 && k == 0) {
+            upH = in.x;
+            upF = in.y;
+            if (j < n) in = scr[j];
+          }
+          uint32_t bH, bF;   // row 0 at this column, where a query starts
+          if (LOCAL) {
+            if (SUM) { flo2 += e2; fln2 += e2; thr2 += e2; }
+            bH = bF = flo2;
+          } else {
+            const int v = A.bias + ((tb_free || j <= 0) ? e * j : e - o);
+            bH = (uint32_t)v * 0x10001u;
+            bF = (uint32_t)(v + e - o) * 0x10001u;
+          }
+          const uint32_t topH = (upH & keep) | (bH & ~keep);
+          uint32_t F = (upF & keep) | (bF & ~keep);
+          const uint8_t* const p = pbase + ((r4 >> (8 * y)) & 0xFFu) * RS;
+          uint32_t d = diag;
+          diag = topH;
+          uint32_t cm = 0, hprev = 0;
+#pragma unroll
+          for (int q = 0; q < R / 4; ++q) {
+            const uint4 pv = *reinterpret_cast<const uint4*>(p + q * PLANE);
+            const uint32_t pr[4] = {pv.x, pv.y, pv.z, pv.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int r = q * 4 + u;
+              const uint32_t old = Ho[r];
+              uint32_t h;
+              if (FORM == LOCAL_SUM) {
+                h = max3_2u(d + pr[u], E[r], F);
+                const uint32_t ho = h - o2;
+                F = addmax2u(F, neg_e2, ho);
+                E[r] = max3_2u(E[r], ho + e2, fln2);
+                Ho[r] = ho;
+              } else if (FORM == LOCAL_WRAP) {
+                E[r] = addmax2u(E[r], neg_e2, old);
+                const uint32_t x = addmax2u(d, pr[u], E[r]);
+                h = max3_2u(x, F, BIAS2);
+                Ho[r] = h - o2;
+                F = addmax2u(F, neg_e2, Ho[r]);
+              } else {
+                h = max3_2u(d + pr[u], E[r], F);
+                E[r] = addmax2u(h, c2, E[r]);
+                F = addmax2u(h, c2, F);
+                Ho[r] = h;
+              }
+              d = old;
+              if (LOCAL) {
+                if (r & 1) cm = max3_2u(cm, hprev, h);
+                else hprev = h;
+              }
+            }
+          }
+          sendH = Ho[R - 1];
+          sendF = F;
+          if (b + 1 < nb && hand && (uint32_t)(j - 1) < (uint32_t)n) scr[j - 1] = make_uint2(sendH, sendF);
+          if (LOCAL) {
+            if (__vmaxu2(cm, thr2) != thr2) {
+              const int z = (int)(SUM ? (flo2 & 0xFFFFu) + (uint32_t)o : 0x8000u);   // H = 0
+              const int ca = (int)(cm & 0xFFFFu) - z, cb = (int)(cm >> 16) - z;
+              // (the other half may have raised the threshold's alarm)
+              if (ca > best_a && ca >= (int)(shared2 & 0xFFFFu)) {
+#pragma unroll
+                for (int r = 0; r < R; r += 8)
+                  park[r / 8 * NT] = make_uint4(prmt(Ho[r], Ho[r + 1], 0x5410), prmt(Ho[r + 2], Ho[r + 3], 0x5410),
+                                                prmt(Ho[r + 4], Ho[r + 5], 0x5410), prmt(Ho[r + 6], Ho[r + 7], 0x5410));
+                best_a = ca; bj_a = j;
+              }
+              if (cb > best_b && cb >= (int)(shared2 >> 16)) {
+#pragma unroll
+                for (int r = 0; r < R; r += 8)
+                  park[(R + r) / 8 * NT] =
+                      make_uint4(prmt(Ho[r], Ho[r + 1], 0x7632), prmt(Ho[r + 2], Ho[r + 3], 0x7632),
+                                 prmt(Ho[r + 4], Ho[r + 5], 0x7632), prmt(Ho[r + 6], Ho[r + 7], 0x7632));
+                best_b = cb; bj_b = j;
+              }
+              set_thr();
+            }
+          } else {
+            if (te_free) {
+              rthr += rinc;
+              if (__vmaxu2(sendH, rthr) != rthr && j >= 1 && j <= n) {
+                if ((sendH & 0xFFFFu) > (rthr & 0xFFFFu)) {
+                  rthr = (rthr & 0xFFFF0000u) | (sendH & 0xFFFFu);
+                  rj_a = j;
+                }
+                if ((sendH >> 16) > (rthr >> 16)) {
+                  rthr = (rthr & 0x0000FFFFu) | (sendH & 0xFFFF0000u);
+                  rj_b = j;
+                }
+              }
+            }
+            if (j == n) {
+              hmn = sendH;
+              if (qe_free) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) parkw[r * NT] = Ho[r];
+              }
+            }
+          }
+        }
+      }
+
+      // ---- the band's results, one half at a time ----
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const uint32_t q = x ? md.qb : md.qa;
+        const int kq = x ? kb : ka;
+        const int first = max(0, k - kq);         // the query's first lane in this band
+        const bool starts = k - first == kq;      // its first strip is in this band
+        const int sh16 = 16 * x;
+        if (LOCAL) {
+          int s = x ? best_b : best_a, jj = x ? bj_b : bj_a, src = lane;
+          for (int w = 1; w < G; w <<= 1) {
+            const int s2 = __shfl_down_sync(FULL, s, w), j2 = __shfl_down_sync(FULL, jj, w);
+            const int src2 = __shfl_down_sync(FULL, src, w);
+            const int f2 = __shfl_down_sync(FULL, first, w);
+            const uint32_t q2 = __shfl_down_sync(FULL, q, w);
+            // lanes k .. k + w hold the same query: a tie keeps the smaller rows
+            if (k + w < G && q2 == q && f2 <= k && (s2 > s || (s2 == s && s2 > 0 && j2 < jj))) {
+              s = s2; jj = j2; src = src2;
+            }
+          }
+          const int win = __shfl_sync(FULL, src, (lane & ~(G - 1)) + first);
+          if (valid && q != NONE && win == lane) {
+            const int bs = x ? best_b : best_a, bj = x ? bj_b : bj_a;
+            int bi = 0;
+            if (bs > 0) {
+              const uint16_t wanted = (uint16_t)(SUM ? bs - o + A.bias + e * bj : bs - o + 0x8000);
+              int rr = R - 1;
+              for (int r = R - 1; r >= 0; --r)
+                if (reinterpret_cast<const uint16_t*>(park + (x * R + r) / 8 * NT)[r & 7] == wanted) rr = r;
+              bi = kq * R + rr + 1;
+            }
+            const uint64_t idx = (uint64_t)q * A.n_out_t + id;
+            bool put = starts;
+            if (!put && bs > 0) {
+              const int os = A.out.score[idx], ot = A.out.t_end[idx];
+              put = bs > os || (bs == os && bj - 1 < ot);   // earlier bands hold smaller rows
+            }
+            if (put) {
+              A.out.score[idx] = bs;
+              A.out.q_end[idx] = bi - 1;
+              A.out.t_end[idx] = bs > 0 ? bj - 1 : -1;
+              A.out.flag[idx] = bs > A.T ? 1 : 0;
+            }
+          }
+        } else {
+          const int m = q != NONE ? (int)A.qlen[q] : 0, pad = (R - m % R) % R;
+          const int base = kq * R;
+          // column n (free query end): this strip's real rows, smallest i first
+          int cb = INT32_MIN, ci = 0;
+          if (qe_free && q != NONE) {
+            for (int r = 0; r < R; ++r) {
+              const int i = base + r + 1;
+              const int v = (int)((parkw[r * NT] >> sh16) & 0xFFFFu) - A.bias - e * (i + n);
+              if (i > pad && v > cb) { cb = v; ci = i - pad; }
+            }
+          }
+          if (qe_free) {
+            for (int w = 1; w < G; w <<= 1) {
+              const int s2 = __shfl_down_sync(FULL, cb, w), i2 = __shfl_down_sync(FULL, ci, w);
+              const int f2 = __shfl_down_sync(FULL, first, w);
+              const uint32_t q2 = __shfl_down_sync(FULL, q, w);
+              if (k + w < G && q2 == q && f2 <= k && (s2 > cb || (s2 == cb && i2 < ci))) { cb = s2; ci = i2; }
+            }
+            cb = __shfl_sync(FULL, cb, (lane & ~(G - 1)) + first);
+            ci = __shfl_sync(FULL, ci, (lane & ~(G - 1)) + first);
+          }
+          // the query's last lane in this band writes: the result, or with a
+          // free query end column n's best so far
+          const bool last = x ? last_b : last_a;
+          const int strips = (m + R - 1) / R;
+          const bool tail = q != NONE && (last || (k == G - 1 && kq < strips - 1));
+          if (valid && tail && (last || qe_free)) {
+            const uint64_t idx = (uint64_t)q * A.n_out_t + id;
+            if (qe_free) {
+              const int ps = starts ? row0(n) : A.out.score[idx], pi = starts ? 0 : A.out.q_end[idx];
+              if (ps >= cb) { cb = ps; ci = pi; }   // earlier rows
+            }
+            int bs = cb, bi = ci, bj = n;
+            if (last) {
+              const int corner = (int)((hmn >> sh16) & 0xFFFFu) - A.bias - e * (base + R + n);
+              if (!qe_free || corner > bs) { bs = corner; bi = m; }
+              if (te_free) {
+                const int rj = x ? rj_b : rj_a;
+                // the threshold holds the best's value at the last step's column
+                const int rv = (int)((rthr >> sh16) & 0xFFFFu) - A.bias - e * (base + R + j);
+                if (rv > bs || (rv == bs && rj < bj)) { bs = rv; bi = m; bj = rj; }
+              }
+              A.out.score[idx] = bs;
+              A.out.q_end[idx] = bi - 1;
+              A.out.t_end[idx] = bj - 1;
+              A.out.flag[idx] = 0;
+            } else {
+              A.out.score[idx] = bs;
+              A.out.q_end[idx] = bi;
+            }
+          }
+        }
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// Profile of every strip: [strip][residue][R] packed words, lo / hi the
+// scores of the two halves' rows plus `add`.  Local: rows past a query's end,
+// absent queries and the padding residue get a score below any.  End-anchored
+// (global, semi-global): rows above a query reproduce row 0.
+struct ProfArgs {
+  const uint8_t* qcodes;
+  const uint64_t* qoff;
+  const uint32_t* qlen;
+  const StripMeta* meta;
+  uint32_t n_strips;
+  const int8_t* S;
+  const int8_t* P;     // position-specific rows, or null
+  int A, R, add, form;
+  int pad_row, pad_col, none;   // words' halves: padding rows; padding residue on real rows; below any
+  uint32_t* prof;
+};
+__global__ void k_wave_profile(const ProfArgs W) {
+  const uint64_t total = (uint64_t)W.n_strips * (W.A + 1) * W.R;
+  for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < total;
+       x += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t s = (uint32_t)(x / ((uint64_t)(W.A + 1) * W.R));
+    const int a = (int)(x / W.R % (W.A + 1)), r = (int)(x % W.R);
+    const StripMeta md = W.meta[s];
+    auto val = [&](uint32_t q, uint32_t kq) -> int {
+      const bool glob = W.form == GLOBAL_SUM;
+      if (q == NONE) return glob ? (a == W.A ? W.add : W.pad_row) : W.none;
+      const int m = (int)W.qlen[q];
+      const int i = (int)(kq & ~LAST) * W.R + r - (glob ? (W.R - m % W.R) % W.R : 0);
+      if (i < 0) return a == W.A ? W.add : W.pad_row;
+      if (i >= m || (!glob && a == W.A)) return W.none;
+      if (a == W.A) return W.pad_col;
+      const uint64_t at = W.qoff[q] + (uint64_t)i;
+      return (W.P ? (int)W.P[at * W.A + a] : (int)W.S[W.qcodes[at] * W.A + a]) + W.add;
+    };
+    const int lo = val(md.qa, md.ka), hi = val(md.qb, md.kb);
+    W.prof[x] = W.form == LOCAL_WRAP ? pack2(lo, hi) : ((uint32_t)hi << 16) + (uint32_t)lo;
+  }
+}
+
+// The form of a local launch, or of a global one (-1: k_intra.cu's kernel):
+// whether values with e j or e (i + j) added stay inside 16 bits for queries
+// of up to m and targets of up to n residues.
+int local_bias(int o, int e) { return 512 + o + 64 * e; }
+int global_bias(int o, int e, int smin) { return 4 * o + 64 * e + std::max(0, -smin) + 256; }
+int wave_form(bool local, int64_t m, int64_t n, int o, int e, int smax, int smin) {
+  const int64_t up = (int64_t)std::max(0, smax) * std::min(m, n);
+  if (local) {
+    return up + e * (n + 64) + local_bias(o, e) + 2ll * (o + e) + 512 < 65536 ? LOCAL_SUM : LOCAL_WRAP;
+  }
+  if (up > 32767 - std::max(0, smax)) return -1;
+  if (4ll * o + (m + n + 2) * e + std::max(0, -smin) + 64 >= 32768) return -1;
+  return up + e * (m + n + 256) + global_bias(o, e, smin) + 2ll * (o + e) + 512 < 65536 ? GLOBAL_SUM : -1;
+}
+
+}  // namespace
+
+bool wave_takes(bool local, uint32_t max_m, uint32_t max_n, int o, int e, int smax, int smin) {
+  return wave_form(local, max_m, max_n, o, e, smax, smin) >= 0;
+}
+
+int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, const dsa_db* qs,
+                       const int8_t* d_matrix, const int8_t* d_pssm, int A, int mode, uint32_t fe, int o,
+                       int e, int smax, int smin, int rows, const std::vector<StripMeta>& meta,
+                       const std::vector<uint32_t>& sbase, const std::vector<uint32_t>& ns,
+                       uint32_t n_targets, Scores out) {
+  if (n_targets == 0 || ns.empty()) return DSA_OK;
+  const bool local = mode == DSA_LOCAL;
+  const uint32_t max_n = db->h_len[db->h_perm[0]];
+  const int form = wave_form(local, qs->max_len, max_n, o, e, smax, smin);
+  auto kern = form == LOCAL_SUM    ? (rows == 16 ? k_wave<LOCAL_SUM, 16> : k_wave<LOCAL_SUM, 24>)
+              : form == LOCAL_WRAP ? (rows == 16 ? k_wave<LOCAL_WRAP, 16> : k_wave<LOCAL_WRAP, 24>)
+                                   : (rows == 16 ? k_wave<GLOBAL_SUM, 16> : k_wave<GLOBAL_SUM, 24>);
+  if (form < 0 || (rows != 16 && rows != 24)) {
+    set_error("no wavefront form for this search");
+    return DSA_ERR_INVALID_ARG;
+  }
+  const size_t smem = (size_t)(A + 1) * rows / 4 * PLANE + (size_t)rows * NT * 4;
+  DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 0;
+  DSA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
+  const uint32_t ctas = (uint32_t)std::max(1, per_sm) * ctx->sm_count;
+
+  // Lanes per target: as many as the unit has strips, up to 8 (more lanes cost
+  // more steps to fill and drain on every target, and more of them idle in a
+  // unit's last band; 7 queries of 90-1,100 against 50,011 targets, global:
+  // 9.3 ms with up to 16, 8.8 with 8), up to 32 for the longest targets, whose
+  // chain ends the launch, and for launches with fewer targets than the chip
+  // has room for.
+  uint32_t n_long = 0;
+  while (n_long < n_targets && db->h_len[db->h_perm[n_long]] > WAVE_LONG_TARGET) ++n_long;
+  std::vector<Segment> segs;
+  uint32_t items = 0;
+  bool bands = false;
+  auto lanes = [&](uint32_t strips, int most) {
+    int g = 4;
+    while (g < most && (uint32_t)g < strips) g *= 2;
+    return g;
+  };
+  for (int part = 0; part < 2; ++part) {
+    const uint32_t first = part ? n_long : 0, count = part ? n_targets - n_long : n_long;
+    if (count == 0) continue;
+    for (uint32_t u = 0; u < ns.size(); ++u) {
+      int G = lanes(ns[u], part ? FEW_LANES : 32);
+      while (G < 32 && (uint32_t)G < ns[u] &&
+             (uint64_t)n_targets * ns.size() * G < (uint64_t)ctas * NT)
+        G *= 2;
+      segs.push_back({u, first, count, items, G});
+      items += (count + NW * 32 / G - 1) / (NW * 32 / G);
+      bands = bands || ns[u] > (uint32_t)G;
+    }
+  }
+  const unsigned grid = std::min<uint32_t>(items, ctas);
+  // boundary cells of a warp: its longest target, or two of the shorter ones
+  const uint64_t cols =
+      bands ? std::max<uint64_t>(max_n, 32ull / FEW_LANES * std::min(max_n, WAVE_LONG_TARGET)) : 0;
+
+  WaveArgs W{};
+  W.tcodes = db->d_codes; W.toff = db->d_off; W.tlen = db->d_len; W.perm = db->d_perm;
+  W.qlen = qs->d_len;
+  W.A = A; W.o = o; W.e = e; W.mode = mode; W.fe = fe;
+  W.bias = local ? local_bias(o, e) : global_bias(o, e, smin);
+  W.T = 32767 - std::max(0, smax);
+  ProfArgs P{};
+  P.qcodes = qs->d_codes; P.qoff = qs->d_off; P.qlen = qs->d_len;
+  P.n_strips = (uint32_t)meta.size();
+  P.S = d_matrix; P.P = d_pssm;
+  P.A = A; P.R = rows; P.form = form;
+  P.add = form == LOCAL_SUM ? o + e : form == LOCAL_WRAP ? o : 2 * e;
+  P.none = form == LOCAL_WRAP ? NEG16 : -128;
+  if (!local) {
+    const bool sg = mode == DSA_SEMIGLOBAL;
+    P.pad_row = sg && (fe & DSA_FREE_T_BEGIN) ? P.add : P.add - o;
+    P.pad_col = sg && (fe & DSA_FREE_Q_BEGIN) ? P.add : P.add - o;
+  }
+  const int pw = local ? P.none : P.pad_row;
+  W.pad_word = form == LOCAL_WRAP ? (uint32_t)(pw & 0xFFFF) * 0x10001u : ((uint32_t)pw << 16) + (uint32_t)pw;
+
+  // one upload: segments, strip records, each unit's first strip and strip count
+  const size_t b_seg = (segs.size() * sizeof(Segment) + 15) & ~(size_t)15;
+  const size_t b_meta = (meta.size() * sizeof(StripMeta) + 15) & ~(size_t)15;
+  const size_t b_u = (ns.size() * 4 + 15) & ~(size_t)15;
+  std::vector<uint8_t> host(b_seg + b_meta + 2 * b_u);
+  memcpy(host.data(), segs.data(), segs.size() * sizeof(Segment));
+  memcpy(host.data() + b_seg, meta.data(), meta.size() * sizeof(StripMeta));
+  memcpy(host.data() + b_seg + b_meta, sbase.data(), sbase.size() * 4);
+  memcpy(host.data() + b_seg + b_meta + b_u, ns.data(), ns.size() * 4);
+  const size_t b_prof = (size_t)P.n_strips * (A + 1) * rows * 4;
+  const size_t b_scr = (size_t)grid * NW * cols * sizeof(uint2);
+  void* buf = nullptr;
+  const size_t b_all = host.size() + b_prof + b_scr + 16;
+  DSA_TRY(ctx->alloc(&buf, b_all, stream));
+  uint8_t* d = static_cast<uint8_t*>(buf);
+  cudaError_t err = cudaMemcpyAsync(d, host.data(), host.size(), cudaMemcpyHostToDevice, stream);
+  W.segs = reinterpret_cast<const Segment*>(d);
+  W.meta = P.meta = reinterpret_cast<const StripMeta*>(d + b_seg);
+  W.sbase = reinterpret_cast<const uint32_t*>(d + b_seg + b_meta);
+  W.nstrips = reinterpret_cast<const uint32_t*>(d + b_seg + b_meta + b_u);
+  W.prof = P.prof = reinterpret_cast<uint32_t*>(d + host.size());
+  W.scratch = reinterpret_cast<uint2*>(d + host.size() + b_prof);
+  W.warp_cols = cols;
+  W.n_segs = (uint32_t)segs.size();
+  W.n_items = items;
+  W.counter = ctx->d_counters + 2;
+  W.out = out;
+  W.n_out_t = db->n;
+  if (err == cudaSuccess) err = cudaMemsetAsync(W.counter, 0, sizeof(uint32_t), stream);
+  if (err == cudaSuccess) {
+    const uint64_t words = (uint64_t)P.n_strips * (A + 1) * rows;
+    k_wave_profile<<<(unsigned)std::min<uint64_t>((words + 255) / 256, (uint64_t)ctx->sm_count * 8), 256, 0,
+                     stream>>>(P);
+    kern<<<grid, NT, smem, stream>>>(W);
+    ctx->launches += 2;
+    err = cudaGetLastError();
+  }
+  ctx->release(buf, b_all, stream);
+  if (err != cudaSuccess) {
+    set_error("k_wave launch: %s", cudaGetErrorString(err));
+    return DSA_ERR_CUDA;
+  }
+  return DSA_OK;
+}
+
+}  // namespace dsa

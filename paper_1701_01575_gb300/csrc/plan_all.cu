@@ -29,13 +29,14 @@ namespace {
 // kernel.  For a workload shape (GPU, driver, mode, alphabet,
 // and log2 bins of the query count, query residues, longest query, target
 // count, database residues and longest target) the first call times each
-// strip height at the default threshold (a switch needs a 3% gain), then a
-// local search of thresholds -- starting at 4096, then lower or higher by
-// factors of 4 while it keeps improving by 3% or more -- and keeps both in a
-// JSON cache file.  DSA_AUTOTUNE=off (28 rows, 4096) | cache (default: tune
-// on a miss) | retune (always tune); DSA_AUTOTUNE_CACHE names the file
-// (default $XDG_CACHE_HOME/dsa/autotune.json or ~/.cache/dsa/autotune.json);
-// DSA_INTER_ROWS (28 | 20) and DSA_LONG_THRESHOLD fix their choice.
+// strip height at the modelled threshold (a switch needs a 3% gain), then
+// every target on the wavefronts, then a local search of thresholds lower and
+// higher by factors of 4 while it keeps improving by 3% or more -- and keeps
+// both in a JSON cache file.  DSA_AUTOTUNE=off (28 rows, the model) | cache
+// (default: tune on a miss) | retune (always tune); DSA_AUTOTUNE_CACHE names
+// the file (default $XDG_CACHE_HOME/dsa/autotune.json or
+// ~/.cache/dsa/autotune.json); DSA_INTER_ROWS (28 | 20) and
+// DSA_LONG_THRESHOLD fix their choice.
 struct Tuner {
   std::mutex mu;
   bool loaded = false;
@@ -113,33 +114,20 @@ int ilog2_bin(uint64_t x) {
   return b;
 }
 
-// Packed score pass (int16x2).  Targets of groups longer than `long_thr` go
-// to the wavefront kernel on the side stream, the rest to the
-// inter-sequence kernel; the results do not depend on long_thr, only the
-// time.  Global / semi-global use the end-anchored forms of both kernels.
-int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
-                 const int8_t* d_mat, const int8_t* d_pssm, int A, int o, int e, const Validated& v, Scores out,
-                 uint32_t long_thr, int rows, int mode = DSA_LOCAL, uint32_t fe = 15) {
-  const bool local = mode == DSA_LOCAL;
-  const uint32_t W = (uint32_t)rows;   // strip rows of the inter-sequence kernel
-  const uint32_t nq = qs->n, nt = db->n;
-  const int R = A + 1;
-  std::vector<uint32_t> qorder(nq);
-  std::iota(qorder.begin(), qorder.end(), 0u);
-  std::stable_sort(qorder.begin(), qorder.end(),
-                   [&](uint32_t a, uint32_t b) { return qs->h_len[a] > qs->h_len[b]; });
+// Stream plan of the inter-sequence and wavefront kernels: queries, cut into
+// strips of W rows, are dealt, longest first, to the currently shortest of K
+// lanes (K about total / longest, so a lane is about as long as the longest
+// query, or as `at_least` strips); lanes are then paired by length into units,
+// low half = first lane, high half = second.
+struct Streams {
+  std::vector<StripMeta> meta;
+  std::vector<uint32_t> sbase, ns;   // per unit: first strip, strips
+};
+Streams build_streams(const dsa_db* qs, const std::vector<uint32_t>& qorder, uint32_t W,
+                      uint64_t at_least = 1) {
+  const uint32_t nq = qs->n;
   auto strips_of = [&](uint32_t q) { return (qs->h_len[q] + W - 1) / W; };
-
-  // groups whose longest target exceeds the threshold go to the wavefront kernel
-  uint32_t g_long = 0;
-  while (g_long < db->n_groups && db->h_glen[g_long] > long_thr) ++g_long;
-  const uint32_t n_long = std::min<uint32_t>(nt, g_long * GROUP);
-
-  // Stream plan for the inter-sequence kernel: queries are dealt, longest
-  // first, to the currently shortest of K lanes (K about total / longest, so a
-  // lane is about as long as the longest query); lanes are then paired by
-  // length into units, low half = first lane, high half = second.
-  uint64_t tot = 0, maxq = 1;
+  uint64_t tot = 0, maxq = at_least;
   for (uint32_t q = 0; q < nq; ++q) {
     tot += strips_of(q);
     maxq = std::max<uint64_t>(maxq, strips_of(q));
@@ -157,36 +145,70 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
   std::vector<uint32_t> lorder(K);
   std::iota(lorder.begin(), lorder.end(), 0u);
   std::stable_sort(lorder.begin(), lorder.end(), [&](uint32_t a, uint32_t b) { return load[a] > load[b]; });
-  std::vector<StripMeta> smeta;
-  std::vector<uint32_t> s_sbase, s_ns;
-  auto lane_meta = [&](const std::vector<uint32_t>& lane, uint64_t s, uint32_t* q, uint32_t* k) {
-    uint64_t start = 0;
+  Streams S;
+  // query and strip index (with the LAST bit) of strip s of a lane, in order
+  auto fill = [&](const std::vector<uint32_t>& lane, uint64_t n, auto put) {
+    uint64_t s = 0;
     for (uint32_t x : lane) {
       const uint32_t ns_q = strips_of(x);
-      if (s < start + ns_q) {
-        *q = x;
-        *k = (uint32_t)(s - start) | (s - start == ns_q - 1 ? LAST : 0u);
-        return;
-      }
-      start += ns_q;
+      for (uint32_t k = 0; k < ns_q; ++k) put(s++, x, k | (k == ns_q - 1 ? LAST : 0u));
     }
-    *q = NONE;
-    *k = 0;
+    for (; s < n; ++s) put(s, NONE, 0u);
   };
   for (uint32_t u = 0; u < K / 2; ++u) {
-    const auto& la = lanes[lorder[2 * u]];
-    const auto& lb = lanes[lorder[2 * u + 1]];
     const uint64_t ns_u = std::max(load[lorder[2 * u]], load[lorder[2 * u + 1]]);
     if (ns_u == 0) continue;
-    s_sbase.push_back((uint32_t)smeta.size());
-    s_ns.push_back((uint32_t)ns_u);
-    for (uint64_t st = 0; st < ns_u; ++st) {
-      StripMeta m;
-      lane_meta(la, st, &m.qa, &m.ka);
-      lane_meta(lb, st, &m.qb, &m.kb);
-      smeta.push_back(m);
-    }
+    const size_t at = S.meta.size();
+    S.sbase.push_back((uint32_t)at);
+    S.ns.push_back((uint32_t)ns_u);
+    S.meta.resize(at + ns_u);
+    fill(lanes[lorder[2 * u]], ns_u, [&](uint64_t st, uint32_t q, uint32_t k) { S.meta[at + st].qa = q; S.meta[at + st].ka = k; });
+    fill(lanes[lorder[2 * u + 1]], ns_u, [&](uint64_t st, uint32_t q, uint32_t k) { S.meta[at + st].qb = q; S.meta[at + st].kb = k; });
   }
+  return S;
+}
+
+// Strip rows of the wavefront search: 24 spread a step's hand-over over more
+// rows, 16 pad short queries less.  Cost per query: strips times (rows of
+// about 11 cycles and a hand-over of about 45).
+int wave_rows(const dsa_db* qs) {
+  auto cost = [&](uint32_t R) {
+    uint64_t c = 0;
+    for (uint32_t m : qs->h_len) c += (uint64_t)((m + R - 1) / R) * (R * 11 + 45);
+    return c;
+  };
+  return cost(16) < cost(24) ? 16 : 24;
+}
+
+// Packed score pass (int16x2).  Targets of groups longer than `long_thr` go
+// to the wavefront kernel, the rest to the inter-sequence kernel; with both,
+// the wavefronts run on the side stream.  The results do not depend on
+// long_thr, only the time.  Global / semi-global use the end-anchored forms
+// of both kernels; searches whose values could pass 16 bits on the wavefronts
+// of k_wave.cu take those of k_intra.cu.
+int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
+                 const int8_t* d_mat, const int8_t* d_pssm, int A, int o, int e, const Validated& v, Scores out,
+                 uint32_t long_thr, int rows, int mode = DSA_LOCAL, uint32_t fe = 15) {
+  const bool local = mode == DSA_LOCAL;
+  const uint32_t W = (uint32_t)rows;   // strip rows of the inter-sequence kernel
+  const uint32_t nq = qs->n, nt = db->n;
+  const int R = A + 1;
+  std::vector<uint32_t> qorder(nq);
+  std::iota(qorder.begin(), qorder.end(), 0u);
+  std::stable_sort(qorder.begin(), qorder.end(),
+                   [&](uint32_t a, uint32_t b) { return qs->h_len[a] > qs->h_len[b]; });
+
+  // groups whose longest target exceeds the threshold go to the wavefront kernel
+  uint32_t g_long = 0;
+  while (g_long < db->n_groups && db->h_glen[g_long] > long_thr) ++g_long;
+  const uint32_t n_long = std::min<uint32_t>(nt, g_long * GROUP);
+  const bool inter = g_long < db->n_groups;
+  const bool wave = n_long && wave_takes(local, qs->max_len, db->h_glen[0], o, e, v.smax, v.smin);
+
+  Streams st;
+  if (inter) st = build_streams(qs, qorder, W);
+  std::vector<StripMeta>& smeta = st.meta;
+  std::vector<uint32_t>&s_sbase = st.sbase, &s_ns = st.ns;
   PackedPlan spl;
   spl.R = R;
   spl.rows = rows;
@@ -219,7 +241,8 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
   std::vector<StripMeta> pmeta;
   std::vector<uint32_t> p_sbase, p_ns, long_ids, litem_words;
   uint64_t long_res = 0;
-  if (n_long) {
+  for (uint32_t li = 0; li < n_long; ++li) long_res += db->h_len[db->h_perm[li]];
+  if (n_long && !wave) {
     ppl.R = R;
     ppl.rows = 32;   // the wavefront kernel's lanes take half-strips of 16 rows
     auto strips32 = [&](uint32_t q) { return (qs->h_len[q] + 31u) / 32u; };
@@ -240,7 +263,6 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
     litems.reserve((size_t)n_long * ppl.n_units);
     for (uint32_t li = 0; li < n_long; ++li) {
       const uint32_t L = db->h_len[long_ids[li]];
-      long_res += L;
       xw.max_long_len = std::max(xw.max_long_len, L);
       for (uint32_t u = 0; u < ppl.n_units; ++u) litems.push_back({(uint64_t)L * p_ns[u], li, u});
     }
@@ -260,22 +282,34 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
     res->phase_cells[PH_INTER] = qsum * (db->n_res - long_res);
   }
 
-  DevBuf d_smeta, d_sbase, d_sns, d_sprof, d_items, d_pmeta, d_pbase, d_pns, d_pprof, d_long, d_litems;
-  DSA_TRY(upload(ctx, d_smeta, smeta));
-  DSA_TRY(upload(ctx, d_sbase, s_sbase));
-  DSA_TRY(upload(ctx, d_sns, s_ns));
-  DSA_TRY(upload(ctx, d_items, item_words));
-  DSA_TRY(d_sprof.alloc(ctx, (size_t)spl.n_strips * R * spl.pitch * sizeof(uint32_t)));
-  spl.d_meta = d_smeta.as<StripMeta>();
-  spl.d_sbase = d_sbase.as<uint32_t>();
-  spl.d_ns = d_sns.as<uint32_t>();
-  spl.d_prof = d_sprof.as<uint32_t>();
-  iw.d_items = d_items.as<uint32_t>();
   // end-anchored strips: the padding rows above a query reproduce row 0
   // (S + o = 0 against the boundary -(o + (j-1)e), o against a free begin)
   const int tpad = (mode == DSA_SEMIGLOBAL && (fe & DSA_FREE_T_BEGIN)) ? o : 0;
-  DSA_TRY(launch_strip_profile(ctx, qs, d_mat, d_pssm, A, o, spl, !local, tpad));
-  if (n_long) {
+  // long targets beside an inter-sequence launch run on the side stream: the
+  // two kernels write disjoint targets' results
+  cudaStream_t ls = ctx->stream;
+  DevBuf d_pmeta, d_pbase, d_pns, d_pprof, d_long, d_litems;
+  if (n_long && inter) {
+    ls = ctx->side;
+    DSA_CUDA_TRY(cudaEventRecord(ctx->fork_ev, ctx->stream));
+    DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0));
+  }
+  if (wave) {
+    const int wr = wave_rows(qs);
+    // longer streams waste fewer lanes and balance the halves better, until the
+    // longest target's pass over a unit would take half the launch: each of the
+    // chip's lanes has total / lanes strip columns to compute, the longest
+    // target's 32 lanes one per column and band
+    uint64_t strips = 0;
+    for (uint32_t m : qs->h_len) strips += (m + wr - 1) / wr;
+    const uint64_t share = strips / 2 * long_res / ((uint64_t)ctx->sm_count * 512);
+    const Streams ws =
+        build_streams(qs, qorder, (uint32_t)wr, 32 * (share / (2ull * db->h_glen[0])));
+    phase_begin(res, PH_INTRA, ls);
+    DSA_TRY(launch_wave_search(ctx, ls, db, qs, d_mat, d_pssm, A, mode, fe, o, e, v.smax, v.smin, wr,
+                               ws.meta, ws.sbase, ws.ns, n_long, out));
+    phase_end(res, PH_INTRA, ls);
+  } else if (n_long) {
     DSA_TRY(upload(ctx, d_pmeta, pmeta));
     DSA_TRY(upload(ctx, d_pbase, p_sbase));
     DSA_TRY(upload(ctx, d_pns, p_ns));
@@ -289,27 +323,66 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
     xw.d_long_ids = d_long.as<uint32_t>();
     xw.d_items = d_litems.as<uint32_t>();
     DSA_TRY(launch_strip_profile(ctx, qs, d_mat, d_pssm, A, o, ppl, !local, tpad));
-    // long targets on the side stream, overlapping the inter-sequence kernel:
-    // the two kernels write disjoint targets' results
-    DSA_CUDA_TRY(cudaEventRecord(ctx->fork_ev, ctx->stream));
-    DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0));
-    phase_begin(res, PH_INTRA, ctx->side);
+    if (inter) {   // the uploads and the profile above
+      DSA_CUDA_TRY(cudaEventRecord(ctx->fork_ev, ctx->stream));
+      DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0));
+    }
+    phase_begin(res, PH_INTRA, ls);
     if (local)
-      DSA_TRY(launch_intra_local16(ctx, ctx->side, db, ppl, xw, o, e, v.smax, out, nt));
+      DSA_TRY(launch_intra_local16(ctx, ls, db, ppl, xw, o, e, v.smax, out, nt));
     else
-      DSA_TRY(launch_intra_glob16(ctx, ctx->side, db, qs, ppl, xw, mode, fe, o, e, v.smax, v.smin,
-                                  out, nt));
-    phase_end(res, PH_INTRA, ctx->side);
-    DSA_CUDA_TRY(cudaEventRecord(ctx->join_ev, ctx->side));
+      DSA_TRY(launch_intra_glob16(ctx, ls, db, qs, ppl, xw, mode, fe, o, e, v.smax, v.smin, out, nt));
+    phase_end(res, PH_INTRA, ls);
   }
-  phase_begin(res, PH_INTER);
-  if (local)
-    DSA_TRY(launch_inter_local16(ctx, db, spl, iw, o, e, v.smax, out, nt));
-  else
-    DSA_TRY(launch_inter_glob16(ctx, db, qs, spl, iw, mode, fe, o, e, v.smax, v.smin, out, nt));
-  phase_end(res, PH_INTER);
-  if (n_long) DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->stream, ctx->join_ev, 0));
+  if (n_long && inter) DSA_CUDA_TRY(cudaEventRecord(ctx->join_ev, ctx->side));
+  if (inter) {
+    DevBuf d_smeta, d_sbase, d_sns, d_sprof, d_items;
+    DSA_TRY(upload(ctx, d_smeta, smeta));
+    DSA_TRY(upload(ctx, d_sbase, s_sbase));
+    DSA_TRY(upload(ctx, d_sns, s_ns));
+    DSA_TRY(upload(ctx, d_items, item_words));
+    DSA_TRY(d_sprof.alloc(ctx, (size_t)spl.n_strips * R * spl.pitch * sizeof(uint32_t)));
+    spl.d_meta = d_smeta.as<StripMeta>();
+    spl.d_sbase = d_sbase.as<uint32_t>();
+    spl.d_ns = d_sns.as<uint32_t>();
+    spl.d_prof = d_sprof.as<uint32_t>();
+    iw.d_items = d_items.as<uint32_t>();
+    DSA_TRY(launch_strip_profile(ctx, qs, d_mat, d_pssm, A, o, spl, !local, tpad));
+    phase_begin(res, PH_INTER);
+    if (local)
+      DSA_TRY(launch_inter_local16(ctx, db, spl, iw, o, e, v.smax, out, nt));
+    else
+      DSA_TRY(launch_inter_glob16(ctx, db, qs, spl, iw, mode, fe, o, e, v.smax, v.smin, out, nt));
+    phase_end(res, PH_INTER);
+  }
+  if (n_long && inter) DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->stream, ctx->join_ev, 0));
   return DSA_OK;
+}
+
+// Targets longer than this go to the wavefronts when nothing is tuned or
+// forced.  The inter-sequence kernel is the faster one where targets abound
+// (32 queries of 64-5,000 against 500,000 targets: 6,900 against 6,100
+// GCUPS), but a thread there works through its target alone: one column of a
+// 28-row strip takes about 1,400 cycles with 16 warps per SM, so its longest
+// item must stay well below the launch (a quarter of it).  5 queries of 60-700
+// against 60,000 targets took 23.3 ms with a threshold of 4,096, 8.6 with
+// 1,024 and 7.2 on the wavefronts alone; 0 where little would be left for the
+// inter-sequence kernel.
+uint32_t model_threshold(const dsa_db* db, const dsa_db* qs) {
+  uint64_t strips = 0, longest = 1;
+  for (uint32_t m : qs->h_len) {
+    const uint64_t n = (m + INTER_ROWS - 1) / INTER_ROWS;
+    strips += n;
+    longest = std::max(longest, n);
+  }
+  const uint64_t pairs = std::max(longest, strips / 2);   // packed strips
+  const double warp_cols = (double)pairs * (double)db->n_res / 32.0;
+  const double total = warp_cols * 344.0 / 608.0;   // cycles at full rate
+  const double thr = 0.25 * total / ((double)longest * 1378.0);
+  const uint32_t t = (uint32_t)std::min(thr, 1e9);
+  uint64_t left = 0;   // residues the inter-sequence kernel would get
+  for (uint32_t g = db->n_groups; g-- > 0 && db->h_glen[g] <= t;) left += (uint64_t)db->h_glen[g] * GROUP;
+  return left * 4 < db->n_res ? 0 : t;
 }
 
 // Strip rows forced by DSA_INTER_ROWS (0: let the tuner choose).
@@ -327,7 +400,6 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
                      const int8_t* d_mat, const int8_t* d_pssm, int A, int o, int e,
                      const Validated& v, Scores out, int mode, uint32_t fe) {
   const bool local = mode == DSA_LOCAL;
-  constexpr uint32_t DEFAULT_THR = 4096;
   const int rows_forced = forced_rows();
   const char* thr_env = getenv("DSA_LONG_THRESHOLD");
   const uint32_t thr_forced = thr_env ? (uint32_t)strtoul(thr_env, nullptr, 10) : 0;
@@ -337,7 +409,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   const char* mode_env = getenv("DSA_AUTOTUNE");
   const std::string tmode = mode_env ? mode_env : "cache";
   const int rows_default = rows_forced ? rows_forced : INTER_ROWS;
-  const uint32_t thr_default = thr_env ? thr_forced : DEFAULT_THR;
+  const uint32_t thr_default = thr_env ? thr_forced : model_threshold(db, qs);
   if (tmode == "off" || (rows_forced && thr_env))
     return run(res, thr_default, rows_default);
   // workload shape key: GPU, driver, mode, alphabet, and log2 bins of the
@@ -351,7 +423,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   int drv = 0;
   cudaDriverGetVersion(&drv);
   char key[512];
-  snprintf(key, sizeof key, "%s|sm%d|drv%d|%s|A%d|q%d|qr%d|qm%d|t%d|tr%d|L%d", prop.name,
+  snprintf(key, sizeof key, "%s|sm%d|drv%d|wave|%s|A%d|q%d|qr%d|qm%d|t%d|tr%d|L%d", prop.name,
            ctx->sm_count, drv, local ? "local" : (mode == DSA_GLOBAL ? "global" : "semi"), A,
            ilog2_bin(qs->n), ilog2_bin(qres), ilog2_bin(qmax), ilog2_bin(db->n),
            ilog2_bin(db->n_res), ilog2_bin(db->max_len));
@@ -396,26 +468,31 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   //    from the default needs a gain of at least 3% (single timings)
   int best_rows = rows_default;
   double best_ms = measure(thr_default, best_rows);
-  if (!rows_forced)
+  if (!rows_forced && groups_over(thr_default) < db->n_groups)
     for (int rows : {INTER_ROWS_SHORT}) {
       const double ms = measure(thr_default, rows);
       if (ms < 0.97 * best_ms) { best_ms = ms; best_rows = rows; }
     }
-  // 2. the long-target threshold, a local search from the
-  //    default by factors of 4 in each direction while it improves;
-  //    thresholds that move the same groups as the last one are skipped
+  // 2. the long-target threshold: every target on the wavefronts, then a local
+  //    search from the default by factors of 4 in each direction while it
+  //    improves; thresholds that move the same groups as the last one are skipped
   uint32_t best = thr_default;
-  if (!thr_env)
+  if (!thr_env) {
+    if (thr_default) {
+      const double ms = measure(0, best_rows);
+      if (ms < 0.97 * best_ms) { best_ms = ms; best = 0; }
+    }
+    const uint64_t start = std::max<uint32_t>(thr_default, 1024);
     for (int dir = -1; dir <= 1 && rc == DSA_OK; dir += 2) {
-      uint64_t cur = DEFAULT_THR;
-      uint32_t last_g = groups_over(DEFAULT_THR);
+      uint64_t cur = start;
+      uint32_t last_g = groups_over(thr_default);
       for (int step = 0; step < 12 && rc == DSA_OK; ++step) {
         const uint64_t nx = dir < 0 ? cur / 4 : cur * 4;
         const uint32_t thr = (dir > 0 && nx >= db->max_len) ? UINT32_MAX : (uint32_t)nx;
         cur = nx;
         const uint32_t g = groups_over(thr);
-        if (g == last_g) {
-          if (thr == 0 || thr == UINT32_MAX) break;
+        if (g == last_g || g == db->n_groups) {
+          if (thr == 0 || thr == UINT32_MAX || g == db->n_groups) break;
           continue;
         }
         last_g = g;
@@ -429,6 +506,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
         if (thr == 0 || thr == UINT32_MAX) break;
       }
     }
+  }
   cudaEventDestroy(ev0);
   cudaEventDestroy(ev1);
   if (rc) {

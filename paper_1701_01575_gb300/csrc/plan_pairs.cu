@@ -22,8 +22,7 @@ namespace dsa {
 // Reads of 150 bp in 500 bp windows, wavefront against per-thread form (ms):
 // semi-global 1,000 pairs 0.15 / 1.12, 60,000 1.28 / 1.63, 120,000 2.52 /
 // 2.57, 200,000 4.17 / 3.97; local 60,000 1.64 / 1.79, 120,000 3.25 / 2.92.
-// Reads of 150 and 250 bp mixed break even near 300,000 and 150,000.
-constexpr uint64_t WAVE_MAX_SHORT_PAIRS = 160000, WAVE_MAX_SHORT_PAIRS_LOCAL = 100000;
+constexpr uint64_t WAVE_MAX_SHORT_PAIRS = 100000;
 
 int PairPass::need_hp(dsa_ctx* ctx) {
   if (hp_ready) return DSA_OK;
@@ -52,7 +51,7 @@ bool pairs_take_wave(const int8_t* matrix, int A, int mode, int o, int e, const 
   // DSA_PAIRS_ROWS fixes a variant of the per-thread form, and re-tuning times it
   const char* tune = getenv("DSA_AUTOTUNE");
   if (getenv("DSA_PAIRS_ROWS") || (tune && std::string(tune) == "retune")) return false;
-  return n_pairs < (mode == DSA_LOCAL ? WAVE_MAX_SHORT_PAIRS_LOCAL : WAVE_MAX_SHORT_PAIRS);
+  return n_pairs < WAVE_MAX_SHORT_PAIRS;
 }
 
 int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairPlanParams& P,
