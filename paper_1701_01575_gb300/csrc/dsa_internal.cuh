@@ -322,6 +322,12 @@ struct TbJob {
   // the checkpoint rows; the table's widths are at most wc
   uint32_t win_off;
 };
+// Decisions of a warp-per-hit job: rows padded to 8, one word per row and 8
+// steps of the wavefront (je columns, up to 31 steps of skew).
+__host__ __device__ inline uint32_t tb_warp_rows(int32_t ie) { return ((uint32_t)ie + 7u) & ~7u; }
+__host__ __device__ inline uint64_t tb_warp_words(int32_t ie, int32_t je) {
+  return (uint64_t)tb_warp_rows(ie) * (((uint32_t)je + 31u + 7u) / 8u);
+}
 // Score-derived traceback windows, shared by the host staging and the
 // device staging of the traceback (see k_traceback.cu for the argument).
 struct TbBounds {

@@ -379,7 +379,7 @@ int tb_run_warp(TbRun& R, std::vector<TbJob>& jobs, uint64_t limit) {
     uint64_t dir = 0, cig = 0, scr = 0;
     size_t k1 = k0;
     while (k1 < jobs.size()) {
-      const uint64_t w = (uint64_t)jobs[k1].ie * jobs[k1].wpr;
+      const uint64_t w = tb_warp_words(jobs[k1].ie, jobs[k1].je);
       if (k1 > k0 && dir + w > limit) break;
       jobs[k1].dir_off = dir;
       jobs[k1].cig_off = cig;
