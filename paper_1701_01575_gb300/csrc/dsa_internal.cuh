@@ -251,15 +251,17 @@ struct IntraWork {
 // with `tpad` as the S + o of padding rows and absent queries.
 int launch_strip_profile(dsa_ctx* ctx, const dsa_db* qs, const int8_t* d_matrix,
                          const int8_t* d_pssm, int A, int o, const PackedPlan& plan,
-                         bool anchored = false, int tpad = 0);
+                         bool anchored = false, int tpad = 0, bool sum = false);
+// sum: the summed form (sum_fits), on a profile built with sum and o + e
+// (local) or 2e (global, tpad 2e or 2e - o) in place of o.
 int launch_inter_local16(dsa_ctx* ctx, const dsa_db* db, const PackedPlan& plan,
-                         const InterWork& work, int o, int e, int smax, Scores out,
+                         const InterWork& work, int o, int e, int smax, bool sum, Scores out,
                          uint32_t n_targets_out);
 // Global / semi-global form of the inter-sequence kernel (end-anchored
 // strips); every target of the database, mode DSA_GLOBAL or DSA_SEMIGLOBAL.
 int launch_inter_glob16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PackedPlan& plan,
                         const InterWork& work, int mode, uint32_t fe, int o, int e, int smax,
-                        int smin, Scores out, uint32_t n_targets_out);
+                        int smin, bool sum, Scores out, uint32_t n_targets_out);
 int inter_blocks_per_sm();
 constexpr int INTER_WARPS = 8;
 constexpr int INTER_ROWS = 28;         // strip rows of the packed inter-sequence kernels
@@ -282,6 +284,8 @@ int launch_intra_glob16(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, con
 // wave_takes: queries of up to max_m against targets of up to max_n residues
 // stay inside its 16-bit range.
 constexpr uint32_t WAVE_LONG_TARGET = 2048;   // longer targets take up to 32 lanes
+int sum_bias(bool local, int o, int e, int smin);
+bool sum_fits(bool local, int64_t m, int64_t n, int o, int e, int smax, int smin);
 bool wave_takes(bool local, uint32_t max_m, uint32_t max_n, int o, int e, int smax, int smin);
 int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, const dsa_db* qs,
                        const int8_t* d_matrix, const int8_t* d_pssm, int A, int mode, uint32_t fe, int o,

@@ -23,7 +23,22 @@
 //   * a persistent grid pops (stream pair, block of 8 groups) items from a
 //     work queue ordered longest-first.
 //
-// Cell update for one row (Gotoh, local), with Ho = H - o and profile S + o:
+// Cell update for one row (Gotoh, local), with Ho = H - o, in two forms.
+//
+// Summed form (SUM), where the launch's scores leave room in 16 bits: values
+// are stored unsigned with a bias and e j added in column j (all of a column's
+// rows alike), the profile holds S + o + e as an integer sum of its halves:
+//   H  = max(Ho_diag + P, E, F)         32-bit add, max3_2u
+//   Ho = H - o                          32-bit subtract
+//   F' = max(F - e, Ho)                 addmax2u  (F of the next row)
+//   E' = max(E, Ho + e, floor(j + 1))   32-bit add, max3_2u
+// Adding e j turns the gap extension of E into nothing, which frees the third
+// operand of its maximum for the floor 0 of local alignment; no half leaves
+// [0, 2^16), so the sums carry nothing between the halves.  Three maxima on the
+// half-rate pipe and three sums, against four and one: 32 queries of 64-5,000
+// against 200,000 targets 413.0 -> 379.3 ms.
+//
+// Wrapping form, with profile S + o:
 //   E  = max(E - e, Ho_left)            addmax2u
 //   t  = max(Ho_diag + (S + o), E)      addmax2u
 //   H  = max(t, F, 0)                   max3_2u
@@ -65,6 +80,8 @@ constexpr int NCOPY = 8;         // profile replicas (one per lane of a quarter-
 constexpr uint32_t RING = 3;     // boundary-row ring slots (blocks of 4 columns)
 
 struct InterArgs {
+  int e;
+  int bias;                        // summed form: the stored value of H = 0 in column 0
   const uint8_t* il;
   const uint64_t* gbase;
   const uint32_t* glen;
@@ -115,11 +132,14 @@ __device__ __forceinline__ void issue_strip(const InterArgs& A, uint8_t* buf, ui
   for (int c = 0; c < NCOPY; ++c) bulk_g2s(buf + c * cstride, src, bytes, bar);
 }
 
-template <int W>
+template <int W, bool SUM>
 __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint64_t bars[2];
   __shared__ uint32_t s_item;
+  // per thread and half, kept out of registers (read when a column triggers
+  // and at a strip's end): best, its column and its row
+  __shared__ int s_best[2][NT], s_bj[2][NT], s_bi[2][NT];
   const int tid = threadIdx.x;
   const int lane = tid & 31;
   const int warp = tid >> 5;
@@ -137,6 +157,9 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
   const uint32_t mo2 = A.neg_o2 ^ BIAS2;                    // -o (offset binary)
   const uint32_t o2 = ((uint32_t)A.o << 16) | (uint32_t)A.o;
   const uint32_t NEG2 = pack2(NEG16, NEG16) ^ BIAS2;
+  const uint32_t e2 = ((uint32_t)A.e << 16) | (uint32_t)A.e;
+  // H = 0 as H - o in column 0, and as the stored H (summed form: plus e j)
+  const uint32_t flo0 = SUM ? (uint32_t)(A.bias - A.o) * 0x10001u : mo2;
 
   if (tid == 0) {
     mbar_init(&bars[0], 1);
@@ -170,7 +193,7 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
     const bool tvalid = gvalid && st < A.n_targets;
     const uint4* res = reinterpret_cast<const uint4*>(A.il + (gvalid ? A.gbase[g] : 0)) + lane;
 
-    int best_lo = 0, best_hi = 0, bj_lo = 0, bj_hi = 0, bi_lo = 0, bi_hi = 0;
+    for (int x = 0; x < 2; ++x) { s_best[x][tid] = 0; s_bj[x][tid] = 0; s_bi[x][tid] = 0; }
 
     for (uint32_t s = 0; s < ns; ++s) {
       const int b = s & 1;
@@ -189,19 +212,18 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
       const uint32_t ka = md.ka & ~LAST, kb = md.kb & ~LAST;
       // a half whose query starts here restarts its best and takes the
       // row-0 boundary (H = 0) instead of the previous strip's bottom row
-      if (ka == 0) { best_lo = 0; bj_lo = 0; bi_lo = 0; }
-      if (kb == 0) { best_hi = 0; bj_hi = 0; bi_hi = 0; }
+      if (ka == 0) { s_best[0][tid] = 0; s_bj[0][tid] = 0; s_bi[0][tid] = 0; }
+      if (kb == 0) { s_best[1][tid] = 0; s_bj[1][tid] = 0; s_bi[1][tid] = 0; }
       const uint32_t keep = (ka == 0 ? 0u : 0x0000FFFFu) | (kb == 0 ? 0u : 0xFFFF0000u);
       const bool first = keep == 0;
-      const int ia = (int)ka * W, ib = (int)kb * W;   // first row of the strip inside each query
-
       uint32_t Ho[W], E[W];
 #pragma unroll
       for (int r = 0; r < W; ++r) {
-        Ho[r] = mo2;
-        E[r] = NEG2;
+        Ho[r] = flo0;
+        E[r] = SUM ? flo0 + o2 + e2 : NEG2;
       }
-      uint32_t diag = mo2;
+      uint32_t diag = flo0;
+      uint32_t flo2 = flo0;   // H = 0 as H - o in the current column
       uint2* scr = scr_base;
       uint4 rv = make_uint4(0, 0, 0, 0);
       // Packed trigger threshold per half, tested as cm > thr with
@@ -209,7 +231,9 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
       // (or is the first positive one) triggers; the exact rule (strictly
       // better, or equal at a smaller column) is applied in the trigger path.
       uint32_t thr2 = 0;
-      auto set_thr = [&]() { thr2 = pack2(max(best_lo - 1, 0), max(best_hi - 1, 0)) ^ BIAS2; };
+      auto set_thr = [&]() {
+        thr2 = pack2(max(s_best[0][tid] - 1, 0), max(s_best[1][tid] - 1, 0)) + (SUM ? flo2 + o2 : BIAS2);
+      };
       set_thr();
       int pend = 0;   // bit 0 / 1: low / high half improved in this strip
 
@@ -240,13 +264,17 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
           if (keep != 0xFFFFFFFFu) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              top[k].x = (top[k].x & keep) | (mo2 & ~keep);
-              top[k].y = (top[k].y & keep) | (mo2 & ~keep);
+              const uint32_t f = SUM ? flo2 + (uint32_t)(k + 1) * e2 : mo2;
+              top[k].x = (top[k].x & keep) | (f & ~keep);
+              top[k].y = (top[k].y & keep) | (f & ~keep);
             }
           }
         } else {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) top[k] = make_uint2(mo2, mo2);
+          for (int k = 0; k < 4; ++k) {
+            const uint32_t f = SUM ? flo2 + (uint32_t)(k + 1) * e2 : mo2;
+            top[k] = make_uint2(f, f);
+          }
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -255,7 +283,13 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
           uint32_t F = top[k].y;
           uint32_t d = diag;
           diag = top[k].x;
-          uint32_t cm = BIAS2, hprev = BIAS2;
+          uint32_t cm = SUM ? 0u : BIAS2, hprev = cm;
+          uint32_t fln2 = 0;   // the floor of the next column
+          if (SUM) {
+            flo2 += e2;
+            thr2 += e2;
+            fln2 = flo2 + o2 + e2;
+          }
 #pragma unroll
           for (int q4 = 0; q4 < W / 4; ++q4) {
             const uint4 pv = prow[q4];
@@ -264,11 +298,20 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
             for (int u = 0; u < 4; ++u) {
               const int r = q4 * 4 + u;
               const uint32_t old = Ho[r];
-              E[r] = addmax2u(E[r], neg_e2, old);
-              const uint32_t t = addmax2u(d, pr[u], E[r]);
-              const uint32_t h = max3_2u(t, F, BIAS2);
-              Ho[r] = h - o2;
-              F = addmax2u(F, neg_e2, Ho[r]);
+              uint32_t h;
+              if (SUM) {
+                h = max3_2u(d + pr[u], E[r], F);
+                const uint32_t ho = h - o2;
+                F = addmax2u(F, neg_e2, ho);
+                E[r] = max3_2u(E[r], ho + e2, fln2);
+                Ho[r] = ho;
+              } else {
+                E[r] = addmax2u(E[r], neg_e2, old);
+                const uint32_t t = addmax2u(d, pr[u], E[r]);
+                h = max3_2u(t, F, BIAS2);
+                Ho[r] = h - o2;
+                F = addmax2u(F, neg_e2, Ho[r]);
+              }
               d = old;
               if (r & 1) cm = max3_2u(cm, hprev, h);
               else hprev = h;
@@ -278,22 +321,23 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
           // end-cell tracking for column j: trigger when cm > thr (per half)
           const int j = (int)c4 + k + 1;
           if (__vmaxu2(cm, thr2) != thr2) {   // some half has cm > thr
-            const int cl = lo16(cm ^ BIAS2), ch = hi16(cm ^ BIAS2);
-            const int thr_lo = best_lo - (j < bj_lo ? 1 : 0);
-            const int thr_hi = best_hi - (j < bj_hi ? 1 : 0);
+            const int z = SUM ? (int)(flo2 & 0xFFFFu) + A.o : 0x8000;   // H = 0
+            const int cl = (int)(cm & 0xFFFFu) - z, ch = (int)(cm >> 16) - z;
+            const int thr_lo = s_best[0][tid] - (j < s_bj[0][tid] ? 1 : 0);
+            const int thr_hi = s_best[1][tid] - (j < s_bj[1][tid] ? 1 : 0);
             // rare: a half improved.  Park the column in that half's area of
             // shared memory; its first row holding the maximum is looked up
             // once, at the end of the strip (a later trigger of the same half
             // supersedes this one)
             if (cl > thr_lo) {
 #pragma unroll
-              for (int r = 0; r < W; ++r) park_lo[r * NT + tid] = (int16_t)lo16(Ho[r] ^ BIAS2);
-              best_lo = cl; bj_lo = j; pend |= 1;
+              for (int r = 0; r < W; ++r) park_lo[r * NT + tid] = (int16_t)(Ho[r] & 0xFFFFu);
+              s_best[0][tid] = cl; s_bj[0][tid] = j; pend |= 1;
             }
             if (ch > thr_hi) {
 #pragma unroll
-              for (int r = 0; r < W; ++r) park_hi[r * NT + tid] = (int16_t)hi16(Ho[r] ^ BIAS2);
-              best_hi = ch; bj_hi = j; pend |= 2;
+              for (int r = 0; r < W; ++r) park_hi[r * NT + tid] = (int16_t)(Ho[r] >> 16);
+              s_best[1][tid] = ch; s_bj[1][tid] = j; pend |= 2;
             }
             set_thr();
           }
@@ -301,35 +345,33 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
       }
       cp_async_wait<0>();   // nothing in flight into the ring past the strip
       if (pend & 1) {   // first row of the last improving column, low half
-        const int want = best_lo - A.o;
+        const int16_t want = (int16_t)(s_best[0][tid] - A.o + (SUM ? A.bias + A.e * s_bj[0][tid] : 0x8000));
         int rr = W - 1;
         for (int r = W - 1; r >= 0; --r)
           if (park_lo[r * NT + tid] == want) rr = r;
-        bi_lo = ia + rr + 1;
+        s_bi[0][tid] = (int)ka * W + rr + 1;
       }
       if (pend & 2) {
-        const int want = best_hi - A.o;
+        const int16_t want = (int16_t)(s_best[1][tid] - A.o + (SUM ? A.bias + A.e * s_bj[1][tid] : 0x8000));
         int rr = W - 1;
         for (int r = W - 1; r >= 0; --r)
           if (park_hi[r * NT + tid] == want) rr = r;
-        bi_hi = ib + rr + 1;
+        s_bi[1][tid] = (int)kb * W + rr + 1;
       }
       if (tvalid) {   // queries that end in this strip: write their results
         const uint32_t orig = A.perm[st];
-        if ((md.ka & LAST) && md.qa != NONE) {
-          const uint64_t idx = (uint64_t)md.qa * A.n_out_t + orig;
-          A.o_score[idx] = best_lo;
-          A.o_qend[idx] = best_lo > 0 ? bi_lo - 1 : -1;
-          A.o_tend[idx] = best_lo > 0 ? bj_lo - 1 : -1;
-          A.o_flag[idx] = best_lo > A.T ? 1 : 0;
-        }
-        if ((md.kb & LAST) && md.qb != NONE) {
-          const uint64_t idx = (uint64_t)md.qb * A.n_out_t + orig;
-          A.o_score[idx] = best_hi;
-          A.o_qend[idx] = best_hi > 0 ? bi_hi - 1 : -1;
-          A.o_tend[idx] = best_hi > 0 ? bj_hi - 1 : -1;
-          A.o_flag[idx] = best_hi > A.T ? 1 : 0;
-        }
+        auto put = [&](int x, uint32_t q, uint32_t kq) {
+          if (!(kq & LAST) || q == NONE) return;
+          const uint64_t idx = (uint64_t)q * A.n_out_t + orig;
+          const int best = s_best[x][tid];
+          A.o_score[idx] = best;
+          A.o_qend[idx] = best > 0 ? s_bi[x][tid] - 1 : -1;
+          A.o_tend[idx] = best > 0 ? s_bj[x][tid] - 1 : -1;
+          A.o_flag[idx] = best > A.T ? 1 : 0;
+        };
+        const StripMeta mr = A.meta[sb + s];   // reloaded: not kept live over the column loop
+        put(0, mr.qa, mr.ka);
+        put(1, mr.qb, mr.kb);
       }
       __syncthreads();
       if (tid == 0 && s + 2 < ns) {
@@ -344,7 +386,14 @@ __global__ void __launch_bounds__(NT, 2) k_inter_local16(const InterArgs A) {
 // ---- global and semi-global form (Sec. II.C.2: DNW, DSG) ----
 //
 // Same work decomposition, staging and cell update as k_inter_local16, with
-// three differences:
+// four differences:
+//   * summed form (SUM): e (i + j) is added to the stored values, i the row of
+//     the query with its padding rows, so that extending either gap adds
+//     nothing: with G = H + e (i + j) and P = S + 2e,
+//       G = max(G_diag + P, E, F);  E' = max(G + e - o, E);  F' = max(G + e - o, F)
+//     -- three maxima and one sum; its launches cannot pass 16 bits in either
+//     direction (sum_fits), so no range is watched (32 queries of 64-2,500
+//     against 200,000 targets, global: 245.0 -> 173.8 ms);
 //   * no floor at 0: H = max(t, F) (max3_2u(t, F, t));
 //   * end-anchored strips: a query of m rows starts (W - m % W) % W rows into
 //     its first strip, so row m is the bottom register of its last strip.
@@ -379,7 +428,7 @@ struct GlobArgs {
 
 // TB: free target begin (row 0 is 0), TE: free target end (row m is
 // tracked): compile-time, so each form carries only the state it uses.
-template <int W, bool TB, bool TE>
+template <int W, bool TB, bool TE, bool SUM>
 __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const GlobArgs G) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint64_t bars[2];
@@ -405,6 +454,7 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
   const int o = A.o, e = G.e;
   const uint32_t NEGG2 = ((uint32_t)e << 16) | (uint32_t)e;   // -2^15 + e in both halves
   const uint32_t neg_e4 = pack2(-4 * e, -4 * e);              // four columns of the boundary
+  const uint32_t c2 = pack2(e - o, e - o);                    // SUM: opening a gap
   const bool sg = G.mode == DSA_SEMIGLOBAL;
   constexpr bool tb_free = TB;
   constexpr bool te_free = TE;
@@ -415,6 +465,9 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
   auto row0 = [&](int j) { return (j == 0 || tb_free) ? 0 : -(o + (j - 1) * e); };
   auto col0 = [&](int i) { return (i <= 0 || qb_free) ? 0 : -(o + (i - 1) * e); };
   auto off2 = [](int lo, int hi) { return pack2(lo, hi) ^ BIAS2; };
+  const int bias = A.bias;
+  // SUM: row 0 at column j (1-based) as stored
+  auto sum0 = [&](int j) { return bias + row0(j) + e * j; };
 
   if (tid == 0) {
     mbar_init(&bars[0], 1);
@@ -482,12 +535,20 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
       const bool first = keep == 0;
 
       uint32_t Ho[W], E[W];
+      // SUM: strips above a query's end count its rows with the padding
+      const int ra = (int)ka * W, rb = (int)kb * W;
 #pragma unroll
       for (int r = 0; r < W; ++r) {
-        Ho[r] = off2(col0(ia0 + r + 1) - o, col0(ib0 + r + 1) - o);
-        E[r] = NEGG2;
+        if (SUM) {
+          Ho[r] = pack2(bias + col0(ia0 + r + 1) + e * (ra + r + 1), bias + col0(ib0 + r + 1) + e * (rb + r + 1));
+          E[r] = add2(Ho[r], c2);
+        } else {
+          Ho[r] = off2(col0(ia0 + r + 1) - o, col0(ib0 + r + 1) - o);
+          E[r] = NEGG2;
+        }
       }
-      uint32_t diag = off2(col0(ia0) - o, col0(ib0) - o);
+      uint32_t diag = SUM ? pack2(bias + col0(ia0) + e * ra, bias + col0(ib0) + e * rb)
+                          : off2(col0(ia0) - o, col0(ib0) - o);
       // row-0 boundary as (H - o, F of row 1) = (B(j) - o, B(j) - o) at the
       // first column of the current block of 4 (only read where a half starts
       // a query)
@@ -495,10 +556,13 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
       // bottom row of a last strip (row m), free target end: best H - o over
       // j <= n, smallest j first, from the candidate (m, 0); a half that does
       // not end here holds the largest value, which nothing exceeds
-      uint32_t rthr = 0xFFFFFFFFu;
+      uint32_t rthr = 0xFFFFFFFFu, rinc = 0;
       s_rj[0][tid] = 0;
       s_rj[1][tid] = 0;
-      if (te_free) {
+      if (te_free && SUM) {   // as stored: the threshold moves with e j
+        if (last_a) { rthr = (rthr & 0xFFFF0000u) | (uint32_t)(bias + col0(ma) + e * (ra + W)); rinc |= (uint32_t)e; }
+        if (last_b) { rthr = (rthr & 0x0000FFFFu) | (uint32_t)(bias + col0(mb) + e * (rb + W)) << 16; rinc |= (uint32_t)e << 16; }
+      } else if (te_free) {
         if (last_a) rthr = (rthr & 0xFFFF0000u) | (off2(col0(ma) - o, 0) & 0xFFFFu);
         if (last_b) rthr = (rthr & 0x0000FFFFu) | (off2(0, col0(mb) - o) & 0xFFFF0000u);
       }
@@ -532,8 +596,10 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
             uint32_t bk = bt;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              top[k].x = (top[k].x & keep) | (bk & ~keep);
-              top[k].y = (top[k].y & keep) | (bk & ~keep);
+              const uint32_t bx = SUM ? (uint32_t)sum0((int)c4 + k + 1) * 0x10001u : bk;
+              const uint32_t by = SUM ? (uint32_t)(sum0((int)c4 + k + 1) + e - o) * 0x10001u : bk;
+              top[k].x = (top[k].x & keep) | (bx & ~keep);
+              top[k].y = (top[k].y & keep) | (by & ~keep);
               if (!tb_free) bk = __vadd2(bk, neg_e2);
             }
           }
@@ -541,7 +607,9 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
           uint32_t bk = bt;
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            top[k] = make_uint2(bk, bk);
+            top[k] = SUM ? make_uint2((uint32_t)sum0((int)c4 + k + 1) * 0x10001u,
+                                      (uint32_t)(sum0((int)c4 + k + 1) + e - o) * 0x10001u)
+                         : make_uint2(bk, bk);
             if (!tb_free) bk = __vadd2(bk, neg_e2);
           }
         }
@@ -562,14 +630,21 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
             for (int u = 0; u < 4; ++u) {
               const int r = q4 * 4 + u;
               const uint32_t old = Ho[r];
-              E[r] = addmax2u(E[r], neg_e2, old);
-              const uint32_t t = addmax2u(d, pr[u], E[r]);
-              const uint32_t h = max3_2u(t, F, t);
-              Ho[r] = h - o2;
-              F = addmax2u(F, neg_e2, Ho[r]);
+              if (SUM) {
+                const uint32_t h = max3_2u(d + pr[u], E[r], F);
+                E[r] = addmax2u(h, c2, E[r]);
+                F = addmax2u(h, c2, F);
+                Ho[r] = h;
+              } else {
+                E[r] = addmax2u(E[r], neg_e2, old);
+                const uint32_t t = addmax2u(d, pr[u], E[r]);
+                const uint32_t h = max3_2u(t, F, t);
+                Ho[r] = h - o2;
+                F = addmax2u(F, neg_e2, Ho[r]);
+                if (r & 1) cm = max3_2u(cm, hprev, h);
+                else hprev = h;
+              }
               d = old;
-              if (r & 1) cm = max3_2u(cm, hprev, h);
-              else hprev = h;
             }
           }
           scr[(uint64_t)(c4 + k) * NT] = make_uint2(Ho[W - 1], F);
@@ -577,7 +652,7 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
           // upward range test of the column (rare); columns past the lane's
           // target end feed no real cell (values only move right and down)
           // and may wrap in a long group: left out
-          if (__vmaxu2(cm, G.hmax2) != G.hmax2 && j <= nl)
+          if (!SUM && __vmaxu2(cm, G.hmax2) != G.hmax2 && j <= nl)
             s_sat[tid] |= ((cm & 0xFFFFu) > (G.hmax2 & 0xFFFFu) ? 1u : 0u) |
                           ((cm >> 16) > (G.hmax2 >> 16) ? 2u : 0u);
           if (j == nl) {   // the lane's own target end: park the column
@@ -585,6 +660,7 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
             for (int r = 0; r < W; ++r) park[r * NT + tid] = Ho[r];
           }
           if (te_free) {
+            if (SUM) rthr += rinc;
             const uint32_t cur = Ho[W - 1];
             if (__vmaxu2(cur, rthr) != rthr && j <= nl) {
               if ((cur & 0xFFFFu) > (rthr & 0xFFFFu)) {
@@ -601,38 +677,43 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
       }
       cp_async_wait<0>();
       if (tvalid) {
-        // H of half `sh` (0 / 16) from a packed H - o in offset binary
-        auto hval = [&](uint32_t w, int sh) { return (int)((w >> sh) & 0xFFFFu) - 0x8000 + o; };
+        // H of half `sh` (0 / 16) from a packed H - o in offset binary, or as
+        // stored at padded row r and column j
+        auto hval = [&](uint32_t w, int sh, int r, int j) {
+          const int v = (int)((w >> sh) & 0xFFFFu);
+          return SUM ? v - bias - e * (r + j) : v - 0x8000 + o;
+        };
         auto finish = [&](int h, uint32_t q, uint32_t kq) {
           const int sh = 16 * h;
           int m, i0;
           bool last;
           geom(q, kq, m, i0, last);
+          const int r0 = (int)(kq & ~LAST) * W;   // padded rows above the strip
           int cb = s_cb[h][tid], ci = s_ci[h][tid];
           const int rj = s_rj[h][tid];
           if (qe_free) {   // column n of this strip's real rows, smallest i first
             for (int r = 0; r < W; ++r) {
               const int i = i0 + r + 1;
-              const int v = hval(park[r * NT + tid], sh);
+              const int v = hval(park[r * NT + tid], sh, r0 + r + 1, nl);
               if (i >= 1 && v > cb) { cb = v; ci = i; }
             }
           }
           s_cb[h][tid] = cb;
           s_ci[h][tid] = ci;
           if (!last) return;
-          int bs = hval(park[(W - 1) * NT + tid], sh), bi = m, bj = nl;   // (m, n)
+          int bs = hval(park[(W - 1) * NT + tid], sh, r0 + W, nl), bi = m, bj = nl;   // (m, n)
           if (qe_free && (cb > bs || (cb == bs && ci < bi))) { bs = cb; bi = ci; }
           if (te_free) {
-            const int rvv = hval(rthr, sh);
+            const int rvv = hval(rthr, sh, r0 + W, (int)ncol);   // the threshold stands at the last column
             if (rvv > bs || (rvv == bs && rj < bj)) { bs = rvv; bi = m; bj = rj; }
           }
-          const bool up = (s_sat[tid] >> h) & 1u;
+          const bool up = !SUM && ((s_sat[tid] >> h) & 1u);
           const int64_t low = 4ll * o + (int64_t)(m + nl + 2) * e + (G.smin < 0 ? -G.smin : 0) + 64;
           const uint64_t idx = (uint64_t)q * A.n_out_t + A.perm[st];
           A.o_score[idx] = bs;
           A.o_qend[idx] = bi - 1;
           A.o_tend[idx] = bj - 1;
-          A.o_flag[idx] = (up || low >= 32768) ? 1 : 0;
+          A.o_flag[idx] = (!SUM && (up || low >= 32768)) ? 1 : 0;
         };
         const StripMeta mr = A.meta[sb + s];   // reloaded: not kept live over the column loop
         if (mr.qa != NONE) finish(0, mr.qa, mr.ka);
@@ -659,12 +740,15 @@ __global__ void __launch_bounds__(NT, 2) k_inter_glob16(const InterArgs A, const
 // rows past its end, absent queries and the padding residue get values that
 // keep every cell inside the int16 range: `tpad` (S + o) for padding rows and
 // absent queries, 0 for the padding residue of a real row.
+//
+// sum: the words are integer sums (hi << 16) + lo of the summed forms, `o` is
+// what those add to S, and NEG16 becomes a score just below any.
 __global__ void k_strip_profile(const uint8_t* __restrict__ qcodes,
                                 const uint64_t* __restrict__ qoff, const uint32_t* __restrict__ qlen,
                                 const StripMeta* __restrict__ meta, uint32_t n_strips,
                                 const int8_t* __restrict__ S, const int8_t* __restrict__ P, int A,
                                 int R, int rows, int pitch, int o, int anchored, int tpad,
-                                uint32_t* __restrict__ prof) {
+                                int sum, uint32_t* __restrict__ prof) {
   auto sub = [&](uint32_t q, int i, int a) -> int {
     const uint64_t k = qoff[q] + (uint64_t)i;
     return P ? (int)P[k * A + a] : (int)S[qcodes[k] * A + a];
@@ -676,9 +760,10 @@ __global__ void k_strip_profile(const uint8_t* __restrict__ qcodes,
     // rows above the query, and (in a unit of the wavefront kernel, whose
     // halves can differ in strips) rows past its end
     if (i < 0 || i >= m) return tpad;
-    if (a >= A) return 0;
+    if (a >= A) return sum ? tpad : 0;
     return sub(q, i, a) + o;
   };
+  const int none = sum ? -128 : NEG16;
   const uint64_t total = (uint64_t)n_strips * R * pitch;
   for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < total;
        x += (uint64_t)gridDim.x * blockDim.x) {
@@ -686,7 +771,7 @@ __global__ void k_strip_profile(const uint8_t* __restrict__ qcodes,
     const int a = (int)((x / pitch) % (uint64_t)R);
     const int r = (int)(x % pitch);
     const StripMeta md = meta[s];
-    int lo = NEG16, hi = NEG16;
+    int lo = none, hi = none;
     if (r >= rows) {
       // row padding, never read
     } else if (anchored) {
@@ -700,7 +785,7 @@ __global__ void k_strip_profile(const uint8_t* __restrict__ qcodes,
       const int i = (int)(md.kb & ~LAST) * rows + r;
       if (i < (int)qlen[md.qb]) hi = sub(md.qb, i, a) + o;
     }
-    prof[x] = pack2(lo, hi);
+    prof[x] = sum ? ((uint32_t)hi << 16) + (uint32_t)lo : pack2(lo, hi);
   }
 }
 
@@ -710,7 +795,7 @@ int inter_blocks_per_sm() { return 2; }
 
 int launch_strip_profile(dsa_ctx* ctx, const dsa_db* qs, const int8_t* d_matrix,
                          const int8_t* d_pssm, int A, int o, const PackedPlan& plan,
-                         bool anchored, int tpad) {
+                         bool anchored, int tpad, bool sum) {
   if (plan.n_strips == 0) return DSA_OK;
   const uint64_t total = (uint64_t)plan.n_strips * plan.R * plan.pitch;
   uint64_t blocks = std::min<uint64_t>((total + 255) / 256, (uint64_t)ctx->sm_count * 8);
@@ -718,17 +803,19 @@ int launch_strip_profile(dsa_ctx* ctx, const dsa_db* qs, const int8_t* d_matrix,
                                                             plan.d_meta, plan.n_strips, d_matrix,
                                                             d_pssm, A, plan.R, plan.rows,
                                                             plan.pitch, o, anchored ? 1 : 0, tpad,
-                                                            plan.d_prof);
+                                                            sum ? 1 : 0, plan.d_prof);
   DSA_CUDA_TRY(cudaGetLastError());
   ++ctx->launches;
   return DSA_OK;
 }
 
 int launch_inter_local16(dsa_ctx* ctx, const dsa_db* db, const PackedPlan& plan,
-                         const InterWork& work, int o, int e, int smax, Scores out,
+                         const InterWork& work, int o, int e, int smax, bool sum, Scores out,
                          uint32_t n_targets_out) {
   if (work.n_items == 0) return DSA_OK;
   InterArgs A;
+  A.e = e;
+  A.bias = sum_bias(true, o, e, 0);
   A.il = db->d_il; A.gbase = db->d_gbase; A.glen = db->d_glen; A.perm = db->d_perm;
   A.n_targets = db->n; A.n_groups = db->n_groups;
   A.prof = plan.d_prof; A.meta = plan.d_meta; A.sbase = plan.d_sbase; A.nstrips = plan.d_ns;
@@ -751,8 +838,9 @@ int launch_inter_local16(dsa_ctx* ctx, const dsa_db* db, const PackedPlan& plan,
   A.status = ctx->d_status;
   const size_t smem = 2ull * NCOPY * replica_stride(plan.R) + 2ull * plan.rows * NT * sizeof(int16_t) +
                       (size_t)RING * 4 * NT * sizeof(uint2);
-  auto kern = plan.rows == INTER_ROWS_SHORT ? k_inter_local16<INTER_ROWS_SHORT>
-                                            : k_inter_local16<INTER_ROWS>;
+  auto kern = plan.rows == INTER_ROWS_SHORT
+                  ? (sum ? k_inter_local16<INTER_ROWS_SHORT, true> : k_inter_local16<INTER_ROWS_SHORT, false>)
+                  : (sum ? k_inter_local16<INTER_ROWS, true> : k_inter_local16<INTER_ROWS, false>);
   if (plan.rows != INTER_ROWS && plan.rows != INTER_ROWS_SHORT) {
     ctx->release(scr, scr_bytes);
     set_error("strip height %d has no kernel", plan.rows);
@@ -774,9 +862,11 @@ int launch_inter_local16(dsa_ctx* ctx, const dsa_db* db, const PackedPlan& plan,
 
 int launch_inter_glob16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PackedPlan& plan,
                         const InterWork& work, int mode, uint32_t fe, int o, int e, int smax,
-                        int smin, Scores out, uint32_t n_targets_out) {
+                        int smin, bool sum, Scores out, uint32_t n_targets_out) {
   if (work.n_items == 0) return DSA_OK;
   InterArgs A;
+  A.e = e;
+  A.bias = sum_bias(false, o, e, smin);
   A.il = db->d_il; A.gbase = db->d_gbase; A.glen = db->d_glen; A.perm = db->d_perm;
   A.n_targets = db->n; A.n_groups = db->n_groups;
   A.prof = plan.d_prof; A.meta = plan.d_meta; A.sbase = plan.d_sbase; A.nstrips = plan.d_ns;
@@ -807,8 +897,11 @@ int launch_inter_glob16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const 
   const bool tb = sg && (fe & DSA_FREE_T_BEGIN), te = sg && (fe & DSA_FREE_T_END);
   auto pick = [&](auto w) {
     constexpr int Wc = decltype(w)::value;
-    return tb ? (te ? k_inter_glob16<Wc, true, true> : k_inter_glob16<Wc, true, false>)
-              : (te ? k_inter_glob16<Wc, false, true> : k_inter_glob16<Wc, false, false>);
+    if (sum)
+      return tb ? (te ? k_inter_glob16<Wc, true, true, true> : k_inter_glob16<Wc, true, false, true>)
+                : (te ? k_inter_glob16<Wc, false, true, true> : k_inter_glob16<Wc, false, false, true>);
+    return tb ? (te ? k_inter_glob16<Wc, true, true, false> : k_inter_glob16<Wc, true, false, false>)
+              : (te ? k_inter_glob16<Wc, false, true, false> : k_inter_glob16<Wc, false, false, false>);
   };
   auto kern = plan.rows == INTER_ROWS_SHORT ? pick(std::integral_constant<int, INTER_ROWS_SHORT>{})
                                             : pick(std::integral_constant<int, INTER_ROWS>{});

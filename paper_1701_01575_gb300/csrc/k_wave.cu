@@ -530,22 +530,30 @@ __global__ void k_wave_profile(const ProfArgs W) {
   }
 }
 
-// The form of a local launch, or of a global one (-1: k_intra.cu's kernel):
-// whether values with e j or e (i + j) added stay inside 16 bits for queries
-// of up to m and targets of up to n residues.
-int local_bias(int o, int e) { return 512 + o + 64 * e; }
-int global_bias(int o, int e, int smin) { return 4 * o + 64 * e + std::max(0, -smin) + 256; }
+// The form of a local launch, or of a global one (-1: k_intra.cu's kernel).
 int wave_form(bool local, int64_t m, int64_t n, int o, int e, int smax, int smin) {
-  const int64_t up = (int64_t)std::max(0, smax) * std::min(m, n);
-  if (local) {
-    return up + e * (n + 64) + local_bias(o, e) + 2ll * (o + e) + 512 < 65536 ? LOCAL_SUM : LOCAL_WRAP;
-  }
-  if (up > 32767 - std::max(0, smax)) return -1;
-  if (4ll * o + (m + n + 2) * e + std::max(0, -smin) + 64 >= 32768) return -1;
-  return up + e * (m + n + 256) + global_bias(o, e, smin) + 2ll * (o + e) + 512 < 65536 ? GLOBAL_SUM : -1;
+  if (sum_fits(local, m, n, o, e, smax, smin)) return local ? LOCAL_SUM : GLOBAL_SUM;
+  return local ? LOCAL_WRAP : -1;
 }
 
 }  // namespace
+
+// The stored value of 0 in the summed forms: every value stays above 0 (gaps
+// fall 3o below, a lane starts up to 63 columns before its target, the score
+// of an absent row is -128).
+int sum_bias(bool local, int o, int e, int smin) {
+  return local ? 512 + o + 64 * e : 4 * o + 64 * e + std::max(0, -smin) + 256;
+}
+// Values with e j (local) or e (i + j) added stay inside 16 bits for queries of
+// up to m and targets of up to n residues; global: and none could have been
+// flagged by the wrapping form's range rules.
+bool sum_fits(bool local, int64_t m, int64_t n, int o, int e, int smax, int smin) {
+  const int64_t up = (int64_t)std::max(0, smax) * std::min(m, n);
+  if (local) return up + e * (n + 64) + sum_bias(true, o, e, smin) + 2ll * (o + e) + 512 < 65536;
+  if (up > 32767 - std::max(0, smax)) return false;
+  if (4ll * o + (m + n + 2) * e + std::max(0, -smin) + 64 >= 32768) return false;
+  return up + e * (m + n + 256) + sum_bias(false, o, e, smin) + 2ll * (o + e) + 512 < 65536;
+}
 
 bool wave_takes(bool local, uint32_t max_m, uint32_t max_n, int o, int e, int smax, int smin) {
   return wave_form(local, max_m, max_n, o, e, smax, smin) >= 0;
@@ -611,7 +619,7 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   W.tcodes = db->d_codes; W.toff = db->d_off; W.tlen = db->d_len; W.perm = db->d_perm;
   W.qlen = qs->d_len;
   W.A = A; W.o = o; W.e = e; W.mode = mode; W.fe = fe;
-  W.bias = local ? local_bias(o, e) : global_bias(o, e, smin);
+  W.bias = sum_bias(local, o, e, smin);
   W.T = 32767 - std::max(0, smax);
   ProfArgs P{};
   P.qcodes = qs->d_codes; P.qoff = qs->d_off; P.qlen = qs->d_len;

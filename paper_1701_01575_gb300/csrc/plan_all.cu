@@ -347,12 +347,15 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
     spl.d_ns = d_sns.as<uint32_t>();
     spl.d_prof = d_sprof.as<uint32_t>();
     iw.d_items = d_items.as<uint32_t>();
-    DSA_TRY(launch_strip_profile(ctx, qs, d_mat, d_pssm, A, o, spl, !local, tpad));
+    const bool sum = sum_fits(local, qs->max_len, iw.max_glen, o, e, v.smax, v.smin);
+    DSA_TRY(sum ? launch_strip_profile(ctx, qs, d_mat, d_pssm, A, local ? o + e : 2 * e, spl, !local,
+                                       2 * e - (tpad ? 0 : o), true)
+                : launch_strip_profile(ctx, qs, d_mat, d_pssm, A, o, spl, !local, tpad));
     phase_begin(res, PH_INTER);
     if (local)
-      DSA_TRY(launch_inter_local16(ctx, db, spl, iw, o, e, v.smax, out, nt));
+      DSA_TRY(launch_inter_local16(ctx, db, spl, iw, o, e, v.smax, sum, out, nt));
     else
-      DSA_TRY(launch_inter_glob16(ctx, db, qs, spl, iw, mode, fe, o, e, v.smax, v.smin, out, nt));
+      DSA_TRY(launch_inter_glob16(ctx, db, qs, spl, iw, mode, fe, o, e, v.smax, v.smin, sum, out, nt));
     phase_end(res, PH_INTER);
   }
   if (n_long && inter) DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->stream, ctx->join_ev, 0));
