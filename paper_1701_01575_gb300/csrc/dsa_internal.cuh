@@ -541,13 +541,14 @@ struct LongPair16 {
 // best from those.
 bool long16_range_ok(int o, int e, int smax, int smin);
 int launch_long_score16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int8_t* d_matrix,
-                        int A, int o, int e, int mode, uint32_t fe, const LongJob* d_jobs,
-                        uint32_t n_jobs, const LongPair16* d_pjobs, const uint32_t* d_items,
+                        int A, int o, int e, int smax, int smin, int mode, uint32_t fe,
+                        const LongJob* d_jobs, uint32_t n_jobs, const LongPair16* d_pjobs,
+                        const uint32_t* d_items,
                         uint32_t n_items, int2* d_bnd, uint32_t* d_prog, void* d_cands,
-                        Scores out, int blocks_per_sm = 0, const uint32_t* d_litems = nullptr,
+                        Scores out, int rows, int blocks_per_sm = 0, const uint32_t* d_litems = nullptr,
                         uint32_t n_litems = 0, uint64_t n_slots = 0);
 int launch_long_reduce(dsa_ctx* ctx, const LongJob* d_jobs, uint32_t n_jobs, const void* d_cands,
-                       int mode, uint32_t fe, int o, int e, Scores out);
+                       int band_rows, int mode, uint32_t fe, int o, int e, Scores out);
 size_t long_cand_size();
 int long_band_rows();   // rows of a score-pass band
 int long_ckpt_rows();   // rows between traceback checkpoints (a traceback band)

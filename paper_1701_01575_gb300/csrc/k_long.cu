@@ -308,12 +308,12 @@ __global__ void __launch_bounds__(WARPS * 32, 4) k_long_score(
 }
 
 __global__ void k_long_reduce(const LongJob* __restrict__ jobs, uint32_t n_jobs,
-                              const Cand* __restrict__ cands, int mode, uint32_t fe, int o, int e,
+                              const Cand* __restrict__ cands, int band, int mode, uint32_t fe, int o, int e,
                               int32_t* __restrict__ o_score, int32_t* __restrict__ o_qend,
                               int32_t* __restrict__ o_tend, uint8_t* __restrict__ o_flag) {
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n_jobs; k += gridDim.x * blockDim.x) {
     const LongJob jb = jobs[k];
-    const int32_t nb = (jb.m + BAND - 1) / BAND;
+    const int32_t nb = (jb.m + band - 1) / band;
     Cand best = {0, 0, 0, 0};
     if (mode == DSA_SEMIGLOBAL && (fe & DSA_FREE_Q_END))
       best = {h_row0(mode, fe, jb.n, o, e), 0, jb.n, 1};   // H[0][n]
@@ -816,15 +816,15 @@ int launch_long_score(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const in
                                               static_cast<Cand*>(d_cands), ctx->d_status);
   DSA_CUDA_TRY(cudaGetLastError());
   ++ctx->launches;
-  return launch_long_reduce(ctx, d_jobs, n_jobs, d_cands, mode, fe, o, e, out);
+  return launch_long_reduce(ctx, d_jobs, n_jobs, d_cands, BAND, mode, fe, o, e, out);
 }
 
 int launch_long_reduce(dsa_ctx* ctx, const LongJob* d_jobs, uint32_t n_jobs, const void* d_cands,
-                       int mode, uint32_t fe, int o, int e, Scores out) {
+                       int band_rows, int mode, uint32_t fe, int o, int e, Scores out) {
   const unsigned rb = (unsigned)std::min<uint64_t>((n_jobs + 127) / 128, 1024);
   k_long_reduce<<<rb, 128, 0, ctx->stream>>>(d_jobs, n_jobs, static_cast<const Cand*>(d_cands),
-                                              mode, fe, o, e, out.score, out.q_end, out.t_end,
-                                              out.flag);
+                                              band_rows, mode, fe, o, e, out.score, out.q_end,
+                                              out.t_end, out.flag);
   DSA_CUDA_TRY(cudaGetLastError());
   ++ctx->launches;
   return DSA_OK;

@@ -5,7 +5,7 @@
 //
 // Layout.  A unit is two long pairs (sorted neighbours by query length);
 // band b of the unit covers rows 512b+1 .. 512b+512 of both, lane k owns 16
-// of those rows and processes column j = step - k.  The unit runs max(nA,
+// of those rows (or 256 and 8, see ROWS) and processes column j = step - k.  The unit runs max(nA,
 // nB) columns and max(bands) bands; rows past a pair's end and columns past
 // its window are computed in its half but never read for it (the half's
 // results and checkpoints are taken from its own rows and columns only, and
@@ -61,14 +61,12 @@
 namespace dsa {
 namespace {
 
-constexpr int ROWS = 16;
-constexpr int BAND = 32 * ROWS;
-constexpr int TB_BAND = BAND / 2;   // checkpoint spacing
+constexpr int TB_BAND = 256;        // checkpoint spacing
 constexpr int WARPS = 4;
 constexpr uint32_t JUNK_S = 0x80808080u;   // S + o = -128 for every residue: rows past a pair's end
 // LOCAL: a lane's state at a block start (Ho, E of its rows, diag, and the H - o
 // and F it hands down)
-constexpr int SNAP_WORDS = 2 * ROWS + 3;
+constexpr int snap_words(int rows) { return 2 * rows + 3; }
 
 // LOCAL: a band's best cell value of one pair, and where to look for it:
 // the start (step) of the first block in which the band's running maximum
@@ -107,16 +105,34 @@ __device__ __forceinline__ int32_t half(uint32_t v, int x) { return x ? hi16(v ^
 // built for 4 blocks (128 registers) and for 2 (198: the steady-state body
 // scheduled with more registers ran 2% faster on the 64 long pairs), the
 // local form for 3 and 2; the blocks-per-SM choice picks the build.
-template <bool LOCAL, int MINB>
+//
+// ROWS: rows per lane.  16 (512-row bands, two checkpoint rows a band) hand
+// over less per cell; with 8 (256-row bands) a step takes little more than
+// half as long, and there are twice as many bands: where a call's bands leave
+// most of the chip's schedulers without a warp, its time is the longest pair's
+// chain of steps.
+template <bool LOCAL, bool SUM, int MINB, int ROWS>
 __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
     const uint8_t* __restrict__ qcodes, const uint8_t* __restrict__ tcodes,
     const int8_t* __restrict__ Sg, int A, int o, int e, int mode, uint32_t fe,
     const LongJob* __restrict__ jobs, const LongPair16* __restrict__ pjobs,
     const uint32_t* __restrict__ items, uint32_t n_items, uint32_t* __restrict__ counter,
     int2* __restrict__ bnd, uint32_t* __restrict__ prog, LongCand* __restrict__ cands,
-    int32_t* __restrict__ status, LongBest* __restrict__ lbest, uint32_t* __restrict__ lsnap) {
-  __shared__ uint32_t Sb[4];                 // row q of S + o as 4 bytes
+    int32_t* __restrict__ status, LongBest* __restrict__ lbest, uint32_t* __restrict__ lsnap,
+    int Kp) {
+  constexpr int BAND = 32 * ROWS;
+  constexpr int CKPTS = BAND / TB_BAND;      // checkpoint rows per band; the last is its bottom row
+  constexpr bool MID = CKPTS == 2;
+  constexpr int SNAP_WORDS = snap_words(ROWS);
+  static_assert(CKPTS == 1 || CKPTS == 2, "bands of 256 or 512 rows");
+  static_assert(!(LOCAL && SUM), "the summed form has no floor");
+  __shared__ uint32_t Sb[4];                 // row q of S + o (SUM: S + 2e + Kp) as 4 bytes
   __shared__ uint2 ring[WARPS][2][32];       // per warp: middle (lane 15) and bottom (lane 31) rows
+  // per warp: lane 0's input row of the block's 32 columns, and the residue
+  // selectors of the block's columns and of the 32 before them (by column mod
+  // 64): loads that no step's chain waits on, where shuffles would
+  __shared__ uint2 inbuf[WARPS][32];
+  __shared__ uint32_t selbuf[WARPS][64];
   // LOCAL: the warp's state at the current block's start (word-major)
   __shared__ uint32_t snap[LOCAL ? WARPS : 1][LOCAL ? SNAP_WORDS : 1][32];
   // per thread and half: the lane's candidate (score, i, j, has)
@@ -126,7 +142,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
     uint32_t w = 0;
     if ((int)threadIdx.x < A)
       for (int a = 0; a < A; ++a)
-        w |= (uint32_t)(uint8_t)(int8_t)(Sg[threadIdx.x * A + a] + o) << (8 * a);
+        w |= (uint32_t)(uint8_t)(int8_t)(Sg[threadIdx.x * A + a] + (SUM ? 2 * e + Kp : o)) << (8 * a);
     Sb[threadIdx.x] = w;
   }
   __syncthreads();
@@ -137,6 +153,10 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
   const bool t_end_free = sg && (fe & DSA_FREE_T_END);
   const uint32_t neg_o2 = pack2(-o, -o), neg_e2 = pack2(-e, -e);
   const uint32_t o2 = ((uint32_t)o << 16) | (uint32_t)o;
+  // SUM: values carry e (i + j), and a stored H is H - Kp
+  const uint32_t K2 = (uint32_t)Kp * 0x10001u, c2 = pack2(Kp + e - o, Kp + e - o);
+  const int32_t hs = SUM ? Kp : o;       // a stored H is H - hs
+  auto ge = [&](int32_t i, int32_t j) { return SUM ? e * (i + j) : 0; };
   bool timed_out = false;
 
   for (;;) {
@@ -162,30 +182,33 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
     const uint8_t* tB = tcodes + JB.t_start;
     // checkpoint rows written by this band: middle (row i0 + 256) and bottom
     // (row i0 + 512, the next band's input)
-    const bool midA = inA && mA > i0 + TB_BAND, midB = inB && mB > i0 + TB_BAND;
+    const bool midA = MID && inA && mA > i0 + TB_BAND, midB = MID && inB && mB > i0 + TB_BAND;
     const bool botA = inA && (int32_t)b < nbA - 1, botB = inB && (int32_t)b < nbB - 1;
-    int2* const ckA = bnd + JA.bnd_off + (uint64_t)(2 * b) * (uint32_t)nA;   // + nA: bottom row
-    int2* const ckB = bnd + JB.bnd_off + (uint64_t)(2 * b) * (uint32_t)nB;
-    const int2* const upA = (b > 0 && inA) ? bnd + JA.bnd_off + (uint64_t)(2 * b - 1) * (uint32_t)nA : nullptr;
-    const int2* const upB = (b > 0 && inB) ? bnd + JB.bnd_off + (uint64_t)(2 * b - 1) * (uint32_t)nB : nullptr;
+    int2* const ckA = bnd + JA.bnd_off + (uint64_t)(CKPTS * b) * (uint32_t)nA;
+    int2* const ckB = bnd + JB.bnd_off + (uint64_t)(CKPTS * b) * (uint32_t)nB;
+    int2* const cbA = ckA + (MID ? (uint32_t)nA : 0u);   // the bottom row
+    int2* const cbB = ckB + (MID ? (uint32_t)nB : 0u);
+    const int2* const upA = (b > 0 && inA) ? bnd + JA.bnd_off + (uint64_t)(CKPTS * b - 1) * (uint32_t)nA : nullptr;
+    const int2* const upB = (b > 0 && inB) ? bnd + JB.bnd_off + (uint64_t)(CKPTS * b - 1) * (uint32_t)nB : nullptr;
     uint32_t* const my_prog = prog + pj.prog_off + b;
     const uint32_t* const up_prog = prog + pj.prog_off + b - 1;
 
     // bases and the lane's rows at column 0
-    int32_t baseA = h_col0(mode, fe, i0 + 1, o, e), baseB = baseA;
+    int32_t baseA = h_col0(mode, fe, i0 + 1, o, e) + ge(i0 + 1, 0), baseB = baseA;
     uint32_t Ho[ROWS], E[ROWS], sA[ROWS], sB[ROWS];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
       const int32_t i = r0 + r + 1;
-      const int32_t hc = h_col0(mode, fe, i, o, e) - o - baseA;
+      const int32_t hc = h_col0(mode, fe, i, o, e) + ge(i, 0) - hs - baseA;
       Ho[r] = bias2(hc, hc);
-      E[r] = Ho[r];   // E(i, 0) = H(i, 0) - o leaves E(i, 1) unchanged
-      sA[r] = i <= mA ? Sb[qA[i - 1]] : JUNK_S;
-      sB[r] = i <= mB ? Sb[qB[i - 1]] : JUNK_S;
+      // E(i, 0) = H(i, 0) - o leaves E(i, 1) unchanged; SUM: E of column 1
+      E[r] = SUM ? add2(Ho[r], c2) : Ho[r];
+      sA[r] = i <= mA ? Sb[qA[i - 1]] : (SUM ? 0u : JUNK_S);
+      sB[r] = i <= mB ? Sb[qB[i - 1]] : (SUM ? 0u : JUNK_S);
     }
-    const int32_t hd = h_col0(mode, fe, r0, o, e) - o - baseA;
+    const int32_t hd = h_col0(mode, fe, r0, o, e) + ge(r0, 0) - hs - baseA;
     uint32_t diag = bias2(hd, hd);
-    uint32_t sendH = 0, sendF = 0, sendS = 0;
+    uint32_t sendH = 0, sendF = 0;
     const bool ownA = inA && r0 < mA && mA <= r0 + ROWS;   // the lane holds row mA
     const bool ownB = inB && r0 < mB && mB <= r0 + ROWS;
     auto cand_set = [&](int x, int32_t sc, int32_t i, int32_t j) {
@@ -236,7 +259,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
     auto fetch_in = [&](int32_t blk) -> uint2 {
       const int32_t jj = blk + lane + 1;
       // a column outside a half's pair gets the relative 0 (see the reset)
-      int32_t ha = o + baseA, fa = baseA, hb = o + baseB, fb = baseB;
+      const int32_t g = ge(i0, jj);
+      int32_t ha = hs + baseA - g, fa = baseA - g, hb = hs + baseB - g, fb = baseB - g;
       if (b == 0) {
         const int32_t h = h_row0(mode, fe, jj, o, e);
         if (inA && jj <= nA) { ha = h; fa = h - o; }
@@ -252,7 +276,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
           hb = x.x; fb = x.y;
         }
       }
-      return make_uint2(bias2(ha - o - baseA, hb - o - baseB), bias2(fa - baseA, fb - baseB));
+      return make_uint2(bias2(ha + g - hs - baseA, hb + g - hs - baseB), bias2(fa + g - baseA, fb + g - baseB));
     };
     // byte-permute selector of the column's two residues (bytes a_lo of the
     // low row table and 4 + a_hi of the high one, each sign-replicated)
@@ -273,16 +297,18 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
       const int32_t jb = f31 + 1 + lane;
       if (jb <= upto31) {
         const uint2 v = ring[wid][1][jb & 31];
+        const int32_t g = ge(i0 + BAND, jb);
         if (botA && jb <= nA)
-          ckA[(uint32_t)nA + jb - 1] = make_int2(half(v.x, 0) + o + baseA, half(v.y, 0) + baseA);
+          cbA[jb - 1] = make_int2(half(v.x, 0) + hs + baseA - g, half(v.y, 0) + baseA - g);
         if (botB && jb <= nB)
-          ckB[(uint32_t)nB + jb - 1] = make_int2(half(v.x, 1) + o + baseB, half(v.y, 1) + baseB);
+          cbB[jb - 1] = make_int2(half(v.x, 1) + hs + baseB - g, half(v.y, 1) + baseB - g);
       }
       const int32_t jm = f15 + 1 + lane;
-      if (jm <= upto15) {
+      if (MID && jm <= upto15) {
         const uint2 v = ring[wid][0][jm & 31];
-        if (midA && jm <= nA) ckA[jm - 1] = make_int2(half(v.x, 0) + o + baseA, half(v.y, 0) + baseA);
-        if (midB && jm <= nB) ckB[jm - 1] = make_int2(half(v.x, 1) + o + baseB, half(v.y, 1) + baseB);
+        const int32_t g = ge(i0 + TB_BAND, jm);
+        if (midA && jm <= nA) ckA[jm - 1] = make_int2(half(v.x, 0) + hs + baseA - g, half(v.y, 0) + baseA - g);
+        if (midB && jm <= nB) ckB[jm - 1] = make_int2(half(v.x, 1) + hs + baseB - g, half(v.y, 1) + baseB - g);
       }
       __threadfence();
       __syncwarp();
@@ -296,27 +322,32 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
     // tests, no result tracking).
     auto step = [&](int32_t s, int k, auto fast_c) {
       constexpr bool FAST = decltype(fast_c)::value;
-      const uint32_t inH = __shfl_sync(FULL, incur.x, k);
-      const uint32_t inF = __shfl_sync(FULL, incur.y, k);
-      const uint32_t inS = __shfl_sync(FULL, selcur, k);
+      const int32_t j = s - lane;
+      const uint2 in = inbuf[wid][k];
+      const uint32_t sel = selbuf[wid][j & 63];
       uint32_t Hup = __shfl_up_sync(FULL, sendH, 1);
       uint32_t Fup = __shfl_up_sync(FULL, sendF, 1);
-      uint32_t sel = __shfl_up_sync(FULL, sendS, 1);
-      Hup = lane == 0 ? inH : Hup;
-      Fup = lane == 0 ? inF : Fup;
-      sel = lane == 0 ? inS : sel;
-      sendS = sel;
-      const int32_t j = s - lane;
+      Hup = lane == 0 ? in.x : Hup;
+      Fup = lane == 0 ? in.y : Fup;
       if (FAST || (j >= 1 && j <= n)) {
         uint32_t d = diag;
         diag = Hup;
         // With H = max(t, F) and e <= o, the next row's F = max(F - e, H - o)
         // is max(F - e, t - o): the F recurrence takes one operation per
         // row, and H - o = max(F - o, t - o) is computed beside it.
-        uint32_t F = addmax2u(Fup, neg_e2, Hup);   // F of the lane's first row
+        // SUM: E and F of the next cells are one operation each from H
+        uint32_t F = SUM ? addmax2u(Hup, c2, Fup) : addmax2u(Fup, neg_e2, Hup);   // F of the lane's first row
         uint32_t cm = 0, hprev = 0;   // LOCAL: the column maximum of H - o
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
+          if (SUM) {
+            const uint32_t hk = max3_2u(d + prmt(sA[r], sB[r], sel), E[r], F) - K2;
+            d = Ho[r];
+            Ho[r] = hk;
+            E[r] = addmax2u(hk, c2, E[r]);
+            if (r + 1 < ROWS) F = addmax2u(hk, c2, F);
+            continue;
+          }
           E[r] = addmax2u(E[r], neg_e2, Ho[r]);
           const uint32_t t = addmax2u(d, prmt(sA[r], sB[r], sel), E[r]);
           d = Ho[r];
@@ -332,7 +363,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
         }
         sendH = Ho[ROWS - 1];
         sendF = F;
-        if (lane == 15 || lane == 31) ring[wid][lane >> 4][j & 31] = make_uint2(sendH, F);
+        if ((MID && lane == 15) || lane == 31) ring[wid][lane >> 4][j & 31] = make_uint2(sendH, F);
         if (LOCAL) {
           // a half past its window holds no real cell in this column
           if (!FAST) cm &= (j <= nA ? 0x0000FFFFu : 0u) | (j <= nB ? 0xFFFF0000u : 0u);
@@ -348,7 +379,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
 #pragma unroll
               for (int r = 0; r < ROWS; ++r) {
                 const int32_t i = r0 + r + 1;
-                const int32_t v = half(Ho[r], x) + o + base;
+                const int32_t v = half(Ho[r], x) + hs + base - ge(i, j);
                 if (i <= mx && (q_end_free || i == mx) && (!ch || v > cs)) {
                   cand_set(x, v, i, j);
                   cs = v;
@@ -360,7 +391,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
 #pragma unroll
               for (int r = 1; r < ROWS; ++r)
                 if (r == mx - r0 - 1) hm = half(Ho[r], x);
-              hm += o + base;
+              hm += hs + base - ge(mx, j);
               if (!c_h[x][tid] || hm > c_s[x][tid]) cand_set(x, hm, mx, j);
             }
           }
@@ -380,8 +411,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
         // move the base to lane 0's first row while lane 0 is on a real
         // column of the half
         const uint32_t v = __shfl_sync(FULL, Ho[0], 0);
-        const int32_t dA = (inA && s0 <= nA) ? half(v, 0) + o : 0;
-        const int32_t dB = (inB && s0 <= nB) ? half(v, 1) + o : 0;
+        const int32_t dA = (inA && s0 <= nA) ? half(v, 0) + hs : 0;
+        const int32_t dB = (inB && s0 <= nB) ? half(v, 1) + hs : 0;
         const uint32_t nd2 = pack2(-dA, -dB);
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
@@ -429,6 +460,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
         snap[wid][2 * ROWS + 2][lane] = sendF;
         bmax2 = 0;
       }
+      inbuf[wid][lane] = incur;
+      selbuf[wid][(s0 + 1 + lane) & 63] = selcur;
+      __syncwarp();
       // lanes' columns in this block: s0 + 1 - 31 .. s0 + 32
       const int32_t jlo = s0 - 30, jhi = s0 + 32;
       const bool evA = inA && (rowmA || (nA >= jlo && nA <= jhi));
@@ -464,6 +498,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
         }
       }
       // block consumed: rotate, fetch the block after the next
+      __syncwarp();
       incur = innxt;
       selcur = selnxt;
       innxt = fetch_in(s0 + 64);
@@ -506,12 +541,14 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
 // in step order is in the block's 32 steps, and a cell of the best at a
 // smaller column j is processed at most 31 steps after its column's first
 // step.  Candidates of all bands merge by (score desc, j asc, i asc).
+template <int ROWS>
 __global__ void __launch_bounds__(WARPS * 32) k_long_locate16(
     const uint8_t* __restrict__ qcodes, const uint8_t* __restrict__ tcodes,
     const int8_t* __restrict__ Sg, int A, int o, int e, const LongJob* __restrict__ jobs,
     const uint32_t* __restrict__ items, uint32_t n_items, const int2* __restrict__ bnd,
     const LongBest* __restrict__ lbest, const uint32_t* __restrict__ lsnap,
     LongCand* __restrict__ cands) {
+  constexpr int BAND = 32 * ROWS, CKPTS = BAND / TB_BAND, SNAP_WORDS = snap_words(ROWS);
   __shared__ uint32_t Sb[4];
   if (threadIdx.x < 4) {
     uint32_t w = 0;
@@ -561,7 +598,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_long_locate16(
     const uint32_t neg_o2 = pack2(-o, -o), neg_e2 = pack2(-e, -e);
     const uint32_t zh = -base - o >= -32768 ? (uint32_t)(-base - o + 32768) & 0xFFFFu : 0u;
     const uint32_t z2o = x ? (zh << 16) : zh;
-    const int2* up = b > 0 ? bnd + J.bnd_off + (uint64_t)(2 * b - 1) * (uint32_t)n : nullptr;
+    const int2* up = b > 0 ? bnd + J.bnd_off + (uint64_t)(CKPTS * b - 1) * (uint32_t)n : nullptr;
     int32_t fj = INT32_MAX, fi = INT32_MAX;   // the lane's first cell of the best
     const int32_t s_end = min(lb.s0 + 64, n + 31);
     for (int32_t s = lb.s0 + 1; s <= s_end; ++s) {
@@ -632,17 +669,36 @@ bool long16_range_ok(int o, int e, int smax, int smin) {
   return 608 * D + 2 * (int64_t)o + e + std::max(-smin, 0) + 64 < 32768;
 }
 
+// The summed form of global and semi-global pairs: bytes S + 2e + K >= 0, and
+// relative values that carry e (i + j).
+int long16_sum_K(int e, int smin) { return std::max(0, -(smin + 2 * e)); }
+bool long16_sum_ok(int o, int e, int smax, int smin) {
+  const int K = long16_sum_K(e, smin);
+  const int64_t D = (int64_t)o + std::max(smax, 0) + e;
+  return std::max(smax, 0) + 2 * e + K <= 127 &&
+         608 * D + 2 * (int64_t)o + e + std::max(-smin, 0) + 2 * K + 192 < 32768;
+}
+
 int launch_long_score16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int8_t* d_matrix,
-                        int A, int o, int e, int mode, uint32_t fe, const LongJob* d_jobs,
-                        uint32_t n_jobs, const LongPair16* d_pjobs, const uint32_t* d_items,
+                        int A, int o, int e, int smax, int smin, int mode, uint32_t fe,
+                        const LongJob* d_jobs, uint32_t n_jobs, const LongPair16* d_pjobs,
+                        const uint32_t* d_items,
                         uint32_t n_items, int2* d_bnd, uint32_t* d_prog, void* d_cands,
-                        Scores out, int blocks_per_sm, const uint32_t* d_litems,
+                        Scores out, int rows, int blocks_per_sm, const uint32_t* d_litems,
                         uint32_t n_litems, uint64_t n_slots) {
   if (n_items == 0) return DSA_OK;
   const bool local = mode == DSA_LOCAL;
   const bool two = blocks_per_sm > 0 && blocks_per_sm <= 2;
-  auto kern = local ? (two ? k_long_score16<true, 2> : k_long_score16<true, 3>)
-                    : (two ? k_long_score16<false, 2> : k_long_score16<false, 4>);
+  // The summed form where warps share a scheduler: fewer operations per cell,
+  // but three in a row on the chain over a column's rows against one, so calls
+  // of few bands, whose warps run alone, keep the other form.
+  const bool sum = !local && rows == 16 && long16_sum_ok(o, e, smax, smin);
+  const int K = sum ? long16_sum_K(e, smin) : 0;
+  auto kern = rows == 8 ? (local ? (two ? k_long_score16<true, false, 2, 8> : k_long_score16<true, false, 4, 8>)
+                                 : (two ? k_long_score16<false, false, 2, 8> : k_long_score16<false, false, 4, 8>))
+              : local   ? (two ? k_long_score16<true, false, 2, 16> : k_long_score16<true, false, 3, 16>)
+              : sum     ? (two ? k_long_score16<false, true, 2, 16> : k_long_score16<false, true, 4, 16>)
+                        : (two ? k_long_score16<false, false, 2, 16> : k_long_score16<false, false, 4, 16>);
   // every warp must be resident at once (bands wait on their predecessors)
   int per_sm = 0;
   DSA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WARPS * 32, 0));
@@ -653,7 +709,7 @@ int launch_long_score16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const 
   void* pb = nullptr;
   void* ps = nullptr;
   const size_t b_bytes = (size_t)n_slots * sizeof(LongBest);
-  const size_t s_bytes = (size_t)n_slots * SNAP_WORDS * 32 * sizeof(uint32_t);
+  const size_t s_bytes = (size_t)n_slots * snap_words(rows) * 32 * sizeof(uint32_t);
   if (local) {
     DSA_TRY(ctx->alloc(&pb, b_bytes));
     DSA_TRY(ctx->alloc(&ps, s_bytes));
@@ -664,11 +720,12 @@ int launch_long_score16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const 
                                               d_jobs, d_pjobs, d_items, n_items, counter, d_bnd,
                                               d_prog, static_cast<LongCand*>(d_cands),
                                               ctx->d_status, static_cast<LongBest*>(pb),
-                                              static_cast<uint32_t*>(ps));
+                                              static_cast<uint32_t*>(ps), K);
   cudaError_t err = cudaGetLastError();
   ++ctx->launches;
   if (err == cudaSuccess && local && n_litems) {
-    k_long_locate16<<<(n_litems + WARPS - 1) / WARPS, WARPS * 32, 0, ctx->stream>>>(
+    auto locate = rows == 8 ? k_long_locate16<8> : k_long_locate16<16>;
+    locate<<<(n_litems + WARPS - 1) / WARPS, WARPS * 32, 0, ctx->stream>>>(
         qs->d_codes, db->d_codes, d_matrix, A, o, e, d_jobs, d_litems, n_litems, d_bnd,
         static_cast<const LongBest*>(pb), static_cast<const uint32_t*>(ps),
         static_cast<LongCand*>(d_cands));
@@ -683,7 +740,7 @@ int launch_long_score16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const 
     set_error("k_long_score16: %s", cudaGetErrorString(err));
     return DSA_ERR_CUDA;
   }
-  return launch_long_reduce(ctx, d_jobs, n_jobs, d_cands, mode, fe, o, e, out);
+  return launch_long_reduce(ctx, d_jobs, n_jobs, d_cands, 32 * rows, mode, fe, o, e, out);
 }
 
 }  // namespace dsa

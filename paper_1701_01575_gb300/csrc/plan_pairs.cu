@@ -23,6 +23,16 @@ namespace dsa {
 // semi-global 1,000 pairs 0.15 / 1.12, 60,000 1.28 / 1.63, 120,000 2.52 /
 // 2.57, 200,000 4.17 / 3.97; local 60,000 1.64 / 1.79, 120,000 3.25 / 2.92.
 constexpr uint64_t WAVE_MAX_SHORT_PAIRS = 100000;
+// Packed long pairs: 512-row bands (of two pairs each) per SM up to which a
+// call takes 256-row bands, and up to which one block per SM.  Score pass of
+// pairs of 10,000-60,000 (100,000), 512-row bands at 2 blocks per SM against
+// 256-row bands at 1 / 2 blocks (ms), by bands per SM:
+//   1.2: global 14.0, 10.8 / 10.6; local 12.6, 11.9 / 10.3
+//   3.6: global 15.2, 12.0 / 14.0; local 13.7, 12.4 / 14.9
+//   5.7: global 17.4, 16.5 / 14.8; local 21.2, 17.8 / 15.3
+//   8.0: global 29.5, 35.2 / 25.1; local 35.5, 38.6 / 27.5
+//   16:  global 33.4, 58.8 / 44.1; local 42.3, 66.2 / 49.2
+constexpr uint64_t LONG_SHORT_BANDS = 10, LONG_ONE_BLOCK = 4;
 
 int PairPass::need_hp(dsa_ctx* ctx) {
   if (hp_ready) return DSA_OK;
@@ -98,7 +108,7 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
   std::vector<uint64_t> p16;   // pairs for the packed int16 kernel
   uint64_t scr = 0, cells = 0, lcells = 0, p16cells = 0;
   uint64_t bnd = 0, prog = 0, cand = 0;
-  const int band = long_band_rows(), ckpt = long_ckpt_rows();
+  const int ckpt = long_ckpt_rows();
   // every pair packed: the device planner lays out the jobs (the wavefront
   // form's pairs are always planned on the device)
   const bool wave = pp.plan.wave;
@@ -146,6 +156,22 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
         if (cls[k] == C_P16) p16[pos++] = k;
     });
   }
+  // Long pairs: the packed form takes two pairs per warp (sorted neighbours by
+  // query and window length) when the alphabet, the byte tables and the range
+  // bound allow it; DSA_LONG_INT32=1 keeps every pair on the int32 kernel.
+  const char* force32 = getenv("DSA_LONG_INT32");
+  const bool l16 = A <= 4 && s_plus_o_fits_int8(matrix, A, o) &&
+                   long16_range_ok(o, e, v.smax, v.smin) && !(force32 && atoi(force32));
+  // rows of a score band: 512, or 256 for packed calls of few bands, whose time
+  // is the longest pair's chain of steps
+  int band = long_band_rows();
+  uint64_t bands = 0;   // 512-row bands
+  if (l16) {
+    for (uint64_t k = 0; k < cls.size(); ++k)
+      if (cls[k] == C_LONG) bands += (qs->h_len[pp.hp[k].query_id] + band - 1) / band;
+    if (bands / 2 <= LONG_SHORT_BANDS * (uint64_t)ctx->sm_count) band = 256;
+    if (const char* rows_env = getenv("DSA_LONG_ROWS")) band = atoi(rows_env) == 8 ? 256 : long_band_rows();
+  }
   for (uint64_t k = 0; k < cls.size(); ++k) {
     if (cls[k] == C_P16) continue;
     const dsa_pair& p = pp.hp[k];
@@ -168,12 +194,6 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
   res->cells = cells;
   res->phase_cells[PH_INT32] = cells;
   if (!ljobs.empty()) {
-    // The packed form takes two pairs per warp (sorted neighbours by query
-    // and window length) when the alphabet, the byte tables and the range
-    // bound allow it; DSA_LONG_INT32=1 keeps every pair on the int32 kernel.
-    const char* force32 = getenv("DSA_LONG_INT32");
-    const bool l16 = A <= 4 && s_plus_o_fits_int8(matrix, A, o) &&
-                     long16_range_ok(o, e, v.smax, v.smin) && !(force32 && atoi(force32));
     std::vector<LongPair16> units;
     std::vector<std::pair<uint32_t, uint32_t>> mn;
     if (l16) {
@@ -230,10 +250,10 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
         return DSA_ERR_CUDA;
       }
       if (l16)
-        return launch_long_score16(ctx, db, qs, d_mat, A, o, e, mode, fe, d_ljobs.as<LongJob>(),
+        return launch_long_score16(ctx, db, qs, d_mat, A, o, e, v.smax, v.smin, mode, fe, d_ljobs.as<LongJob>(),
                                    (uint32_t)ljobs.size(), d_units.as<LongPair16>(),
                                    d_items.as<uint32_t>(), (uint32_t)(items.size() / 2),
-                                   res->d_bnd, d_prog.as<uint32_t>(), d_cands.p, sc, bps,
+                                   res->d_bnd, d_prog.as<uint32_t>(), d_cands.p, sc, band / 32, bps,
                                    d_litems.as<uint32_t>(), (uint32_t)(litems.size() / 2), cand);
       return launch_long_score(ctx, db, qs, d_mat, A, o, e, mode, fe,
                                s_plus_o_fits_int8(matrix, A, o), d_ljobs.as<LongJob>(),
@@ -248,11 +268,14 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
     // it, else the autotuner times both on the first call of a shape
     // (kernel, mode, and log2 bins of the pair count, the longest query and
     // the longest window) and keeps the faster (a switch needs 3%).
-    int bps = 4;
+    int bps = l16 ? 2 : 4;
     const char* bps_env = getenv("DSA_LONG_BLOCKS");
     const char* tune_env = getenv("DSA_AUTOTUNE");
     if (bps_env) {
       bps = std::min(4, std::max(1, atoi(bps_env)));
+    } else if (band == 256 && bands / 2 <= LONG_ONE_BLOCK * (uint64_t)ctx->sm_count &&
+               !(tune_env && std::string(tune_env) == "retune")) {
+      bps = 1;   // a warp per scheduler holds them all, or nearly
     } else if (ctx->tune && !(tune_env && std::string(tune_env) == "off")) {
       uint32_t mmax = 0, nmax = 0;
       for (const LongJob& lj : ljobs) {
@@ -260,7 +283,7 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
         nmax = std::max(nmax, (uint32_t)lj.n);
       }
       char k[160];
-      snprintf(k, sizeof k, "|long|%s|%s|p%d|m%d|n%d|bps", l16 ? "p16" : "i32",
+      snprintf(k, sizeof k, "|long|%s|%s|p%d|m%d|n%d|bps", l16 ? (band == 256 ? "p16r8" : "p16r16") : "i32",
                mode == DSA_LOCAL ? "local" : (mode == DSA_GLOBAL ? "global" : "semi"),
                tuner_bin(ljobs.size()), tuner_bin(mmax), tuner_bin(nmax));
       const std::string key = tuner_shape_prefix(ctx) + k;

@@ -303,3 +303,23 @@ def test_packed_traceback_fill_matches_int32_fill(ctx, mode, fe, case, monkeypat
     for f in ("score", "q_end", "t_end", "q_begin", "t_begin", "cigar_len"):
         assert np.array_equal(h16[f], h32[f]), f
     assert np.array_equal(r16.cigar(), r32.cigar())
+
+
+@pytest.mark.parametrize("rows,blocks", [("8", "1"), ("8", "4"), ("16", "1")])
+@pytest.mark.parametrize("mode,fe", MODES[:4])
+def test_band_heights_match_oracle_with_traceback(ctx, rows, blocks, mode, fe, monkeypatch):
+    """256-row bands (8 rows a lane, one checkpoint row a band) and 512-row
+    bands (16 rows, two), at every number of blocks per SM."""
+    monkeypatch.setenv("DSA_LONG_ROWS", rows)
+    monkeypatch.setenv("DSA_LONG_BLOCKS", blocks)
+    rng = np.random.default_rng(2900 + 16 * mode + fe)
+    qs, db, pairs = _ragged_set(rng, mode)
+    S = W.dna_matrix(2, -3)
+    r = _run(ctx, qs, db, pairs, S, 5, 2, mode, fe)
+    h = r.hits()
+    want = oracle.score_pairs(qs.codes, qs.offsets, db.codes, db.offsets, pairs["query_id"],
+                              pairs["target_id"], S, 5, 2, mode, fe, pair_toff=pairs["t_offset"],
+                              pair_tlen=pairs["t_len"])
+    assert_same((h["score"], h["q_end"], h["t_end"]), want, f"rows={rows} mode={mode} fe={fe}")
+    assert r.phase_cells()["intra16"] > 0
+    check_traceback(h, r.cigar(), qs, db, S, 5, 2, mode, fe)
