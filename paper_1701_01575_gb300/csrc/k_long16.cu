@@ -252,42 +252,40 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
         timed_out = true;
       }
     };
-    // lane 0's input row for columns blk+1 .. blk+32 (lane k: column blk+k+1),
-    // (H - o, F) of the row above per half, relative to the current base
-    // (the pending blocks move with the base): the band above, or row 0
-    // (whose F is taken as H - o, so that row 1's F is H(0, j) - o)
-    auto fetch_in = [&](int32_t blk) -> uint2 {
+    // lane 0's input row and the residues of columns blk+1 .. blk+32 (lane k:
+    // column blk+k+1), as loaded: nothing is computed from them until their
+    // block starts, so the loads' latency passes behind the block before
+    struct Ahead { int2 a, b; uint32_t ra, rb; };
+    auto fetch = [&](int32_t blk) -> Ahead {
       const int32_t jj = blk + lane + 1;
-      // a column outside a half's pair gets the relative 0 (see the reset)
-      const int32_t g = ge(i0, jj);
-      int32_t ha = hs + baseA - g, fa = baseA - g, hb = hs + baseB - g, fb = baseB - g;
-      if (b == 0) {
-        const int32_t h = h_row0(mode, fe, jj, o, e);
-        if (inA && jj <= nA) { ha = h; fa = h - o; }
-        if (inB && jj <= nB) { hb = h; fb = h - o; }
-      } else {
-        if (blk < n) wait_for((uint32_t)min(blk + 32, n));
-        if (upA && jj <= nA) {
-          const int2 x = upA[jj - 1];
-          ha = x.x; fa = x.y;
-        }
-        if (upB && jj <= nB) {
-          const int2 x = upB[jj - 1];
-          hb = x.x; fb = x.y;
-        }
-      }
-      return make_uint2(bias2(ha + g - hs - baseA, hb + g - hs - baseB), bias2(fa + g - baseA, fb + g - baseB));
+      Ahead x;
+      x.a = x.b = make_int2(0, 0);
+      if (b > 0 && blk < n) wait_for((uint32_t)min(blk + 32, n));
+      if (upA && jj <= nA) x.a = upA[jj - 1];
+      if (upB && jj <= nB) x.b = upB[jj - 1];
+      x.ra = jj <= nA ? tA[jj - 1] : 0u;
+      x.rb = jj <= nB ? tB[jj - 1] : 0u;
+      return x;
+    };
+    // (H - o, F) of the row above per half, relative to the current base: the
+    // band above, or row 0 (whose F is taken as H - o, so that row 1's F is
+    // H(0, j) - o); a column outside a half's pair gets the relative 0 (see
+    // the reset)
+    auto input = [&](const Ahead& x, int32_t blk) -> uint2 {
+      const int32_t jj = blk + lane + 1, g = ge(i0, jj);
+      const int32_t h = h_row0(mode, fe, jj, o, e);
+      const int32_t ha = b == 0 ? h : x.a.x, fa = b == 0 ? h - o : x.a.y;
+      const int32_t hb = b == 0 ? h : x.b.x, fb = b == 0 ? h - o : x.b.y;
+      const bool okA = inA && jj <= nA, okB = inB && jj <= nB;
+      return make_uint2(bias2(okA ? ha + g - hs - baseA : 0, okB ? hb + g - hs - baseB : 0),
+                        bias2(okA ? fa + g - baseA : 0, okB ? fb + g - baseB : 0));
     };
     // byte-permute selector of the column's two residues (bytes a_lo of the
     // low row table and 4 + a_hi of the high one, each sign-replicated)
-    auto fetch_sel = [&](int32_t blk) -> uint32_t {
-      const int32_t jj = blk + lane + 1;
-      const uint32_t aa = jj <= nA ? tA[jj - 1] : 0u;
-      const uint32_t ab = jj <= nB ? tB[jj - 1] : 0u;
-      return (aa * 0x11u + 0x80u) | ((ab * 0x11u + 0xC4u) << 8);
+    auto selector = [&](const Ahead& x) -> uint32_t {
+      return (x.ra * 0x11u + 0x80u) | ((x.rb * 0x11u + 0xC4u) << 8);
     };
-    uint2 incur = fetch_in(0), innxt = fetch_in(32);
-    uint32_t selcur = fetch_sel(0), selnxt = fetch_sel(32);
+    Ahead cur = fetch(0), nxt = fetch(32);
 
     // checkpoint ring: columns (f31, ..] of lane 31 and (f15, ..] of lane 15
     // are pending; flushed with the base they were computed under
@@ -310,11 +308,15 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
         if (midA && jm <= nA) ckA[jm - 1] = make_int2(half(v.x, 0) + hs + baseA - g, half(v.y, 0) + baseA - g);
         if (midB && jm <= nB) ckB[jm - 1] = make_int2(half(v.x, 1) + hs + baseB - g, half(v.y, 1) + baseB - g);
       }
-      __threadfence();
       __syncwarp();
       f31 = upto31;
       f15 = upto15;
-      if (lane == 0 && (botA || botB)) st_release_u32(my_prog, (uint32_t)upto31);
+    };
+    // told to the band below: the release orders every lane's stores before it
+    // (the barrier after them makes them precede lane 0's), and waits for them,
+    // so it comes after the block's other preparations
+    auto publish = [&]() {
+      if (lane == 0 && (botA || botB)) st_release_u32(my_prog, (uint32_t)f31);
     };
 
     // One step: column j = s - lane of the lane's rows.  FAST: every lane
@@ -422,8 +424,6 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
         diag = add2(diag, nd2);
         sendH = add2(sendH, nd2);
         sendF = add2(sendF, nd2);
-        incur = make_uint2(add2(incur.x, nd2), add2(incur.y, nd2));
-        innxt = make_uint2(add2(innxt.x, nd2), add2(innxt.y, nd2));
         baseA += dA;
         baseB += dB;
         // A half whose pair has no cell in the lane's current column (no
@@ -460,8 +460,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
         snap[wid][2 * ROWS + 2][lane] = sendF;
         bmax2 = 0;
       }
-      inbuf[wid][lane] = incur;
-      selbuf[wid][(s0 + 1 + lane) & 63] = selcur;
+      inbuf[wid][lane] = input(cur, s0);
+      selbuf[wid][(s0 + 1 + lane) & 63] = selector(cur);
+      if (s0 > 0) publish();
       __syncwarp();
       // lanes' columns in this block: s0 + 1 - 31 .. s0 + 32
       const int32_t jlo = s0 - 30, jhi = s0 + 32;
@@ -499,12 +500,11 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
       }
       // block consumed: rotate, fetch the block after the next
       __syncwarp();
-      incur = innxt;
-      selcur = selnxt;
-      innxt = fetch_in(s0 + 64);
-      selnxt = fetch_sel(s0 + 64);
+      cur = nxt;
+      nxt = fetch(s0 + 64);
     }
     flush(n, n);
+    publish();
     if (LOCAL) {
       if (lane == 0) {
         if (inA) lbest[JA.cand_off + b] = LongBest{bestA, bs0A, bbaseA, 0};

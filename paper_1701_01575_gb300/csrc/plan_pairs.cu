@@ -23,16 +23,18 @@ namespace dsa {
 // semi-global 1,000 pairs 0.15 / 1.12, 60,000 1.28 / 1.63, 120,000 2.52 /
 // 2.57, 200,000 4.17 / 3.97; local 60,000 1.64 / 1.79, 120,000 3.25 / 2.92.
 constexpr uint64_t WAVE_MAX_SHORT_PAIRS = 100000;
-// Packed long pairs: 512-row bands (of two pairs each) per SM up to which a
-// call takes 256-row bands, and up to which one block per SM.  Score pass of
-// pairs of 10,000-60,000 (100,000), 512-row bands at 2 blocks per SM against
-// 256-row bands at 1 / 2 blocks (ms), by bands per SM:
-//   1.2: global 14.0, 10.8 / 10.6; local 12.6, 11.9 / 10.3
-//   3.6: global 15.2, 12.0 / 14.0; local 13.7, 12.4 / 14.9
-//   5.7: global 17.4, 16.5 / 14.8; local 21.2, 17.8 / 15.3
-//   8.0: global 29.5, 35.2 / 25.1; local 35.5, 38.6 / 27.5
-//   16:  global 33.4, 58.8 / 44.1; local 42.3, 66.2 / 49.2
-constexpr uint64_t LONG_SHORT_BANDS = 10, LONG_ONE_BLOCK = 4;
+// Packed long pairs by 512-row bands (of two pairs each) per SM: up to FEW a
+// call takes 256-row bands and one block per SM; up to MANY global and
+// semi-global pairs keep the short bands (at two blocks), and local ones,
+// whose steps do more and share a scheduler worse, take 512-row bands at one
+// block.  Score pass of pairs of 10,000-60,000 (100,000) (ms):
+//   bands  global 512x1 512x2 256x1 256x2  local 512x1 512x2 256x1 256x2
+//   1.2          13.2  13.1  11.2  10.0         11.7  11.7   9.6   9.6
+//   3.6          14.3  14.4  11.1  13.6         13.5  13.8  12.6  17.2
+//   5.7          14.9  16.7  15.0  13.4         13.0  21.5  16.1  16.2
+//   8.0          26.2  27.9  31.1  24.5         23.8  36.0  35.4  27.9
+//   16           47.9  30.8  52.9  39.2         43.6  41.4  59.2  44.9
+constexpr uint64_t LONG_FEW_BANDS = 4, LONG_MANY_BANDS = 9;
 
 int PairPass::need_hp(dsa_ctx* ctx) {
   if (hp_ready) return DSA_OK;
@@ -169,7 +171,8 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
   if (l16) {
     for (uint64_t k = 0; k < cls.size(); ++k)
       if (cls[k] == C_LONG) bands += (qs->h_len[pp.hp[k].query_id] + band - 1) / band;
-    if (bands / 2 <= LONG_SHORT_BANDS * (uint64_t)ctx->sm_count) band = 256;
+    const uint64_t most = mode == DSA_LOCAL ? LONG_FEW_BANDS : LONG_MANY_BANDS;
+    if (bands / 2 <= most * (uint64_t)ctx->sm_count) band = 256;
     if (const char* rows_env = getenv("DSA_LONG_ROWS")) band = atoi(rows_env) == 8 ? 256 : long_band_rows();
   }
   for (uint64_t k = 0; k < cls.size(); ++k) {
@@ -273,9 +276,10 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
     const char* tune_env = getenv("DSA_AUTOTUNE");
     if (bps_env) {
       bps = std::min(4, std::max(1, atoi(bps_env)));
-    } else if (band == 256 && bands / 2 <= LONG_ONE_BLOCK * (uint64_t)ctx->sm_count &&
-               !(tune_env && std::string(tune_env) == "retune")) {
-      bps = 1;   // a warp per scheduler holds them all, or nearly
+    } else if (l16 && !(tune_env && std::string(tune_env) == "retune") &&
+               bands / 2 <= (mode == DSA_LOCAL ? LONG_MANY_BANDS : LONG_FEW_BANDS) *
+                                (uint64_t)ctx->sm_count) {
+      bps = 1;
     } else if (ctx->tune && !(tune_env && std::string(tune_env) == "off")) {
       uint32_t mmax = 0, nmax = 0;
       for (const LongJob& lj : ljobs) {
