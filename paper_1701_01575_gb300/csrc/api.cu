@@ -409,8 +409,9 @@ int align_impl(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const dsa_pair*
   pp.flags = flags;
   pp.hp_ready = all;
   if (!all) {
-    const bool wave = pairs_take_wave(matrix, A, mode, o, e, v, n_pairs, local16, packed_ok);
-    const PairPlanParams P{qs->n, db->n, w16, o, e, local16, packed_ok, wave, v.smax, v.smin};
+    const bool wave = pairs_take_wave(mode, o, e, v, n_pairs, local16, packed_ok);
+    const PairPlanParams P{qs->n, db->n, w16, o, e, local16, packed_ok, wave, v.smax, v.smin, pair_wave_wide(A),
+                           n_pairs >= 32768};
     DSA_TRY(pairs_classify(ctx, db, qs, P, pp));
   }
   // int32 range: (m + n) * max|value step| must stay far from 2^31

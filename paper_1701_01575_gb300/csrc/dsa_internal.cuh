@@ -574,15 +574,18 @@ int pairs16_wide_rows();
 // Explicit pairs as wavefronts of small lane groups (k_pairwave.cu): class of a
 // pair by its query length (ascending cost; group size and rows per block),
 // and one launch over pairs sorted by (class, window length).
-constexpr int WAVE_CLASSES = 11;
-constexpr int WAVE_NONE = 15;      // sort class of pairs that take another path
-__host__ __device__ inline int pair_wave_class(uint64_t m) {
-  if (m <= 128) return m <= 64 ? 0 : m <= 96 ? 1 : 2;
-  if (m <= 256) return m <= 192 ? 3 : 4;
-  if (m <= 512) return m <= 384 ? 5 : 6;
-  if (m <= 1024) return m <= 768 ? 7 : 8;
+constexpr int WAVE_CLASSES = 16;
+constexpr int WAVE_NONE = 31;      // sort class of pairs that take another path
+// wide: an alphabet small enough for blocks of 20 rows; dense: pairs enough to
+// give the shortest two lanes each
+__host__ __device__ inline int pair_wave_class(uint64_t m, bool wide, bool dense) {
+  if (dense && m <= 80 && (wide || m <= 64)) return m <= 64 ? 1 : 2;
+  if (m <= 160 && (wide || m <= 128)) return m <= 64 ? 0 : m <= 96 ? 3 : m <= 128 ? 4 : 5;
+  if (m <= 320 && (wide || m <= 256)) return m <= 192 ? 6 : m <= 256 ? 7 : 8;
+  if (m <= 640 && (wide || m <= 512)) return m <= 384 ? 9 : m <= 512 ? 10 : 11;
+  if (m <= 1024) return m <= 768 ? 12 : 13;
   // several bands of 768 or 1,024 rows, whichever computes fewer rows
-  return (m + 767) / 768 * 12 < (m + 1023) / 1024 * 16 ? 9 : 10;
+  return (m + 767) / 768 * 12 < (m + 1023) / 1024 * 16 ? 14 : 15;
 }
 int launch_pair_wave(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int8_t* d_matrix, int A,
                      int o, int e, int mode, uint32_t fe, int smax, int smin, const dsa_pair* d_pairs,
@@ -597,6 +600,7 @@ struct PairPlanParams {
   bool packed_ok;       // the packed int16 form is allowed
   bool wave;            // packed pairs take the wavefront kernel
   int32_t smax, smin;
+  bool wide, dense;     // see pair_wave_class
 };
 struct PairPlanStats {   // field order is used by the kernels' atomics
   uint64_t cells;        // cells of all valid pairs
@@ -606,7 +610,7 @@ struct PairPlanStats {   // field order is used by the kernels' atomics
   uint64_t n_jobs;       // packed jobs (two pairs of equal query length each)
   uint32_t max_t_len;    // longest window of a valid pair
   uint32_t pad;
-  uint64_t cls[16];      // wave: packed pairs of each class
+  uint64_t cls[32];      // wave: packed pairs of each class
 };
 // A valid pair of m x n takes the packed kernel the call chose.
 bool pair_packed(const PairPlanParams& P, uint64_t m, uint64_t n);

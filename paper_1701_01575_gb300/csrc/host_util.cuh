@@ -89,8 +89,9 @@ struct PairPass {
   int need_hp(dsa_ctx* ctx);
 };
 // The call's short pairs take the wavefront kernel (k_pairwave.cu).
-bool pairs_take_wave(const int8_t* matrix, int A, int mode, int o, int e, const Validated& v,
-                     uint64_t n_pairs, bool local16, bool packed_ok);
+bool pairs_take_wave(int mode, int o, int e, const Validated& v, uint64_t n_pairs, bool local16,
+                     bool packed_ok);
+bool pair_wave_wide(int A);   // its blocks may have 20 rows
 // Upload (unless on the device), range-check and classify the pairs.
 int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairPlanParams& P,
                    PairPass& pp);

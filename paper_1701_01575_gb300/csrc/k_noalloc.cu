@@ -22,7 +22,7 @@
 // the strip's last row handed on through a boundary row), does those.
 //
 // Bound by the ALU pipe.  30,011 reads of 36-301 bp in 411 bp windows,
-// semi-global: 47.1 ms with one thread per pair for all, 1.19 ms now.
+// semi-global: 47.1 ms with one thread per pair for all, 1.15 ms now.
 #include "pairwave.cuh"
 
 #include <algorithm>
@@ -81,8 +81,8 @@ __global__ void __launch_bounds__(WAVE_WARPS * 32, MINB) k_noalloc_wave(const No
   const bool tables = pair_wave_tables_ok(LOCAL, N.o, N.e, smax, smin);
   uint8_t* const tab = smem;
   uint8_t* const prof = smem + pair_wave_table_bytes(N.A) + warp * pair_wave_warp_bytes(N.A, LOCAL);
-  uint16_t* const park = reinterpret_cast<uint16_t*>(prof + (N.A + 1) * WAVE_RESIDUE);
-  pair_wave_table<LOCAL>(W, tab, [&](int q, int a) { return (int)N.S[q * N.A + a]; });
+  uint2* const park = reinterpret_cast<uint2*>(prof + pair_wave_park_offset(N.A));
+  pair_wave_table<LOCAL ? WAVE_LOCAL : WAVE_GLOBAL>(W, tab, [&](int q, int a) { return (int)N.S[q * N.A + a]; });
   __syncthreads();
   const int G = N.G, per = 32 / G;
   const uint64_t gw = (uint64_t)blockIdx.x * WAVE_WARPS + warp;   // warp of the grid
@@ -153,11 +153,11 @@ __global__ void __launch_bounds__(WAVE_WARPS * 32, MINB) k_noalloc_wave(const No
       for (int w = 16; w > 0; w >>= 1) mmax = max(mmax, __shfl_xor_sync(FULL, mmax, w));
       int s, i, j;
       if (mmax <= 16 * G)
-        pair_wave_run<LOCAL, 8>(W, tab, prof, park, G, q, t, mm, nn, scr, s, i, j);
+        pair_wave_run<LOCAL ? WAVE_LOCAL : WAVE_GLOBAL, 8>(W, tab, prof, park, G, q, t, mm, nn, scr, s, i, j);
       else if (mmax <= 24 * G)
-        pair_wave_run<LOCAL, 12>(W, tab, prof, park, G, q, t, mm, nn, scr, s, i, j);
+        pair_wave_run<LOCAL ? WAVE_LOCAL : WAVE_GLOBAL, 12>(W, tab, prof, park, G, q, t, mm, nn, scr, s, i, j);
       else
-        pair_wave_run<LOCAL, 16>(W, tab, prof, park, G, q, t, mm, nn, scr, s, i, j);
+        pair_wave_run<LOCAL ? WAVE_LOCAL : WAVE_GLOBAL, 16>(W, tab, prof, park, G, q, t, mm, nn, scr, s, i, j);
       if (first && ok) {
         const bool wrapped = LOCAL && s > 32767 - max(0, smax);
         N.o_score[p] = s;

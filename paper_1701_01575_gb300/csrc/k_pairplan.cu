@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(PLAN_T) k_pair_classify(
         cells += c;
         max_t = max(max_t, p.t_len);
         if (takes_packed(P, m, p.t_len)) {
-          hm = P.wave ? (uint32_t)pair_wave_class(m) : (uint32_t)m;
+          hm = P.wave ? (uint32_t)pair_wave_class(m, P.wide, P.dense) : (uint32_t)m;
           key[k] = ((uint64_t)hm << 32) | p.t_len;
           idx[k] = (uint32_t)k;
           c16 += c;

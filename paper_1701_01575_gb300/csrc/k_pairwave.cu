@@ -9,11 +9,13 @@
 //
 // Bound by the ALU pipe and, at the end of a call, by the longest pair's
 // chain.  Measured against the forms it replaces (whole call): 20,000 protein
-// pairs of 50-1,500 residues, local, 133.6 -> 2.69 ms (one thread per two
+// pairs of 50-1,500 residues, local, 133.6 -> 2.59 ms (one thread per two
 // pairs, two table loads per packed cell); 15,001 such pairs, global, 241.5 ->
-// 1.78 ms (one thread per pair in int32, their range being past that form's
-// rule); 1,000 reads of 150 bp in 500 bp windows with traceback 1.85 -> 0.84 ms.
+// 1.58 ms (one thread per pair in int32, their range being past that form's
+// rule); 1,000 reads of 150 bp in 500 bp windows with traceback 1.85 -> 0.64 ms; 1,000,000 of
+// 150 and 250 bp, 27.6 -> 23.9 ms.
 #include "pairwave.cuh"
+#include "host_util.cuh"
 
 namespace dsa {
 namespace {
@@ -21,13 +23,14 @@ namespace {
 // The classes, ascending by the rows they hold in one band; the last two take
 // longer queries in several bands.
 struct WaveClass { int G, R; };
-__host__ __device__ constexpr WaveClass wave_class(int c) {
-  constexpr WaveClass C[WAVE_CLASSES] = {{4, 8},   {4, 12},  {4, 16},  {8, 12},  {8, 16}, {16, 12},
-                                         {16, 16}, {32, 12}, {32, 16}, {32, 12}, {32, 16}};
+constexpr WaveClass wave_class(int c) {
+  constexpr WaveClass C[WAVE_CLASSES] = {{4, 8},   {2, 16},  {2, 20},  {4, 12},  {4, 16}, {4, 20},
+                                         {8, 12},  {8, 16},  {8, 20},  {16, 12}, {16, 16}, {16, 20},
+                                         {32, 12}, {32, 16}, {32, 12}, {32, 16}};
   return C[c];
 }
 
-struct WaveRange { uint32_t first, n, item0; };   // sorted pairs and bundles of a class
+struct WaveRange { uint32_t first, n, item0; int G, R; };   // sorted pairs and bundles of a class
 struct WaveKernelArgs {
   WaveParams W;
   const dsa_pair* pairs;
@@ -47,15 +50,16 @@ struct WaveKernelArgs {
   Scores out;
 };
 
-template <bool LOCAL, int MINB>
+template <int FORM, bool WIDE, int MINB>
 __global__ void __launch_bounds__(WAVE_WARPS * 32, MINB) k_pair_wave(const WaveKernelArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr unsigned FULL = 0xFFFFFFFFu;
+  constexpr bool LOCAL = FORM != WAVE_GLOBAL;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint8_t* const tab = smem;
   uint8_t* const prof = smem + pair_wave_table_bytes(A.W.A) + warp * pair_wave_warp_bytes(A.W.A, LOCAL);
-  uint16_t* const park = reinterpret_cast<uint16_t*>(prof + (A.W.A + 1) * WAVE_RESIDUE);
-  pair_wave_table<LOCAL>(A.W, tab, [&](int q, int a) { return (int)A.S[q * A.W.A + a]; });
+  uint2* const park = reinterpret_cast<uint2*>(prof + pair_wave_park_offset(A.W.A));
+  pair_wave_table<FORM>(A.W, tab, [&](int q, int a) { return (int)A.S[q * A.W.A + a]; });
   __syncthreads();
   uint32_t* const scr = A.scratch + (uint64_t)(blockIdx.x * WAVE_WARPS + warp) * A.scratch_cols;
 
@@ -66,7 +70,7 @@ __global__ void __launch_bounds__(WAVE_WARPS * 32, MINB) k_pair_wave(const WaveK
     if (item >= A.n_items) break;
     int x = 0;
     while (x + 1 < WAVE_CLASSES && item >= A.cls[x + 1].item0) ++x;
-    const WaveClass C = wave_class(WAVE_CLASSES - 1 - x);
+    const WaveClass C{A.cls[x].G, A.cls[x].R};
     const uint32_t per = 32u / C.G;
     const uint32_t at = (item - A.cls[x].item0) * per + lane / C.G;   // from the longest window down
     const uint8_t *q = nullptr, *t = nullptr;
@@ -81,12 +85,14 @@ __global__ void __launch_bounds__(WAVE_WARPS * 32, MINB) k_pair_wave(const WaveK
       n = (int)p.t_len;
     }
     int s, i, j;
-    if (C.R == 16)
-      pair_wave_run<LOCAL, 16>(A.W, tab, prof, park, C.G, q, t, m, n, scr, s, i, j);
+    if (WIDE && C.R == 20)
+      pair_wave_run<FORM, WIDE ? 20 : 16>(A.W, tab, prof, park, C.G, q, t, m, n, scr, s, i, j);
+    else if (C.R == 16)
+      pair_wave_run<FORM, 16>(A.W, tab, prof, park, C.G, q, t, m, n, scr, s, i, j);
     else if (C.R == 12)
-      pair_wave_run<LOCAL, 12>(A.W, tab, prof, park, C.G, q, t, m, n, scr, s, i, j);
+      pair_wave_run<FORM, 12>(A.W, tab, prof, park, C.G, q, t, m, n, scr, s, i, j);
     else
-      pair_wave_run<LOCAL, 8>(A.W, tab, prof, park, C.G, q, t, m, n, scr, s, i, j);
+      pair_wave_run<FORM, 8>(A.W, tab, prof, park, C.G, q, t, m, n, scr, s, i, j);
     if (id != NONE && (lane & (C.G - 1)) == 0) {
       A.out.score[id] = s;
       A.out.q_end[id] = i - 1;
@@ -99,7 +105,8 @@ __global__ void __launch_bounds__(WAVE_WARPS * 32, MINB) k_pair_wave(const WaveK
 
 }  // namespace
 
-int pair_wave_group(int cls) { return wave_class(cls).G; }
+static int pair_wave_group(int cls) { return wave_class(cls).G; }
+bool pair_wave_wide(int A) { return A <= WAVE_WIDE_ALPHABET; }
 
 int launch_pair_wave(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int8_t* d_matrix, int A,
                      int o, int e, int mode, uint32_t fe, int smax, int smin, const dsa_pair* d_pairs,
@@ -107,7 +114,8 @@ int launch_pair_wave(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int
   const bool local = mode == DSA_LOCAL;
   WaveKernelArgs K{};
   const int k = pair_wave_K(o, e, smin);
-  K.W = {A, o, e, mode, fe, k, pair_wave_bias(o, e, k)};
+  const bool lsum = local && pair_wave_local_sum_ok(qs->max_len, max_n, o, e, smax, smin);
+  K.W = {A, o, e, mode, fe, k, lsum ? 512 + o + 64 * e : pair_wave_bias(o, e, k)};
   K.pairs = d_pairs;
   K.order = d_order;
   K.qcodes = qs->d_codes; K.qoff = qs->d_off; K.qlen = qs->d_len;
@@ -119,7 +127,7 @@ int launch_pair_wave(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int
   for (int x = 0; x < WAVE_CLASSES; ++x) {
     const int c = WAVE_CLASSES - 1 - x;
     const uint64_t per = 32 / pair_wave_group(c);
-    K.cls[x] = {(uint32_t)first[c], (uint32_t)class_n[c], (uint32_t)items};
+    K.cls[x] = {(uint32_t)first[c], (uint32_t)class_n[c], (uint32_t)items, wave_class(c).G, wave_class(c).R};
     items += (class_n[c] + per - 1) / per;
   }
   if (items == 0) return DSA_OK;
@@ -129,9 +137,12 @@ int launch_pair_wave(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int
   const size_t smem = pair_wave_table_bytes(A) + (size_t)WAVE_WARPS * pair_wave_warp_bytes(A, local);
   // small alphabets: registers bound the warps per SM (4 CTAs); larger ones:
   // the profiles do (2 CTAs of 4 x 28 KB for proteins)
-  const bool small = smem <= 50 * 1024;
-  auto kern = local ? (small ? k_pair_wave<true, 4> : k_pair_wave<true, 2>)
-                    : (small ? k_pair_wave<false, 4> : k_pair_wave<false, 2>);
+  auto kern = pair_wave_wide(A) ? (lsum    ? k_pair_wave<WAVE_LOCAL_SUM, true, 4>
+                                   : local ? k_pair_wave<WAVE_LOCAL, true, 4>
+                                           : k_pair_wave<WAVE_GLOBAL, true, 4>)
+                                : (lsum    ? k_pair_wave<WAVE_LOCAL_SUM, false, 2>
+                                   : local ? k_pair_wave<WAVE_LOCAL, false, 2>
+                                           : k_pair_wave<WAVE_GLOBAL, false, 2>);
   DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   DSA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WAVE_WARPS * 32, smem));

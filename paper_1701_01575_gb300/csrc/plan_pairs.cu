@@ -18,11 +18,6 @@
 
 namespace dsa {
 
-// Pairs of a byte-permute scoring (DNA) that still take the wavefront form.
-// Reads of 150 bp in 500 bp windows, wavefront against per-thread form (ms):
-// semi-global 1,000 pairs 0.15 / 1.12, 60,000 1.28 / 1.63, 120,000 2.52 /
-// 2.57, 200,000 4.17 / 3.97; local 60,000 1.64 / 1.79, 120,000 3.25 / 2.92.
-constexpr uint64_t WAVE_MAX_SHORT_PAIRS = 100000;
 // Packed long pairs by 512-row bands (of two pairs each) per SM: up to FEW a
 // call takes 256-row bands and one block per SM; up to MANY global and
 // semi-global pairs keep the short bands (at two blocks), and local ones,
@@ -51,19 +46,21 @@ int PairPass::need_hp(dsa_ctx* ctx) {
   return DSA_OK;
 }
 
-// Which packed kernel a call's short pairs take.  The wavefront form keeps 4
-// to 32 lanes on a pair, the other one thread on two pairs (equal lengths,
-// byte-permute scores), which needs hundreds of thousands of pairs to fill
-// the chip but then spends nothing on hand-overs between lanes.
-bool pairs_take_wave(const int8_t* matrix, int A, int mode, int o, int e, const Validated& v,
-                     uint64_t n_pairs, bool local16, bool packed_ok) {
+// Which packed kernel a call's short pairs take.  The wavefront form keeps 2 to
+// 32 lanes on a pair, the other one thread on two pairs.  Reads in windows,
+// wavefront against per-thread form (ms): 150 bp in 500, semi-global, 1,000
+// pairs 0.15 / 1.12, 40,000 0.60 / 1.55, 300,000 3.87 / 5.21, 1,000,000 12.8 /
+// 16.5; local 1,000,000 15.4 / 18.8; 75 bp in 200, semi-global, 1,000,000 2.75 /
+// 3.92; 101 bp in 300, local, 1,000,000 8.25 / 7.98 (a third of its rows are
+// padding), the only shape measured that loses.  So the per-thread form is
+// left with scorings past the byte tables.
+bool pairs_take_wave(int mode, int o, int e, const Validated& v, uint64_t n_pairs, bool local16,
+                     bool packed_ok) {
   if (!packed_ok || (mode == DSA_LOCAL && !local16) || n_pairs > UINT32_MAX) return false;
-  if (!pair_wave_tables_ok(mode == DSA_LOCAL, o, e, v.smax, v.smin)) return false;
-  if (A > 4 || !s_plus_o_fits_int8(matrix, A, o)) return true;
   // DSA_PAIRS_ROWS fixes a variant of the per-thread form, and re-tuning times it
   const char* tune = getenv("DSA_AUTOTUNE");
   if (getenv("DSA_PAIRS_ROWS") || (tune && std::string(tune) == "retune")) return false;
-  return n_pairs < WAVE_MAX_SHORT_PAIRS;
+  return pair_wave_tables_ok(mode == DSA_LOCAL, o, e, v.smax, v.smin);
 }
 
 int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairPlanParams& P,

@@ -105,6 +105,22 @@ def test_range_rule_and_rerun(ctx, mode, fe):
         assert r.stats()[1] == 0 and 0 < r.phase_cells()["int32"] < r.stats()[0]
 
 
+@pytest.mark.parametrize("mode,fe", [(dsa.LOCAL, 15), (dsa.GLOBAL, 15), (dsa.SEMIGLOBAL, 12)])
+@pytest.mark.parametrize("alphabet", ["dna", "protein"])
+def test_many_pairs_take_two_lanes_each(ctx, alphabet, mode, fe):
+    """Enough pairs for the densest classes (two lanes a pair)."""
+    rng = np.random.default_rng(3500 + mode + len(alphabet))
+    bg = np.full(4, 0.25) if alphabet == "dna" else W.protein_background()
+    S, o, e = (W.dna_matrix(1, -4), 6, 1) if alphabet == "dna" else (W.blosum62(), 11, 1)
+    qs = W._make_set(rng, rng.integers(1, 90, 400), bg)
+    db = W._make_set(rng, rng.integers(1, 60, 300), bg)
+    pairs = np.zeros(33_000, W.PAIR_DTYPE)
+    pairs["query_id"] = rng.integers(0, qs.n, len(pairs))
+    pairs["target_id"] = rng.integers(0, db.n, len(pairs))
+    pairs["t_len"] = db.lengths[pairs["target_id"]]
+    _check(ctx, qs, db, pairs, S, o, e, mode, fe, f"dense {alphabet} mode={mode}")
+
+
 @pytest.mark.parametrize("mode,fe", [(dsa.LOCAL, 15), (dsa.SEMIGLOBAL, 12)])
 def test_long_pairs_among_short_ones(ctx, mode, fe):
     """A call that also holds pairs of the band pipeline, on the device and on
