@@ -49,6 +49,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 namespace dsa {
@@ -568,10 +569,14 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   const bool local = mode == DSA_LOCAL;
   const uint32_t max_n = db->h_len[db->h_perm[0]];
   const int form = wave_form(local, qs->max_len, max_n, o, e, smax, smin);
-  auto kern = form == LOCAL_SUM    ? (rows == 16 ? k_wave<LOCAL_SUM, 16> : k_wave<LOCAL_SUM, 24>)
-              : form == LOCAL_WRAP ? (rows == 16 ? k_wave<LOCAL_WRAP, 16> : k_wave<LOCAL_WRAP, 24>)
-                                   : (rows == 16 ? k_wave<GLOBAL_SUM, 16> : k_wave<GLOBAL_SUM, 24>);
-  if (form < 0 || (rows != 16 && rows != 24)) {
+  auto pick = [&](auto f) {
+    constexpr int F = decltype(f)::value;
+    return rows == 8 ? k_wave<F, 8> : rows == 16 ? k_wave<F, 16> : k_wave<F, 24>;
+  };
+  auto kern = form == LOCAL_SUM    ? pick(std::integral_constant<int, LOCAL_SUM>{})
+              : form == LOCAL_WRAP ? pick(std::integral_constant<int, LOCAL_WRAP>{})
+                                   : pick(std::integral_constant<int, GLOBAL_SUM>{});
+  if (form < 0 || (rows != 8 && rows != 16 && rows != 24)) {
     set_error("no wavefront form for this search");
     return DSA_ERR_INVALID_ARG;
   }

@@ -170,13 +170,22 @@ Streams build_streams(const dsa_db* qs, const std::vector<uint32_t>& qorder, uin
 
 // Strip rows of the wavefront search: 24 spread a step's hand-over over more
 // rows, 16 pad short queries less.  Cost per query: strips times (rows of
-// about 11 cycles and a hand-over of about 45).
-int wave_rows(const dsa_db* qs) {
-  auto cost = [&](uint32_t R) {
+// about 11 cycles and a hand-over of about 45).  A search whose queries fill one
+// band (32 lanes) at 8 rows, and whose lanes fill the chip three times at most,
+// lasts about as long as its longest target, so it takes the shortest steps:
+// 128 residues against 2,000 targets 0.53 ms (16 rows 0.75, 24 rows 1.01),
+// against 12,000 0.91 (1.14, 1.56).  Past one band they lose, 300 residues 1.24
+// (0.86, 1.01), and with more lanes too, 16 queries against 2,000 1.48 (1.19,
+// 1.18).
+int wave_rows(const dsa_ctx* ctx, const dsa_db* qs, uint32_t n_targets) {
+  auto strips = [&](uint32_t R) {
     uint64_t c = 0;
-    for (uint32_t m : qs->h_len) c += (uint64_t)((m + R - 1) / R) * (R * 11 + 45);
+    for (uint32_t m : qs->h_len) c += (m + R - 1) / R;
     return c;
   };
+  auto cost = [&](uint32_t R) { return strips(R) * (R * 11 + 45); };
+  const uint64_t lanes = std::max<uint64_t>((qs->max_len + 7) / 8, (strips(8) + 1) / 2);
+  if (lanes <= 32 && lanes * n_targets <= 3ull * 512 * ctx->sm_count) return 8;
   return cost(16) < cost(24) ? 16 : 24;
 }
 
@@ -295,7 +304,7 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
     DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0));
   }
   if (wave) {
-    const int wr = wave_rows(qs);
+    const int wr = wave_rows(ctx, qs, n_long);
     // longer streams waste fewer lanes and balance the halves better, until the
     // longest target's pass over a unit would take half the launch: each of the
     // chip's lanes has total / lanes strip columns to compute, the longest

@@ -98,3 +98,19 @@ def test_modelled_threshold_matches_the_wavefronts(ctx, monkeypatch):
     monkeypatch.setenv("DSA_LONG_THRESHOLD", "0")
     b = ctx.align(ctx.load_set(db, 24), ctx.load_set(queries, 24), S, 11, 1)
     assert (a.hits() == b.hits()).all()
+
+
+@pytest.mark.parametrize("lengths", [[1], [8], [9], [255], [256], [256, 256], [1, 7, 8, 9, 15, 16, 17, 64, 65, 100],
+                                     [250, 3, 3, 120, 100, 31]])
+@pytest.mark.parametrize("mode,fe", [(dsa.LOCAL, 15), (dsa.GLOBAL, 15), (dsa.SEMIGLOBAL, 6)])
+def test_short_strips_of_small_searches(ctx, lengths, mode, fe, monkeypatch):
+    """Queries that fill one band at 8 rows at most."""
+    monkeypatch.setenv("DSA_LONG_THRESHOLD", "0")
+    rng = np.random.default_rng(5500 + sum(lengths) + mode)
+    bg = W.protein_background()
+    queries = W._make_set(rng, np.asarray(lengths), bg)
+    db = _db(rng, queries, bg, 700)
+    S = W.blosum62()
+    g = gpu_all(ctx, queries, db, S, 11, 1, mode=mode, fe=fe)
+    assert_same(g[:3], oracle_all(queries, db, S, 11, 1, mode, fe), f"{lengths} mode={mode}")
+    assert g[5].phase_cells()["inter16"] == 0
