@@ -287,11 +287,12 @@ constexpr uint32_t WAVE_LONG_TARGET = 2048;   // longer targets take up to 32 la
 int sum_bias(bool local, int o, int e, int smin);
 bool sum_fits(bool local, int64_t m, int64_t n, int o, int e, int smax, int smin);
 bool wave_takes(bool local, uint32_t max_m, uint32_t max_n, int o, int e, int smax, int smin);
+bool wave_dual_takes(bool local, uint32_t max_m, uint32_t max_n, int o, int e, int smax, int smin);
 int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, const dsa_db* qs,
                        const int8_t* d_matrix, const int8_t* d_pssm, int A, int mode, uint32_t fe, int o,
-                       int e, int smax, int smin, int rows, const std::vector<StripMeta>& meta,
+                       int e, int smax, int smin, int rows, bool dual, const std::vector<StripMeta>& meta,
                        const std::vector<uint32_t>& sbase, const std::vector<uint32_t>& ns,
-                       uint32_t n_targets, Scores out);
+                       uint32_t n_targets, uint64_t residues, Scores out);
 
 // Top-k per query over a dense [n_queries][n_targets] score matrix.
 int launch_topk(dsa_ctx* ctx, const Scores& s, uint32_t n_queries, uint32_t n_targets,

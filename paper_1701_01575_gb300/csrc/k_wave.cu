@@ -29,6 +29,15 @@
 //   are max(H - o + e, E) and max(H - o + e, F): three maxima and one sum.
 //   Launches whose scores or gaps could pass 16 bits stay on the kernels of
 //   k_intra.cu, so nothing is flagged here.
+// Two targets a lane (DUAL).  One query, or one much longer than the rest,
+// would leave one stream and so half of every register idle.  Such searches
+// follow one stream of all queries, and the halves hold neighbouring targets of
+// the length order.  Their columns hold different residues, so the profile is a
+// byte per (residue, row), lifted by K to 0..127: two loads give 16 rows of both
+// halves and one byte permute a packed cell joins them; K is taken off in the
+// same addition.  A step costs about 1.17 of the other form's.  One query
+// against 50,000 targets: of 700 residues, local, 4.7 -> 3.0 ms, of 2,000, 13.2
+// -> 9.1, global 11.1 -> 7.4; of 128 against 200,000 3.4 -> 2.2.
 // Lanes start one after another: before a target's first column they hold the
 // padding residue, under which a strip's column-0 state is a fixed point.
 //
@@ -42,8 +51,8 @@
 // Bound by the ALU pipe; 128 registers keep 16 warps per SM.  Measured (whole
 // score pass, before: the inter-sequence kernel with the longest targets on
 // the wavefronts of k_intra.cu): 7 queries of 90-1,100 against 50,011 targets,
-// global, 16.1 -> 8.8 ms (6,100 GCUPS); 5 of 60-700 against 60,000, local, 17.1
-// -> 7.4 ms; 32 of 64-5,000 against 100,000, local, 225.6 -> 225.3 ms.
+// global, 16.1 -> 7.5 ms (7,200 GCUPS); 5 of 60-700 against 60,000, local, 17.1
+// -> 5.9 ms; 32 of 64-5,000 against 100,000, local, 225.6 -> 225.3 ms.
 #include "dsa_internal.cuh"
 #include "dpx.cuh"
 
@@ -59,13 +68,14 @@ constexpr int NW = 8;              // warps per CTA
 constexpr int NT = NW * 32;
 constexpr int FEW_LANES = 8;       // lanes per target where targets abound
 constexpr int PLANE = 512;         // bytes of one row quad of 32 strips
+constexpr int MIN_WARPS = 2;       // busy warps per CTA of spread launches and longest targets
 enum Form { LOCAL_SUM = 0, LOCAL_WRAP = 1, GLOBAL_SUM = 2 };
 
 // Targets first .. first + count of the length order against one unit, `G`
-// lanes a target, CTA items of NW * 32 / G targets.
+// lanes a target (or two), CTA items of `warps` * 32 / G such groups.
 struct Segment {
   uint32_t unit, first, count, item0;
-  int32_t G;
+  int32_t G, warps;
 };
 
 struct WaveArgs {
@@ -73,14 +83,15 @@ struct WaveArgs {
   const uint64_t* toff;
   const uint32_t* tlen;
   const uint32_t* perm;            // length order -> target id
-  const uint32_t* prof;            // [strip][residue][R] packed
+  const uint32_t* prof;            // [strip][residue][R] packed (DUAL: bytes)
   const StripMeta* meta;
   const uint32_t* sbase;
   const uint32_t* nstrips;
   const uint32_t* qlen;
   int A, o, e, mode, bias, T;
+  int K;                           // DUAL: what the profile's bytes have too much
   uint32_t fe;
-  uint32_t pad_word;               // profile word of strips past a unit's end
+  uint32_t pad_word;               // profile word (DUAL: 4 bytes) of strips past a unit's end
   const Segment* segs;
   uint32_t n_segs, n_items;
   uint32_t* counter;
@@ -90,13 +101,15 @@ struct WaveArgs {
   uint32_t n_out_t;
 };
 
-template <int FORM, int R>
+template <int FORM, int R, bool DUAL>
 __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
+  static_assert(!DUAL || FORM != LOCAL_WRAP, "two targets a lane: summed forms");
   constexpr bool LOCAL = FORM != GLOBAL_SUM;
   constexpr bool SUM = FORM != LOCAL_WRAP;
   constexpr unsigned FULL = 0xFFFFFFFFu;
   constexpr uint32_t BIAS2 = 0x80008000u;
-  constexpr int RS = R / 4 * PLANE;   // profile bytes per residue
+  constexpr int RS = DUAL ? 32 * R : R / 4 * PLANE;   // profile bytes per residue
+  constexpr int MIN_SLOTS = DUAL ? 16 : 8;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ Segment s_seg;
   __shared__ uint32_t s_tile;
@@ -108,7 +121,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
   const int o = A.o, e = A.e;
   const uint32_t e2 = (uint32_t)e * 0x10001u, o2 = (uint32_t)o * 0x10001u;
   const uint32_t neg_e2 = pack2(-e, -e), c2 = pack2(e - o, e - o);
-  const uint32_t mo2 = pack2(-o, -o) ^ BIAS2;
+  const uint32_t mo2 = pack2(-o, -o) ^ BIAS2, K2 = (uint32_t)A.K * 0x10001u;
   const bool sg = A.mode == DSA_SEMIGLOBAL;
   const bool qb_free = sg && (A.fe & DSA_FREE_Q_BEGIN), qe_free = sg && (A.fe & DSA_FREE_Q_END);
   const bool tb_free = sg && (A.fe & DSA_FREE_T_BEGIN), te_free = sg && (A.fe & DSA_FREE_T_END);
@@ -137,23 +150,33 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
     if (s_tile == NONE) break;
     const int G = s_seg.G, k = lane & (G - 1);
     const uint32_t ns = A.nstrips[s_seg.unit], sb = A.sbase[s_seg.unit];
-    const uint32_t in_seg = s_tile * (NW * 32 / G) + warp * (32 / G) + lane / G;
-    const bool valid = in_seg < s_seg.count;
-    uint32_t id = 0;
-    int n = 0;
-    const uint8_t* t = A.tcodes;
+    const uint32_t in_seg = (s_tile * (s_seg.warps * 32 / G) + warp * (32 / G) + lane / G) * (DUAL ? 2 : 1);
+    // the halves' targets: the same, or (DUAL) neighbours, the longer one first
+    const bool valid = in_seg < s_seg.count && warp < s_seg.warps;
+    const bool valid2 = DUAL ? valid && in_seg + 1 < s_seg.count : valid;
+    uint32_t id = 0, id2 = 0;
+    int n = 0, n2 = 0;
+    const uint8_t *t = A.tcodes, *t2 = A.tcodes;
     if (valid) {
       id = A.perm[s_seg.first + in_seg];
       n = (int)A.tlen[id];
       t = A.tcodes + A.toff[id];
     }
-    int nmax = n, nmin = n;
+    if (!DUAL) {
+      id2 = id;
+      n2 = n;
+    } else if (valid2) {
+      id2 = A.perm[s_seg.first + in_seg + 1];
+      n2 = (int)A.tlen[id2];
+      t2 = A.tcodes + A.toff[id2];
+    }
+    int nmax = n, nmin = n2;
 #pragma unroll
     for (int w = 16; w > 0; w >>= 1) {
       nmax = max(nmax, __shfl_xor_sync(FULL, nmax, w));
       nmin = min(nmin, __shfl_xor_sync(FULL, nmin, w));
     }
-    const uint32_t sh = 8u * (uint32_t)((uintptr_t)(t - k) & 3);
+    const uint32_t sh = 8u * (uint32_t)((uintptr_t)(t - k) & 3), sh2 = 8u * (uint32_t)((uintptr_t)(t2 - k) & 3);
     uint2* const scr = scr_warp + (uint64_t)(lane / G) * nmax;
     const int steps = nmax + G - 1;
     const int nb = ((int)ns + G - 1) / G;
@@ -162,12 +185,22 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
       const uint32_t want = (sb + (uint32_t)(b * G)) * 64u + (uint32_t)G;
       if (held != want) {
         __syncthreads();
-        // slot x of 8 or more holds strip x mod G: 4 lanes a target read two copies
-        const int slots = max(G, 8), lg = 31 - __clz(slots);
-        const int total = slots * (A.A + 1) * (R / 4);
+        // slot x of 8 (DUAL: 16) or more holds strip x mod G: fewer lanes a target
+        // read copies
+        const int slots = max(G, MIN_SLOTS), lg = 31 - __clz(slots);
+        const int total = slots * (A.A + 1) * (DUAL ? R / 8 : R / 4);
         for (int x = tid; x < total; x += NT) {
           const int slot = x & (slots - 1), rest = x >> lg;
           const uint32_t strip = (uint32_t)(b * G + (slot & (G - 1)));
+          if (DUAL) {   // 8 rows, into a plane of 16 or (the last 8 rows) of 8 bytes a slot
+            constexpr int C = R / 8;
+            const int a = rest / C, c = rest - a * C;
+            uint2 v = make_uint2(A.pad_word, A.pad_word);
+            if (strip < ns)
+              v = __ldg(reinterpret_cast<const uint2*>(A.prof + (uint64_t)(sb + strip) * (A.A + 1) * (R / 4)) + rest);
+            *reinterpret_cast<uint2*>(smem + a * RS + (R != 8 && c < 2 ? slot * 16 + c * 8 : (R != 8 ? PLANE : 0) + slot * 8)) = v;
+            continue;
+          }
           uint4 v = make_uint4(A.pad_word, A.pad_word, A.pad_word, A.pad_word);
           if (strip < ns)
             v = __ldg(reinterpret_cast<const uint4*>(A.prof + (uint64_t)(sb + strip) * (A.A + 1) * R) + rest);
@@ -176,7 +209,8 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
         __syncthreads();
         held = want;
       }
-      const uint8_t* const pbase = smem + (lane & (max(G, 8) - 1)) * 16;
+      const int slot = lane & (max(G, MIN_SLOTS) - 1);
+      const uint8_t* const pbase = smem + slot * (DUAL && R == 8 ? 8 : 16);
       StripMeta md{NONE, 0, NONE, 0};
       if ((uint32_t)(b * G + k) < ns) md = A.meta[sb + b * G + k];
       const int ka = (int)(md.ka & ~LAST), kb = (int)(md.kb & ~LAST);
@@ -234,7 +268,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
       uint32_t shared2 = 0, thr2 = 0;
       if (LOCAL && b > 0 && valid) {
         if (ka > k) shared2 = (uint32_t)min(A.out.score[(uint64_t)md.qa * A.n_out_t + id], 0xFFFF);
-        if (kb > k) shared2 |= (uint32_t)min(A.out.score[(uint64_t)md.qb * A.n_out_t + id], 0xFFFF) << 16;
+        if (kb > k && valid2) shared2 |= (uint32_t)min(A.out.score[(uint64_t)md.qb * A.n_out_t + id2], 0xFFFF) << 16;
       }
       auto set_thr = [&]() {   // columns whose maximum reaches the best trigger
         const uint32_t v = __vmaxu2(shared2, pack2(best_a, best_b));
@@ -248,7 +282,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
       // residues of 4 steps, one block ahead: two aligned words, or (edge) the
       // four bytes with the padding residue outside the target
       auto edge_at = [&](int s0) { return s0 < G - 1 || s0 + 4 > nmin; };
-      auto fetch = [&](int s0) -> uint2 {
+      auto fetch = [&](int s0, const uint8_t* t, int n) -> uint2 {
         const int x = s0 - k;
         if (!edge_at(s0)) {
           const uint32_t* p = reinterpret_cast<const uint32_t*>((uintptr_t)(t + x) & ~(uintptr_t)3);
@@ -260,10 +294,15 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
           w |= ((uint32_t)(x + y) < (uint32_t)n ? (uint32_t)__ldg(t + x + y) : (uint32_t)A.A) << (8 * y);
         return make_uint2(w, 0);
       };
-      uint2 nxt = fetch(0);
+      uint2 nxt = fetch(0, t, n), nxt2 = DUAL ? fetch(0, t2, n2) : make_uint2(0, 0);
       for (int s0 = 0; s0 < steps; s0 += 4) {
         const uint32_t r4 = edge_at(s0) ? nxt.x : __funnelshift_r(nxt.x, nxt.y, sh);
-        nxt = fetch(s0 + 4);
+        nxt = fetch(s0 + 4, t, n);
+        uint32_t r4b = 0;
+        if (DUAL) {
+          r4b = edge_at(s0) ? nxt2.x : __funnelshift_r(nxt2.x, nxt2.y, sh2);
+          nxt2 = fetch(s0 + 4, t2, n2);
+        }
         if (LOCAL && ((s0 & 31) == 28 || s0 == 4 || s0 == 12)) {
           // the best of the query's lanes: maxima over the lanes above and
           // below that hold the same query, per half
@@ -301,14 +340,38 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
           }
           const uint32_t topH = (upH & keep) | (bH & ~keep);
           uint32_t F = (upF & keep) | (bF & ~keep);
-          const uint8_t* const p = pbase + ((r4 >> (8 * y)) & 0xFFu) * RS;
+          const uint32_t aoff = ((r4 >> (8 * y)) & 0xFFu) * RS, boff = ((r4b >> (8 * y)) & 0xFFu) * RS;
+          const uint8_t* const p = pbase + aoff;
+          uint32_t pa[DUAL ? R / 4 : 1], pb[DUAL ? R / 4 : 1];   // DUAL: the rows' bytes of the two residues
+          if (DUAL) {
+            if (R == 8) {
+              const uint2 va = *reinterpret_cast<const uint2*>(p), vb = *reinterpret_cast<const uint2*>(pbase + boff);
+              pa[0] = va.x; pa[1] = va.y; pb[0] = vb.x; pb[1] = vb.y;
+            } else {
+              const uint4 va = *reinterpret_cast<const uint4*>(p), vb = *reinterpret_cast<const uint4*>(pbase + boff);
+              pa[0] = va.x; pa[1] = va.y; pa[2] = va.z; pa[3] = va.w;
+              pb[0] = vb.x; pb[1] = vb.y; pb[2] = vb.z; pb[3] = vb.w;
+            }
+            if (R == 24) {
+              const uint8_t* const p8 = smem + PLANE + slot * 8;
+              const uint2 va = *reinterpret_cast<const uint2*>(p8 + aoff), vb = *reinterpret_cast<const uint2*>(p8 + boff);
+              pa[R / 4 - 2] = va.x; pa[R / 4 - 1] = va.y; pb[R / 4 - 2] = vb.x; pb[R / 4 - 1] = vb.y;
+            }
+          }
           uint32_t d = diag;
           diag = topH;
           uint32_t cm = 0, hprev = 0;
 #pragma unroll
           for (int q = 0; q < R / 4; ++q) {
-            const uint4 pv = *reinterpret_cast<const uint4*>(p + q * PLANE);
-            const uint32_t pr[4] = {pv.x, pv.y, pv.z, pv.w};
+            uint32_t pr[4];
+            if (DUAL) {   // the bytes are at most 127: the selector's sign copies are zeros
+#pragma unroll
+              for (uint32_t u = 0; u < 4; ++u)
+                pr[u] = prmt(pa[q], pb[q], u | (8 + u) << 4 | (4 + u) << 8 | (12 + u) << 12) - K2;
+            } else {
+              const uint4 pv = *reinterpret_cast<const uint4*>(p + q * PLANE);
+              pr[0] = pv.x; pr[1] = pv.y; pr[2] = pv.z; pr[3] = pv.w;
+            }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               const int r = q * 4 + u;
@@ -372,13 +435,28 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
                   rthr = (rthr & 0xFFFF0000u) | (sendH & 0xFFFFu);
                   rj_a = j;
                 }
-                if ((sendH >> 16) > (rthr >> 16)) {
+                if ((sendH >> 16) > (rthr >> 16) && (!DUAL || j <= n2)) {
                   rthr = (rthr & 0x0000FFFFu) | (sendH & 0xFFFF0000u);
                   rj_b = j;
                 }
               }
             }
-            if (j == n) {
+            if (DUAL) {   // each half at its own column n
+              if (j == n) {
+                hmn = (hmn & 0xFFFF0000u) | (sendH & 0xFFFFu);
+                if (qe_free) {
+#pragma unroll
+                  for (int r = 0; r < R; ++r) reinterpret_cast<uint16_t*>(parkw + r * NT)[0] = (uint16_t)Ho[r];
+                }
+              }
+              if (j == n2) {
+                hmn = (hmn & 0x0000FFFFu) | (sendH & 0xFFFF0000u);
+                if (qe_free) {
+#pragma unroll
+                  for (int r = 0; r < R; ++r) reinterpret_cast<uint16_t*>(parkw + r * NT)[1] = (uint16_t)(Ho[r] >> 16);
+                }
+              }
+            } else if (j == n) {
               hmn = sendH;
               if (qe_free) {
 #pragma unroll
@@ -392,7 +470,9 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
       // ---- the band's results, one half at a time ----
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
-        const uint32_t q = x ? md.qb : md.qa;
+        const uint32_t q = x ? md.qb : md.qa, idx_t = x ? id2 : id;
+        const int nx = x ? n2 : n;
+        const bool validx = x ? valid2 : valid;
         const int kq = x ? kb : ka;
         const int first = max(0, k - kq);         // the query's first lane in this band
         const bool starts = k - first == kq;      // its first strip is in this band
@@ -410,7 +490,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
             }
           }
           const int win = __shfl_sync(FULL, src, (lane & ~(G - 1)) + first);
-          if (valid && q != NONE && win == lane) {
+          if (validx && q != NONE && win == lane) {
             const int bs = x ? best_b : best_a, bj = x ? bj_b : bj_a;
             int bi = 0;
             if (bs > 0) {
@@ -420,7 +500,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
                 if (reinterpret_cast<const uint16_t*>(park + (x * R + r) / 8 * NT)[r & 7] == wanted) rr = r;
               bi = kq * R + rr + 1;
             }
-            const uint64_t idx = (uint64_t)q * A.n_out_t + id;
+            const uint64_t idx = (uint64_t)q * A.n_out_t + idx_t;
             bool put = starts;
             if (!put && bs > 0) {
               const int os = A.out.score[idx], ot = A.out.t_end[idx];
@@ -441,7 +521,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
           if (qe_free && q != NONE) {
             for (int r = 0; r < R; ++r) {
               const int i = base + r + 1;
-              const int v = (int)((parkw[r * NT] >> sh16) & 0xFFFFu) - A.bias - e * (i + n);
+              const int v = (int)((parkw[r * NT] >> sh16) & 0xFFFFu) - A.bias - e * (i + nx);
               if (i > pad && v > cb) { cb = v; ci = i - pad; }
             }
           }
@@ -460,15 +540,15 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
           const bool last = x ? last_b : last_a;
           const int strips = (m + R - 1) / R;
           const bool tail = q != NONE && (last || (k == G - 1 && kq < strips - 1));
-          if (valid && tail && (last || qe_free)) {
-            const uint64_t idx = (uint64_t)q * A.n_out_t + id;
+          if (validx && tail && (last || qe_free)) {
+            const uint64_t idx = (uint64_t)q * A.n_out_t + idx_t;
             if (qe_free) {
-              const int ps = starts ? row0(n) : A.out.score[idx], pi = starts ? 0 : A.out.q_end[idx];
+              const int ps = starts ? row0(nx) : A.out.score[idx], pi = starts ? 0 : A.out.q_end[idx];
               if (ps >= cb) { cb = ps; ci = pi; }   // earlier rows
             }
-            int bs = cb, bi = ci, bj = n;
+            int bs = cb, bi = ci, bj = nx;
             if (last) {
-              const int corner = (int)((hmn >> sh16) & 0xFFFFu) - A.bias - e * (base + R + n);
+              const int corner = (int)((hmn >> sh16) & 0xFFFFu) - A.bias - e * (base + R + nx);
               if (!qe_free || corner > bs) { bs = corner; bi = m; }
               if (te_free) {
                 const int rj = x ? rj_b : rj_a;
@@ -507,6 +587,7 @@ struct ProfArgs {
   int A, R, add, form;
   int pad_row, pad_col, none;   // words' halves: padding rows; padding residue on real rows; below any
   uint32_t* prof;
+  bool dual;           // a byte per row, none negative
 };
 __global__ void k_wave_profile(const ProfArgs W) {
   const uint64_t total = (uint64_t)W.n_strips * (W.A + 1) * W.R;
@@ -526,7 +607,12 @@ __global__ void k_wave_profile(const ProfArgs W) {
       const uint64_t at = W.qoff[q] + (uint64_t)i;
       return (W.P ? (int)W.P[at * W.A + a] : (int)W.S[W.qcodes[at] * W.A + a]) + W.add;
     };
-    const int lo = val(md.qa, md.ka), hi = val(md.qb, md.kb);
+    const int lo = val(md.qa, md.ka);
+    if (W.dual) {
+      reinterpret_cast<uint8_t*>(W.prof)[x] = (uint8_t)lo;
+      continue;
+    }
+    const int hi = val(md.qb, md.kb);
     W.prof[x] = W.form == LOCAL_WRAP ? pack2(lo, hi) : ((uint32_t)hi << 16) + (uint32_t)lo;
   }
 }
@@ -556,31 +642,45 @@ bool sum_fits(bool local, int64_t m, int64_t n, int o, int e, int smax, int smin
   return up + e * (m + n + 256) + sum_bias(false, o, e, smin) + 2ll * (o + e) + 512 < 65536;
 }
 
+// What makes the bytes of a two-target profile at least 0, and whether they
+// then fit 7 bits.
+static int wave_dual_K(bool local, int o, int e, int smin) {
+  return local ? std::max(0, -(smin + o + e)) : std::max({0, -(smin + 2 * e), o - 2 * e});
+}
+bool wave_dual_takes(bool local, uint32_t max_m, uint32_t max_n, int o, int e, int smax, int smin) {
+  const int add = local ? o + e : 2 * e;
+  return sum_fits(local, max_m, max_n, o, e, smax, smin) &&
+         std::max(0, smax) + add + wave_dual_K(local, o, e, smin) <= 127;
+}
+
 bool wave_takes(bool local, uint32_t max_m, uint32_t max_n, int o, int e, int smax, int smin) {
   return wave_form(local, max_m, max_n, o, e, smax, smin) >= 0;
 }
 
 int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, const dsa_db* qs,
                        const int8_t* d_matrix, const int8_t* d_pssm, int A, int mode, uint32_t fe, int o,
-                       int e, int smax, int smin, int rows, const std::vector<StripMeta>& meta,
+                       int e, int smax, int smin, int rows, bool dual, const std::vector<StripMeta>& meta,
                        const std::vector<uint32_t>& sbase, const std::vector<uint32_t>& ns,
-                       uint32_t n_targets, Scores out) {
+                       uint32_t n_targets, uint64_t residues, Scores out) {
   if (n_targets == 0 || ns.empty()) return DSA_OK;
   const bool local = mode == DSA_LOCAL;
   const uint32_t max_n = db->h_len[db->h_perm[0]];
   const int form = wave_form(local, qs->max_len, max_n, o, e, smax, smin);
   auto pick = [&](auto f) {
     constexpr int F = decltype(f)::value;
-    return rows == 8 ? k_wave<F, 8> : rows == 16 ? k_wave<F, 16> : k_wave<F, 24>;
+    constexpr bool D = F != LOCAL_WRAP;
+    if (dual) return rows == 8 ? k_wave<F, 8, D> : rows == 16 ? k_wave<F, 16, D> : k_wave<F, 24, D>;
+    return rows == 8 ? k_wave<F, 8, false> : rows == 16 ? k_wave<F, 16, false> : k_wave<F, 24, false>;
   };
   auto kern = form == LOCAL_SUM    ? pick(std::integral_constant<int, LOCAL_SUM>{})
               : form == LOCAL_WRAP ? pick(std::integral_constant<int, LOCAL_WRAP>{})
                                    : pick(std::integral_constant<int, GLOBAL_SUM>{});
-  if (form < 0 || (rows != 8 && rows != 16 && rows != 24)) {
+  if (form < 0 || (dual && !wave_dual_takes(local, qs->max_len, max_n, o, e, smax, smin)) || (rows != 8 && rows != 16 && rows != 24)) {
     set_error("no wavefront form for this search");
     return DSA_ERR_INVALID_ARG;
   }
-  const size_t smem = (size_t)(A + 1) * rows / 4 * PLANE + (size_t)rows * NT * 4;
+  const int halves = dual ? 2 : 1;   // targets per lane group
+  const size_t smem = (size_t)(A + 1) * (dual ? 32 * rows : rows / 4 * PLANE) + (size_t)rows * NT * 4;
   DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   DSA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
@@ -589,36 +689,65 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   // Lanes per target: as many as the unit has strips, up to 8 (more lanes cost
   // more steps to fill and drain on every target, and more of them idle in a
   // unit's last band; 7 queries of 90-1,100 against 50,011 targets, global:
-  // 9.3 ms with up to 16, 8.8 with 8), up to 32 for the longest targets, whose
-  // chain ends the launch, and for launches with fewer targets than the chip
-  // has room for.
-  uint32_t n_long = 0;
-  while (n_long < n_targets && db->h_len[db->h_perm[n_long]] > WAVE_LONG_TARGET) ++n_long;
+  // 9.3 ms with up to 16, 8.8 with 8).  A target's chain, its columns times the
+  // unit's bands, must stay below 0.6 of the launch, whose length in steps is the
+  // strip columns per lane of the chip: longer targets take 16 or 32 lanes (one
+  // query of 2,000 against 50,000 targets, two targets a lane: 12.3 ms with 32
+  // lanes past 2,048 columns alone, 9.1 so; 2 queries of 100 and 800: 3.8 ms at
+  // 0.35, 3.25 at 0.5 and 0.7).  Launches with fewer targets than the chip has
+  // room for take as many lanes as they can.
+  const uint64_t slots = (uint64_t)ctas * NT;
+  uint64_t strip_cols = 0;
+  for (uint32_t x : ns) strip_cols += x * residues / halves;
+  const uint64_t limit = strip_cols / slots * 3 / 5;
   std::vector<Segment> segs;
-  uint32_t items = 0;
-  bool bands = false;
-  auto lanes = [&](uint32_t strips, int most) {
-    int g = 4;
-    while (g < most && (uint32_t)g < strips) g *= 2;
-    return g;
-  };
-  for (int part = 0; part < 2; ++part) {
-    const uint32_t first = part ? n_long : 0, count = part ? n_targets - n_long : n_long;
-    if (count == 0) continue;
+  size_t n_first = 0;
+  uint64_t cols = 0;   // boundary cells of a warp
+  std::vector<uint32_t> next(ns.size(), 0);   // the unit's targets dealt so far
+  for (int most = 32; most >= FEW_LANES; most /= 2) {
     for (uint32_t u = 0; u < ns.size(); ++u) {
-      int G = lanes(ns[u], part ? FEW_LANES : 32);
-      while (G < 32 && (uint32_t)G < ns[u] &&
-             (uint64_t)n_targets * ns.size() * G < (uint64_t)ctas * NT)
-        G *= 2;
-      segs.push_back({u, first, count, items, G});
-      items += (count + NW * 32 / G - 1) / (NW * 32 / G);
-      bands = bands || ns[u] > (uint32_t)G;
+      // targets whose chain on half the lanes is too long
+      uint32_t end = n_targets;
+      if (most > FEW_LANES) {
+        const uint64_t bands = (ns[u] + most / 2 - 1) / (most / 2);
+        const uint64_t longest = std::min<uint64_t>(limit / bands, WAVE_LONG_TARGET);
+        end = (uint32_t)(std::partition_point(db->h_perm.begin() + next[u], db->h_perm.begin() + n_targets,
+                                              [&](uint32_t t) { return db->h_len[t] > longest; }) -
+                         db->h_perm.begin());
+      }
+      const uint32_t first = next[u], count = end - first;
+      if (count == 0) continue;
+      next[u] = end;
+      int G = 4;
+      while (G < 32 && (uint32_t)G < ns[u] && (G < most || n_targets / halves * ns.size() * G < slots)) G *= 2;
+      segs.push_back({u, first, count, 0, G, NW});
+      n_first += most == 32;
+      if (ns[u] > (uint32_t)G) cols = std::max<uint64_t>(cols, 32ull / G * db->h_len[db->h_perm[first]]);
     }
   }
+  auto items_of = [&](size_t from, size_t to, int warps) {
+    uint64_t x = 0;
+    for (size_t k = from; k < to; ++k) {
+      const uint32_t per = warps * 32 / segs[k].G * halves;
+      x += (segs[k].count + per - 1) / per;
+    }
+    return x;
+  };
+  // A launch that does not fill the chip, and the longest targets of any, use
+  // fewer warps of more CTAs: a chain's step takes 600 cycles on a scheduler of
+  // its own and 1,300 beside three others (128 residues against 2,000 targets
+  // 0.60 -> 0.54 ms, against 200,000 2.58 -> 2.15).
+  int w_all = NW;
+  while (w_all > MIN_WARPS && items_of(0, segs.size(), w_all / 2) <= ctas) w_all /= 2;
+  int w_first = w_all;
+  while (w_first > MIN_WARPS && items_of(0, n_first, w_first / 2) <= ctas / 4) w_first /= 2;
+  uint32_t items = 0;
+  for (size_t k = 0; k < segs.size(); ++k) {
+    segs[k].warps = k < n_first ? w_first : w_all;
+    segs[k].item0 = items;
+    items += (uint32_t)items_of(k, k + 1, segs[k].warps);
+  }
   const unsigned grid = std::min<uint32_t>(items, ctas);
-  // boundary cells of a warp: its longest target, or two of the shorter ones
-  const uint64_t cols =
-      bands ? std::max<uint64_t>(max_n, 32ull / FEW_LANES * std::min(max_n, WAVE_LONG_TARGET)) : 0;
 
   WaveArgs W{};
   W.tcodes = db->d_codes; W.toff = db->d_off; W.tlen = db->d_len; W.perm = db->d_perm;
@@ -631,15 +760,17 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   P.n_strips = (uint32_t)meta.size();
   P.S = d_matrix; P.P = d_pssm;
   P.A = A; P.R = rows; P.form = form;
-  P.add = form == LOCAL_SUM ? o + e : form == LOCAL_WRAP ? o : 2 * e;
-  P.none = form == LOCAL_WRAP ? NEG16 : -128;
+  W.K = dual ? wave_dual_K(local, o, e, smin) : 0;
+  P.dual = dual;
+  P.add = (form == LOCAL_SUM ? o + e : form == LOCAL_WRAP ? o : 2 * e) + W.K;
+  P.none = dual ? 0 : form == LOCAL_WRAP ? NEG16 : -128;
   if (!local) {
     const bool sg = mode == DSA_SEMIGLOBAL;
     P.pad_row = sg && (fe & DSA_FREE_T_BEGIN) ? P.add : P.add - o;
     P.pad_col = sg && (fe & DSA_FREE_Q_BEGIN) ? P.add : P.add - o;
   }
   const int pw = local ? P.none : P.pad_row;
-  W.pad_word = form == LOCAL_WRAP ? (uint32_t)(pw & 0xFFFF) * 0x10001u : ((uint32_t)pw << 16) + (uint32_t)pw;
+  W.pad_word = dual ? (uint32_t)pw * 0x01010101u : form == LOCAL_WRAP ? (uint32_t)(pw & 0xFFFF) * 0x10001u : ((uint32_t)pw << 16) + (uint32_t)pw;
 
   // one upload: segments, strip records, each unit's first strip and strip count
   const size_t b_seg = (segs.size() * sizeof(Segment) + 15) & ~(size_t)15;
@@ -650,7 +781,7 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   memcpy(host.data() + b_seg, meta.data(), meta.size() * sizeof(StripMeta));
   memcpy(host.data() + b_seg + b_meta, sbase.data(), sbase.size() * 4);
   memcpy(host.data() + b_seg + b_meta + b_u, ns.data(), ns.size() * 4);
-  const size_t b_prof = (size_t)P.n_strips * (A + 1) * rows * 4;
+  const size_t b_prof = ((size_t)P.n_strips * (A + 1) * rows * (dual ? 1 : 4) + 15) & ~(size_t)15;
   const size_t b_scr = (size_t)grid * NW * cols * sizeof(uint2);
   void* buf = nullptr;
   const size_t b_all = host.size() + b_prof + b_scr + 16;

@@ -118,13 +118,17 @@ int ilog2_bin(uint64_t x) {
 // strips of W rows, are dealt, longest first, to the currently shortest of K
 // lanes (K about total / longest, so a lane is about as long as the longest
 // query, or as `at_least` strips); lanes are then paired by length into units,
-// low half = first lane, high half = second.
+// low half = first lane, high half = second.  A pair of unequal lanes wastes the
+// difference, so fewer lanes are taken where they waste less (5 queries of
+// 60-700: 33 packed strips of 24 rows with 2 lanes, 39 with 4, the local search
+// of 60,000 targets 7.2 -> 5.9 ms).  dual: both halves of a unit follow one
+// lane, against two targets.
 struct Streams {
   std::vector<StripMeta> meta;
   std::vector<uint32_t> sbase, ns;   // per unit: first strip, strips
 };
 Streams build_streams(const dsa_db* qs, const std::vector<uint32_t>& qorder, uint32_t W,
-                      uint64_t at_least = 1) {
+                      uint64_t at_least = 1, bool dual = false) {
   const uint32_t nq = qs->n;
   auto strips_of = [&](uint32_t q) { return (qs->h_len[q] + W - 1) / W; };
   uint64_t tot = 0, maxq = at_least;
@@ -132,19 +136,33 @@ Streams build_streams(const dsa_db* qs, const std::vector<uint32_t>& qorder, uin
     tot += strips_of(q);
     maxq = std::max<uint64_t>(maxq, strips_of(q));
   }
-  uint32_t K = (uint32_t)std::max<uint64_t>(1, (tot + maxq - 1) / maxq);
-  K = std::min<uint32_t>(K, nq);
-  K = (K + 1) & ~1u;   // even: lanes come in pairs
-  std::vector<std::vector<uint32_t>> lanes(K);
-  std::vector<uint64_t> load(K, 0);
-  for (uint32_t q : qorder) {
-    const uint32_t l = (uint32_t)(std::min_element(load.begin(), load.end()) - load.begin());
-    lanes[l].push_back(q);
-    load[l] += strips_of(q);
+  const uint32_t most = std::min<uint32_t>((uint32_t)std::max<uint64_t>(1, (tot + maxq - 1) / maxq), nq);
+  std::vector<std::vector<uint32_t>> lanes;
+  std::vector<uint64_t> load;
+  std::vector<uint32_t> lorder;
+  auto deal = [&](uint32_t K) -> uint64_t {   // strips of all units
+    lanes.assign(K, {});
+    load.assign(K, 0);
+    for (uint32_t q : qorder) {
+      const uint32_t l = (uint32_t)(std::min_element(load.begin(), load.end()) - load.begin());
+      lanes[l].push_back(q);
+      load[l] += strips_of(q);
+    }
+    lorder.resize(K);
+    std::iota(lorder.begin(), lorder.end(), 0u);
+    std::stable_sort(lorder.begin(), lorder.end(), [&](uint32_t a, uint32_t b) { return load[a] > load[b]; });
+    uint64_t strips = 0;
+    for (uint32_t l = 0; l < K; l += dual ? 1 : 2) strips += load[lorder[l]];
+    return strips;
+  };
+  uint32_t K = dual ? most : (most + 1) & ~1u;   // even: lanes come in pairs
+  if (dual || K < 4) {
+    deal(K);
+  } else {
+    const uint64_t more = deal(K), fewer = deal(K - 2);
+    if (fewer < more) K -= 2;
+    else deal(K);
   }
-  std::vector<uint32_t> lorder(K);
-  std::iota(lorder.begin(), lorder.end(), 0u);
-  std::stable_sort(lorder.begin(), lorder.end(), [&](uint32_t a, uint32_t b) { return load[a] > load[b]; });
   Streams S;
   // query and strip index (with the LAST bit) of strip s of a lane, in order
   auto fill = [&](const std::vector<uint32_t>& lane, uint64_t n, auto put) {
@@ -155,7 +173,14 @@ Streams build_streams(const dsa_db* qs, const std::vector<uint32_t>& qorder, uin
     }
     for (; s < n; ++s) put(s, NONE, 0u);
   };
-  for (uint32_t u = 0; u < K / 2; ++u) {
+  for (uint32_t u = 0; dual && u < K; ++u) {
+    const size_t at = S.meta.size();
+    S.sbase.push_back((uint32_t)at);
+    S.ns.push_back((uint32_t)load[u]);
+    S.meta.resize(at + load[u]);
+    fill(lanes[u], load[u], [&](uint64_t st, uint32_t q, uint32_t k) { S.meta[at + st] = {q, k, q, k}; });
+  }
+  for (uint32_t u = 0; !dual && u < K / 2; ++u) {
     const uint64_t ns_u = std::max(load[lorder[2 * u]], load[lorder[2 * u + 1]]);
     if (ns_u == 0) continue;
     const size_t at = S.meta.size();
@@ -177,16 +202,27 @@ Streams build_streams(const dsa_db* qs, const std::vector<uint32_t>& qorder, uin
 // against 12,000 0.91 (1.14, 1.56).  Past one band they lose, 300 residues 1.24
 // (0.86, 1.01), and with more lanes too, 16 queries against 2,000 1.48 (1.19,
 // 1.18).
-int wave_rows(const dsa_ctx* ctx, const dsa_db* qs, uint32_t n_targets) {
+int wave_rows(const dsa_ctx* ctx, const dsa_db* qs, uint32_t n_targets, bool dual) {
   auto strips = [&](uint32_t R) {
     uint64_t c = 0;
     for (uint32_t m : qs->h_len) c += (m + R - 1) / R;
     return c;
   };
   auto cost = [&](uint32_t R) { return strips(R) * (R * 11 + 45); };
-  const uint64_t lanes = std::max<uint64_t>((qs->max_len + 7) / 8, (strips(8) + 1) / 2);
-  if (lanes <= 32 && lanes * n_targets <= 3ull * 512 * ctx->sm_count) return 8;
+  const uint64_t lanes = dual ? strips(8) : std::max<uint64_t>((qs->max_len + 7) / 8, (strips(8) + 1) / 2);
+  if (lanes <= 32 && lanes * n_targets / (dual ? 2 : 1) <= 3ull * 512 * ctx->sm_count) return 8;
   return cost(16) < cost(24) ? 16 : 24;
+}
+
+// Few queries, or one much longer than the rest, leave one of two query
+// streams idle: the wavefronts then take two targets a lane.  Such a step reads
+// bytes for both residues and joins them (about 1.17 of the time of a step on
+// two queries: 32 queries of 200-1,500 against 60,000 targets 80.0 and 93.3 ms).
+bool wave_dual(const dsa_db* qs, const Validated& v, bool local, uint32_t max_n, int o, int e) {
+  if (!wave_dual_takes(local, qs->max_len, max_n, o, e, v.smax, v.smin)) return false;
+  uint64_t sum = 0;
+  for (uint32_t m : qs->h_len) sum += m;
+  return 2ull * qs->max_len * 10 > sum * 12;
 }
 
 // Packed score pass (int16x2).  Targets of groups longer than `long_thr` go
@@ -304,7 +340,19 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
     DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0));
   }
   if (wave) {
-    const int wr = wave_rows(ctx, qs, n_long);
+    bool dual = wave_dual(qs, v, local, db->h_glen[0], o, e);
+    int wr = wave_rows(ctx, qs, n_long, dual);
+    // two targets a lane halve the work but not the longest target's chain: not
+    // where the work, as strip columns per lane of the chip, is the shorter (one
+    // query of 300 residues against 2,000 targets, global, 0.70 and 0.96 ms, of
+    // 700 against 50,000 4.0 and 2.5)
+    if (dual) {
+      const uint64_t steps = (uint64_t)((qs->max_len + wr - 1) / wr) * long_res / (ctx->sm_count * 512ull);
+      if (steps * 4 < 3ull * db->h_glen[0]) {
+        dual = false;
+        wr = wave_rows(ctx, qs, n_long, dual);
+      }
+    }
     // longer streams waste fewer lanes and balance the halves better, until the
     // longest target's pass over a unit would take half the launch: each of the
     // chip's lanes has total / lanes strip columns to compute, the longest
@@ -313,10 +361,10 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
     for (uint32_t m : qs->h_len) strips += (m + wr - 1) / wr;
     const uint64_t share = strips / 2 * long_res / ((uint64_t)ctx->sm_count * 512);
     const Streams ws =
-        build_streams(qs, qorder, (uint32_t)wr, 32 * (share / (2ull * db->h_glen[0])));
+        build_streams(qs, qorder, (uint32_t)wr, 32 * (share / (2ull * db->h_glen[0])), dual);
     phase_begin(res, PH_INTRA, ls);
     DSA_TRY(launch_wave_search(ctx, ls, db, qs, d_mat, d_pssm, A, mode, fe, o, e, v.smax, v.smin, wr,
-                               ws.meta, ws.sbase, ws.ns, n_long, out));
+                               dual, ws.meta, ws.sbase, ws.ns, n_long, long_res, out));
     phase_end(res, PH_INTRA, ls);
   } else if (n_long) {
     DSA_TRY(upload(ctx, d_pmeta, pmeta));
@@ -380,7 +428,9 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
 // against 60,000 targets took 23.3 ms with a threshold of 4,096, 8.6 with
 // 1,024 and 7.2 on the wavefronts alone; 0 where little would be left for the
 // inter-sequence kernel.
-uint32_t model_threshold(const dsa_db* db, const dsa_db* qs) {
+uint32_t model_threshold(const dsa_db* db, const dsa_db* qs, const Validated& v, bool local, int o, int e) {
+  // the inter-sequence kernel would leave one of its two streams idle
+  if (wave_dual(qs, v, local, db->h_glen[0], o, e)) return 0;
   uint64_t strips = 0, longest = 1;
   for (uint32_t m : qs->h_len) {
     const uint64_t n = (m + INTER_ROWS - 1) / INTER_ROWS;
@@ -421,7 +471,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   const char* mode_env = getenv("DSA_AUTOTUNE");
   const std::string tmode = mode_env ? mode_env : "cache";
   const int rows_default = rows_forced ? rows_forced : INTER_ROWS;
-  const uint32_t thr_default = thr_env ? thr_forced : model_threshold(db, qs);
+  const uint32_t thr_default = thr_env ? thr_forced : model_threshold(db, qs, v, local, o, e);
   if (tmode == "off" || (rows_forced && thr_env))
     return run(res, thr_default, rows_default);
   // workload shape key: GPU, driver, mode, alphabet, and log2 bins of the

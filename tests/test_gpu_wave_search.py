@@ -114,3 +114,22 @@ def test_short_strips_of_small_searches(ctx, lengths, mode, fe, monkeypatch):
     g = gpu_all(ctx, queries, db, S, 11, 1, mode=mode, fe=fe)
     assert_same(g[:3], oracle_all(queries, db, S, 11, 1, mode, fe), f"{lengths} mode={mode}")
     assert g[5].phase_cells()["inter16"] == 0
+
+
+@pytest.mark.parametrize("lengths", [[7], [100], [257], [24 * 16 + 1], [24 * 32, 5], [700, 30, 100], [1100, 16, 17, 3]])
+@pytest.mark.parametrize("mode,fe", MODES)
+@pytest.mark.parametrize("n_targets", [1, 2, 150])
+def test_two_targets_a_lane(ctx, lengths, mode, fe, n_targets, monkeypatch):
+    """Queries whose streams would leave one half idle: one of them, or one much
+    longer than the rest; odd and even numbers of targets, and tails."""
+    monkeypatch.setenv("DSA_LONG_THRESHOLD", "0")
+    rng = np.random.default_rng(5600 + sum(lengths) + 16 * mode + fe)
+    bg = W.protein_background()
+    queries = W._make_set(rng, np.asarray(lengths), bg)
+    db = _db(rng, queries, bg, 2600)
+    if n_targets < db.n:
+        db = W.SeqSet.from_list([db.seq(db.n - 1 - k) for k in range(n_targets)])
+    for S, o, e in ((W.blosum62(), 11, 1), (W.blosum62(), 2, 1)):   # bytes as they are; lifted by K
+        g = gpu_all(ctx, queries, db, S, o, e, mode=mode, fe=fe)
+        assert_same(g[:3], oracle_all(queries, db, S, o, e, mode, fe), f"{lengths} mode={mode} o={o}")
+        assert g[5].phase_cells()["inter16"] == 0
