@@ -153,9 +153,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
   const bool t_end_free = sg && (fe & DSA_FREE_T_END);
   const uint32_t neg_o2 = pack2(-o, -o), neg_e2 = pack2(-e, -e);
   const uint32_t o2 = ((uint32_t)o << 16) | (uint32_t)o;
-  // SUM: values carry e (i + j), and a stored H is H - Kp
-  const uint32_t K2 = (uint32_t)Kp * 0x10001u, c2 = pack2(Kp + e - o, Kp + e - o);
-  const int32_t hs = SUM ? Kp : o;       // a stored H is H - hs
+  // SUM: values carry e (i + j); the bytes' Kp is taken off in the same addition
+  const uint32_t K2 = (uint32_t)Kp * 0x10001u, c2 = pack2(e - o, e - o);
+  const int32_t hs = SUM ? 0 : o;        // a stored H is H - hs
   auto ge = [&](int32_t i, int32_t j) { return SUM ? e * (i + j) : 0; };
   bool timed_out = false;
 
@@ -343,11 +343,11 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_long_score16(
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
           if (SUM) {
-            const uint32_t hk = max3_2u(d + prmt(sA[r], sB[r], sel), E[r], F) - K2;
+            const uint32_t h = max3_2u(d + prmt(sA[r], sB[r], sel) - K2, E[r], F);
             d = Ho[r];
-            Ho[r] = hk;
-            E[r] = addmax2u(hk, c2, E[r]);
-            if (r + 1 < ROWS) F = addmax2u(hk, c2, F);
+            Ho[r] = h;
+            E[r] = addmax2u(h, c2, E[r]);
+            if (r + 1 < ROWS) F = addmax2u(h, c2, F);
             continue;
           }
           E[r] = addmax2u(E[r], neg_e2, Ho[r]);

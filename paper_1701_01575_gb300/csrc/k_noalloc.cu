@@ -22,7 +22,7 @@
 // the strip's last row handed on through a boundary row), does those.
 //
 // Bound by the ALU pipe.  30,011 reads of 36-301 bp in 411 bp windows,
-// semi-global: 47.1 ms with one thread per pair for all, 1.15 ms now.
+// semi-global: 47.1 ms with one thread per pair for all, 1.2 ms now.
 #include "pairwave.cuh"
 
 #include <algorithm>

@@ -9,11 +9,11 @@
 //
 // Bound by the ALU pipe and, at the end of a call, by the longest pair's
 // chain.  Measured against the forms it replaces (whole call): 20,000 protein
-// pairs of 50-1,500 residues, local, 133.6 -> 2.59 ms (one thread per two
-// pairs, two table loads per packed cell); 15,001 such pairs, global, 241.5 ->
-// 1.58 ms (one thread per pair in int32, their range being past that form's
-// rule); 1,000 reads of 150 bp in 500 bp windows with traceback 1.85 -> 0.64 ms; 1,000,000 of
-// 150 and 250 bp, 27.6 -> 23.9 ms.
+// pairs of 50-1,500 residues, local, 135 -> 2.61 ms (one thread per two
+// pairs, two table loads per packed cell); 15,001 such pairs, global, 244 ->
+// 1.49 ms (one thread per pair in int32, their range being past that form's
+// rule); 1,000 reads of 150 bp in 500 bp windows with traceback 1.76 -> 0.64 ms; 1,000,000 of
+// 150 and 250 bp, 27.4 -> 23.5 ms.
 #include "pairwave.cuh"
 #include "host_util.cuh"
 

@@ -37,11 +37,13 @@
 // Cell update, global and semi-global: every value is kept with e (i + j)
 // added, so extending a gap adds nothing, and E and F of the next cell are one
 // operation each; with G = value + e (i + j) and P = S + 2e + K >= 0:
-//   x = Gk_diag + P;  G = max(x, E, F);  Gk = G - K;
-//   E' = max(Gk + (K + e - o), E);  F' = max(Gk + (K + e - o), F)
-// The two sums are plain 32-bit additions: no half leaves [0, 2^16), so
+//   x = G_diag + P - K;  G = max(x, E, F);
+//   E' = max(G + (e - o), E);  F' = max(G + (e - o), F)
+// The sum is one 32-bit addition of three terms: no half leaves [0, 2^16), so
 // nothing carries from one into the other.  Three of the five operations are
-// maxima on the half-rate pipe, against four of five before.
+// maxima on the half-rate pipe.  (Taking K off after the maxima instead put a
+// third operation per row on F's chain: 20,000 protein pairs of 1,024 x 1,024,
+// two warps per scheduler, 4.59 ms so and 3.93 now.)
 //
 // Range.  Local: the saturation rule of the other packed kernels (a best above
 // 32767 - max S is rerun in int32 by the caller).  Global and semi-global:
@@ -160,7 +162,7 @@ __device__ __forceinline__ void pair_wave_run(const WaveParams& W, const uint8_t
   const bool tb_free = sg && (W.fe & DSA_FREE_T_BEGIN), te_free = sg && (W.fe & DSA_FREE_T_END);
   const uint32_t neg_e2 = pack2(-e, -e), o2 = pack2(o, 0) + ((uint32_t)o << 16);
   const uint32_t K2 = (uint32_t)W.K * 0x10001u;
-  const uint32_t c2 = pack2(W.K + e - o, W.K + e - o);
+  const uint32_t c2 = pack2(e - o, e - o);
   const uint32_t e2 = (uint32_t)e * 0x10001u;
   const int jl0 = -2 * k;   // the low half's column before step 1
   // local: H = 0 as H - o (summed: at the halves' columns before step 1)
@@ -179,7 +181,7 @@ __device__ __forceinline__ void pair_wave_run(const WaveParams& W, const uint8_t
   // rows: 0), and of F entering row i' + 1 there, with e (i' + j) added
   auto hv = [&](int i, int j) {
     const int h = (i <= pad || qb_free) ? 0 : -(o + (i - pad - 1) * e);
-    return W.bias + h + e * (i + j) - W.K;
+    return W.bias + h + e * (i + j);
   };
   auto fv = [&](int i, int j) {
     const int f = (i <= pad || qb_free) ? -o : -(o + (i - pad) * e);
@@ -274,9 +276,9 @@ __device__ __forceinline__ void pair_wave_run(const WaveParams& W, const uint8_t
     uint32_t inH = mo2 << 16, inF = mo2 << 16, inc = LSUM ? (uint32_t)e << 16 : 0u, inw = 0;
     if (!LOCAL) {
       // row 0: constant from column 1 on, or rising by e with a free begin
-      const uint32_t v = (uint32_t)(W.bias - W.K + (tb_free ? 0 : e - o));
+      const uint32_t v = (uint32_t)(W.bias + (tb_free ? 0 : e - o));
       inH = v << 16;
-      inF = (v + (uint32_t)(W.K + e - o)) << 16;
+      inF = (v + (uint32_t)(e - o)) << 16;
       inc = tb_free ? (uint32_t)e << 16 : 0u;
     }
     if (b > 0 && k == 0 && n > 0) inw = scr[0];
@@ -351,11 +353,10 @@ __device__ __forceinline__ void pair_wave_run(const WaveParams& W, const uint8_t
           if (r & 1) cm = max3_2u(cm, hprev, h);
           else hprev = h;
         } else {
-          const uint32_t h = max3_2u(d + sp, E[r], F);
-          const uint32_t hk = h - K2;
-          Ho[r] = hk;
-          E[r] = addmax2u(hk, c2, E[r]);
-          F = addmax2u(hk, c2, F);
+          const uint32_t h = max3_2u(d + sp - K2, E[r], F);
+          Ho[r] = h;
+          E[r] = addmax2u(h, c2, E[r]);
+          F = addmax2u(h, c2, F);
         }
         d = old;
       }
@@ -366,17 +367,19 @@ __device__ __forceinline__ void pair_wave_run(const WaveParams& W, const uint8_t
         if (__vmaxu2(cm, thr2) != thr2) {
           const int cl = (int)(cm & 0xFFFFu) - (LSUM ? (int)(flo2 & 0xFFFFu) + o : 0x8000);
           const int ch = (int)(cm >> 16) - (LSUM ? (int)(flo2 >> 16) + o : 0x8000);
-          if (cl >= gbest && cl > best_lo - (j < bj_lo ? 1 : 0)) {
+          const bool lo = cl >= gbest && cl > best_lo - (j < bj_lo ? 1 : 0);
+          const bool hi = ch >= gbest && ch > best_hi - (j - 1 < bj_hi ? 1 : 0);
+          // lanes that raise either half park it in one pass
+          if (lo | hi) {
+            auto keep_half = [&](uint2* p, uint32_t sel) {
 #pragma unroll
-            for (int r = 0; r < R; r += 4)
-              park[r / 4 * 32] = make_uint2(prmt(Ho[r], Ho[r + 1], 0x5410), prmt(Ho[r + 2], Ho[r + 3], 0x5410));
-            best_lo = cl; bj_lo = j; pend |= 1;
-          }
-          if (ch >= gbest && ch > best_hi - (j - 1 < bj_hi ? 1 : 0)) {
-#pragma unroll
-            for (int r = 0; r < R; r += 4)
-              park[(Q + r / 4) * 32] = make_uint2(prmt(Ho[r], Ho[r + 1], 0x7632), prmt(Ho[r + 2], Ho[r + 3], 0x7632));
-            best_hi = ch; bj_hi = j - 1; pend |= 2;
+              for (int r = 0; r < R; r += 4)
+                p[r / 4 * 32] = make_uint2(prmt(Ho[r], Ho[r + 1], sel), prmt(Ho[r + 2], Ho[r + 3], sel));
+            };
+            keep_half(park + (lo ? 0 : Q * 32), lo ? 0x5410u : 0x7632u);
+            if (lo & hi) keep_half(park + Q * 32, 0x7632u);
+            if (lo) { best_lo = cl; bj_lo = j; pend |= 1; }
+            if (hi) { best_hi = ch; bj_hi = j - 1; pend |= 2; }
           }
           set_thr();
         }
@@ -389,19 +392,19 @@ __device__ __forceinline__ void pair_wave_run(const WaveParams& W, const uint8_t
               rthr = own_lo ? (rthr & 0xFFFF0000u) | (sendH & 0xFFFFu)
                             : (rthr & 0x0000FFFFu) | (sendH & 0xFFFF0000u);
               rj = jj;
-              rbest = (int)(own_lo ? sendH & 0xFFFFu : sendH >> 16) + W.K - W.bias - e * (mp + jj);
+              rbest = (int)(own_lo ? sendH & 0xFFFFu : sendH >> 16) - W.bias - e * (mp + jj);
             }
           }
         }
         if (EDGE && (uint32_t)(j - n) <= 1u) {   // column n, low half then high half
           const int x = j - n, sh = 16 * x;
           if (x ? own_hi : own_lo)
-            hmn = (int)((sendH >> sh) & 0xFFFFu) + W.K - W.bias - e * (mp + n);
+            hmn = (int)((sendH >> sh) & 0xFFFFu) - W.bias - e * (mp + n);
           if (qe_free) {
 #pragma unroll
             for (int r = 0; r < R; ++r) {
               const int i = base + x * R + r + 1;
-              const int v = (int)((Ho[r] >> sh) & 0xFFFFu) + W.K - W.bias - e * (i + n);
+              const int v = (int)((Ho[r] >> sh) & 0xFFFFu) - W.bias - e * (i + n);
               if (i > pad && i <= mp && v > cb) { cb = v; ci = i - pad; }
             }
           }
