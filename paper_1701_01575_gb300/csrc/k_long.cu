@@ -632,16 +632,28 @@ __global__ void __launch_bounds__(128) k_long_tb_windows(
 // ending at the walk's column -- and reloads it with coalesced row loads
 // whenever the walk leaves it (the walk only moves up and left), so each step
 // reads shared memory instead of waiting on a global load.
-constexpr int WIN_WORDS = 32;
+//
+// AHEAD: bound by these reloads' latency, one or two a band (a band is walked
+// in about 2 us and a reload takes about as long), so a second window is
+// filled with the next band's words around the diagonal while this band is
+// walked, and taken if the walk arrives inside it.  Two windows allow 3 walks
+// per SM: for calls of no more hits than that.  64 global pairs of
+// 10,000-100,000: traceback 11.4 -> 10.65 ms; 7 local pairs up to 60,000: 3.82
+// -> 3.43.
+constexpr int WIN_WORDS = 36;   // 256 columns of a band's diagonal and 4 words of drift
 constexpr int WIN_ROWS = 256;   // a window word's rows are consecutive (as in global memory)
+constexpr int WIN_SIZE = WIN_WORDS * WIN_ROWS;
 
+template <bool AHEAD>
 __global__ void __launch_bounds__(32) k_long_tb_walk(const LongTbJob* __restrict__ jobs,
                                                      uint32_t n_jobs, int mode, uint32_t fe,
                                                      const uint32_t* __restrict__ dir,
                                                      uint32_t* __restrict__ cig_tmp,
                                                      dsa_hit* __restrict__ hits,
                                                      const int2* __restrict__ bwin) {
-  __shared__ __align__(16) uint32_t win[WIN_WORDS * WIN_ROWS];
+  extern __shared__ __align__(16) uint32_t walk_windows[];
+  uint32_t* win = walk_windows;          // the window in use
+  uint32_t* other = walk_windows + (AHEAD ? WIN_SIZE : 0);
   constexpr unsigned FULL = 0xFFFFFFFFu;
   const int lane = threadIdx.x;
   const bool local = mode == DSA_LOCAL;
@@ -651,6 +663,33 @@ __global__ void __launch_bounds__(32) k_long_tb_walk(const LongTbJob* __restrict
     const uint32_t* D = dir + jb.dir_off;
     const uint32_t wpr = jb.wpr;
     int32_t wb = -1, wlo = 0, wr0 = 0, wr1 = 0;   // window: band, first word, rows [wr0, wr1)
+    int32_t pb = -1, plo = 0;                     // AHEAD: the other window's band and first word
+    int32_t kept = -1, kept_lo = 0, kept_w = 0;   // lane k: stored columns of band kept - k
+    auto columns = [&](int32_t b, int32_t& lo, int32_t& w) {
+      if (b > kept || b <= kept - 32) {
+        kept = b;
+        if (b - lane >= 0) band_window(jb, bwin, b - lane, kept_lo, kept_w);
+      }
+      lo = __shfl_sync(FULL, kept_lo, kept - b);
+      w = __shfl_sync(FULL, kept_w, kept - b);
+    };
+    // words w0 .. of rows r0 .. r1 - 1 of band b (multiples of 4): each word's
+    // rows are consecutive in the decision layout and in the window, so the
+    // warp copies 16-byte pieces (4 rows), every copy in flight at once
+    auto copy = [&](uint32_t* to, int32_t b, int32_t w0, int32_t r0, int32_t r1) {
+      const uint32_t* Db = D + (uint64_t)b * wpr * TB_BAND;
+      const int32_t n4 = (r1 - r0) >> 2;
+#pragma unroll 4
+      for (int k = 0; k < WIN_WORDS; ++k) {
+        const int32_t w = w0 + k;
+        for (int c = lane; c < n4; c += 32) {
+          uint32_t* dst = to + k * WIN_ROWS + 4 * c;
+          if (w < (int32_t)wpr) cp_async16(dst, Db + (uint64_t)w * TB_BAND + (uint32_t)(r0 + 4 * c));
+          else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+        }
+      }
+      cp_async_commit();
+    };
     RevCigar c;
     c.out = cig_tmp + jb.cig_off;
     c.writer = lane == 0;
@@ -744,39 +783,40 @@ __global__ void __launch_bounds__(32) k_long_tb_walk(const LongTbJob* __restrict
       const int32_t ci = __shfl_sync(FULL, i, 0), cj = __shfl_sync(FULL, j, 0);
       wb = (ci - 1) / TB_BAND;
       int32_t jlo, wcb;
-      band_window(jb, bwin, wb, jlo, wcb);
+      columns(wb, jlo, wcb);
       if (cj < jlo || cj >= jlo + wcb) break;
       const int32_t wi = (cj - jlo) >> 3;
-      wlo = max(0, wi - (WIN_WORDS - 1));
       wr1 = ci - wb * TB_BAND;
       rr = wr1 - 1;
-      // rows from a multiple of 4 (16-byte copies), ending at or after the
-      // walk's row
-      const int32_t wr1a = min((wr1 + 3) & ~3, TB_BAND);
-      wr0 = max(0, wr1a - WIN_ROWS);
       jc = cj - jlo;
+      cp_async_wait<0>();   // the other window's copies
       __syncwarp();
-      // words wlo .. wlo + 31 of rows wr0 .. wr1a - 1 of band wb: each
-      // word's rows are consecutive in the decision layout and in the window,
-      // so the warp copies 16-byte pieces (4 rows), every copy in flight at
-      // once: a reload costs about one memory latency
-      {
-        const uint32_t* Db = D + (uint64_t)wb * wpr * TB_BAND;
-        const int32_t n4 = (wr1a - wr0) >> 2;
-#pragma unroll 4
-        for (int k = 0; k < WIN_WORDS; ++k) {
-          const int32_t w = wlo + k;
-          for (int c = lane; c < n4; c += 32) {
-            uint32_t* dst = win + k * WIN_ROWS + 4 * c;
-            if (w < (int32_t)wpr) cp_async16(dst, Db + (uint64_t)w * TB_BAND + (uint32_t)(wr0 + 4 * c));
-            else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
-          }
-        }
+      if (AHEAD && pb == wb && wi >= plo && wi < plo + WIN_WORDS) {
+        uint32_t* const t = win;
+        win = other;
+        other = t;
+        wlo = plo;
+        wr0 = 0;
+      } else {
+        // rows from a multiple of 4 (16-byte copies), ending at or after the
+        // walk's row
+        wlo = max(0, wi - (WIN_WORDS - 1));
+        const int32_t wr1a = min((wr1 + 3) & ~3, TB_BAND);
+        wr0 = max(0, wr1a - WIN_ROWS);
+        copy(win, wb, wlo, wr0, wr1a);
+        cp_async_wait<0>();
+        __syncwarp();
       }
-      cp_async_commit();
-      cp_async_wait<0>();
-      __syncwarp();
+      if (AHEAD && wb > 0) {   // the next band, entered about wr1 columns from here
+        int32_t nlo, nw;
+        columns(wb - 1, nlo, nw);
+        pb = wb - 1;
+        plo = max(0, min((cj - wr1 - nlo) >> 3, (nw - 1) >> 3) + 2 - (WIN_WORDS - 1));
+        copy(other, pb, plo, 0, TB_BAND);
+      }
     }
+    cp_async_wait<0>();
+    __syncwarp();
     if (lane == 0) {
       c.flush();
       dsa_hit* h = hits + jb.hit;
@@ -865,8 +905,11 @@ int launch_long_tb_walk(dsa_ctx* ctx, cudaStream_t stream, const LongTbJob* d_jo
                         uint32_t n_jobs, int mode, uint32_t fe, const uint32_t* d_dir,
                         uint32_t* d_cig_tmp, dsa_hit* d_hits, const int2* d_win) {
   if (n_jobs == 0) return DSA_OK;
-  k_long_tb_walk<<<n_jobs, 32, 0, stream>>>(d_jobs, n_jobs, mode, fe, d_dir, d_cig_tmp, d_hits,
-                                            d_win);
+  const bool ahead = n_jobs <= 3u * (uint32_t)ctx->sm_count;
+  const size_t smem = (ahead ? 2 : 1) * WIN_SIZE * sizeof(uint32_t);
+  auto walk = ahead ? k_long_tb_walk<true> : k_long_tb_walk<false>;
+  DSA_CUDA_TRY(cudaFuncSetAttribute(walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  walk<<<n_jobs, 32, smem, stream>>>(d_jobs, n_jobs, mode, fe, d_dir, d_cig_tmp, d_hits, d_win);
   DSA_CUDA_TRY(cudaGetLastError());
   ++ctx->launches;
   return DSA_OK;

@@ -43,3 +43,32 @@ def test_lane_band_and_word_edges(ctx, mode, fe):
     r = ctx.align(ctx.load_set(db, 4), ctx.load_set(qs, 4), S, 3, 1, mode=mode, free_ends=fe, pairs=pairs)
     ctx.traceback(r)
     check_traceback(r.hits(), r.cigar(), qs, db, S, 3, 1, mode, fe)
+
+
+@pytest.mark.parametrize("n", [1, 480])
+@pytest.mark.parametrize("indels", [0.0, 0.08])
+def test_long_walk_with_and_without_the_next_window(ctx, n, indels):
+    """Few hits walk with the next band's window loaded ahead, many without;
+    indels take the walk off the predicted diagonal."""
+    rng = np.random.default_rng(6200 + n)
+    q = rng.integers(0, 4, 5200).astype(np.uint8)
+    t = W.mutate(rng, q, 0.1, indels, alphabet=4)
+    Q = W.SeqSet.from_list([q])
+    T = W.SeqSet.from_list([t])
+    pairs = np.zeros(n, W.PAIR_DTYPE)
+    pairs["t_len"] = len(t)
+    res = ctx.align(ctx.load_set(T, 4), ctx.load_set(Q, 4), W.dna_matrix(2, -3), 5, 2, mode=dsa.GLOBAL, pairs=pairs)
+    ctx.traceback(res)
+    hits, cigar = res.hits(), res.cigar()
+    for h in (hits[0], hits[-1]):
+        ops = cigar[int(h["cigar_off"]):int(h["cigar_off"]) + int(h["cigar_len"])]
+        i = j = score = 0
+        for c in ops:
+            length, op = int(c) >> 4, int(c) & 15
+            if op == 0:
+                score += int(np.where(q[i:i + length] == t[j:j + length], 2, -3).sum())
+            else:
+                score -= 5 + 2 * (length - 1)
+            i += length if op in (0, 1) else 0
+            j += length if op in (0, 2) else 0
+        assert (i, j, score) == (len(q), len(t), int(h["score"]))
