@@ -267,22 +267,21 @@ constexpr int INTER_WARPS = 8;
 constexpr int INTER_ROWS = 28;         // strip rows of the packed inter-sequence kernels
 constexpr int INTER_ROWS_SHORT = 20;   // their short-strip variant (short queries)
 
-// Long-target intra-sequence (wavefront) kernel; each unit of `plan` must
-// hold one query per half (no stream switches).  Runs on `stream`
-// (allocation and release of its scratch are ordered there).
-int launch_intra_local16(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db,
-                         const PackedPlan& plan, const IntraWork& work, int o, int e, int smax,
-                         Scores out, uint32_t n_targets_out);
-// Its global / semi-global form: `plan` built with end-anchored 32-row strips.
+// Long-target intra-sequence (wavefront) kernel of global and semi-global
+// searches past the range of k_wave.cu; each unit of `plan`, built with
+// end-anchored 32-row strips, must hold one query per half (no stream
+// switches).  Runs on `stream` (allocation and release of its scratch are
+// ordered there).
 int launch_intra_glob16(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, const dsa_db* qs,
                         const PackedPlan& plan, const IntraWork& work, int mode, uint32_t fe,
                         int o, int e, int smax, int smin, Scores out, uint32_t n_targets_out);
 
 // Wavefront search of the first n_targets of the length order (k_wave.cu) on
-// `stream`: units of strips of `rows` (16 or 24) query rows as for the
+// `stream`: units of strips of `rows` (8, 16 or 24) query rows as for the
 // inter-sequence kernel (records, each unit's first strip and strip count).
 // wave_takes: queries of up to max_m against targets of up to max_n residues
-// stay inside its 16-bit range.
+// stay inside its 16-bit range.  dual (wave_dual_takes): both halves of a unit
+// follow one stream, against two targets; residues: those of the targets.
 constexpr uint32_t WAVE_LONG_TARGET = 2048;   // longer targets take up to 32 lanes
 int sum_bias(bool local, int o, int e, int smin);
 bool sum_fits(bool local, int64_t m, int64_t n, int o, int e, int smax, int smin);

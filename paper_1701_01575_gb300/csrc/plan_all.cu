@@ -385,10 +385,7 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
       DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0));
     }
     phase_begin(res, PH_INTRA, ls);
-    if (local)
-      DSA_TRY(launch_intra_local16(ctx, ls, db, ppl, xw, o, e, v.smax, out, nt));
-    else
-      DSA_TRY(launch_intra_glob16(ctx, ls, db, qs, ppl, xw, mode, fe, o, e, v.smax, v.smin, out, nt));
+    DSA_TRY(launch_intra_glob16(ctx, ls, db, qs, ppl, xw, mode, fe, o, e, v.smax, v.smin, out, nt));
     phase_end(res, PH_INTRA, ls);
   }
   if (n_long && inter) DSA_CUDA_TRY(cudaEventRecord(ctx->join_ev, ctx->side));
