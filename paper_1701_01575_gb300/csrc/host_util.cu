@@ -1,7 +1,7 @@
 // Host-side helpers (declared in host_util.cuh): host-thread loops, the
 // stable radix order used by the planners, argument checks, and the device
-// gather of saturated pairs for the exact int32 rerun (the benchmark spec (d);
-// scores stay exact, Sec. II.B.1).
+// gather of saturated pairs for the exact int32 rerun (scores stay
+// exact, Sec. II.B.1).
 #include "host_util.cuh"
 
 #include <algorithm>
