@@ -116,20 +116,36 @@ def test_short_strips_of_small_searches(ctx, lengths, mode, fe, monkeypatch):
     assert g[5].phase_cells()["inter16"] == 0
 
 
-@pytest.mark.parametrize("lengths", [[7], [100], [257], [24 * 16 + 1], [24 * 32, 5], [700, 30, 100], [1100, 16, 17, 3]])
+@pytest.mark.parametrize("lengths", [[100], [176], [300], [24 * 16 + 1], [700, 30, 100], [1100, 16, 17, 3]])
 @pytest.mark.parametrize("mode,fe", MODES)
-@pytest.mark.parametrize("n_targets", [1, 2, 150])
+@pytest.mark.parametrize("n_targets", [24000, 24001])
 def test_two_targets_a_lane(ctx, lengths, mode, fe, n_targets, monkeypatch):
-    """Queries whose streams would leave one half idle: one of them, or one much
-    longer than the rest; odd and even numbers of targets, and tails."""
+    """Queries whose streams would leave one half idle (one of them, or one much
+    longer than the rest) against enough targets that the work outlasts the
+    longest one's chain: strips of 8 (100), 16 (176) and 24 rows, even and odd
+    numbers of targets; by matrix and, in local mode, as a profile."""
     monkeypatch.setenv("DSA_LONG_THRESHOLD", "0")
     rng = np.random.default_rng(5600 + sum(lengths) + 16 * mode + fe)
     bg = W.protein_background()
     queries = W._make_set(rng, np.asarray(lengths), bg)
-    db = _db(rng, queries, bg, 2600)
-    if n_targets < db.n:
-        db = W.SeqSet.from_list([db.seq(db.n - 1 - k) for k in range(n_targets)])
-    for S, o, e in ((W.blosum62(), 11, 1), (W.blosum62(), 2, 1)):   # bytes as they are; lifted by K
+    lens = rng.integers(1, 100, n_targets)
+    lens[:4] = (100, 1, 2, 130) if sum(lengths) < 1000 else (900, 1, 500, 300)
+    assert max(lengths) * 2 * 10 > sum(lengths) * 12
+    rows = 8 if max(lengths) <= 100 else 24
+    assert (max(lengths) // rows) * int(lens.sum()) * 4 >= 3 * int(lens.max()) * 152 * 512
+    db = W._make_set(rng, lens, bg)
+    for k, n in enumerate(lengths):   # a mutated piece of each query inside a target
+        at = int(db.offsets[3 + 5 * k])
+        room = int(db.offsets[4 + 5 * k]) - at
+        piece = W.mutate(rng, queries.seq(k), 0.2, 0.02, alphabet=len(bg))[:room]
+        db.codes[at:at + len(piece)] = piece
+    S = W.blosum62()
+    for o, e in ((11, 1), (2, 1)):   # the profile's bytes as they are; lifted to 0 or more
         g = gpu_all(ctx, queries, db, S, o, e, mode=mode, fe=fe)
         assert_same(g[:3], oracle_all(queries, db, S, o, e, mode, fe), f"{lengths} mode={mode} o={o}")
         assert g[5].phase_cells()["inter16"] == 0
+    if mode == dsa.LOCAL:
+        d, q = ctx.load_set(db, 24), ctx.load_set(queries, 24)
+        a = ctx.align(d, q, S, 11, 1, top_k=50)
+        b = ctx.align_pssm(d, q, S[queries.codes].astype(np.int8), 11, 1, top_k=50)
+        assert (a.hits() == b.hits()).all()
