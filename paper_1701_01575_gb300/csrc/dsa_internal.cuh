@@ -19,6 +19,11 @@ namespace dsa {
 constexpr int32_t NEG32 = INT32_MIN / 4;
 constexpr int32_t NEG16 = -16384;
 
+// Dynamic shared memory.  A kernel's limit (cudaFuncSetAttribute) belongs to the
+// device and so to every thread that launches the kernel there; a launch sets it
+// to what the largest alphabet needs, not to its own need, so that no thread
+// takes it back between another's setting and its launch.
+
 // Launch / layout constants.
 constexpr int GROUP = 32;          // targets per interleaved group (one warp)
 constexpr int CHUNK = 16;          // residues per 16-byte interleaved word

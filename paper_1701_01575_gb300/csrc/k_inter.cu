@@ -793,6 +793,12 @@ __global__ void k_strip_profile(const uint8_t* __restrict__ qcodes,
 
 int inter_blocks_per_sm() { return 2; }
 
+// Profile replicas (two buffers), the parked columns and the boundary ring.
+static size_t inter_smem(int residues, int rows) {
+  return 2ull * NCOPY * replica_stride(residues) + (size_t)rows * NT * sizeof(uint32_t) +
+         (size_t)RING * 4 * NT * sizeof(uint2);
+}
+
 int launch_strip_profile(dsa_ctx* ctx, const dsa_db* qs, const int8_t* d_matrix,
                          const int8_t* d_pssm, int A, int o, const PackedPlan& plan,
                          bool anchored, int tpad, bool sum) {
@@ -836,8 +842,7 @@ int launch_inter_local16(dsa_ctx* ctx, const dsa_db* db, const PackedPlan& plan,
   A.o_score = out.score; A.o_qend = out.q_end; A.o_tend = out.t_end; A.o_flag = out.flag;
   A.n_out_t = n_targets_out;
   A.status = ctx->d_status;
-  const size_t smem = 2ull * NCOPY * replica_stride(plan.R) + 2ull * plan.rows * NT * sizeof(int16_t) +
-                      (size_t)RING * 4 * NT * sizeof(uint2);
+  const size_t smem = inter_smem(plan.R, plan.rows);
   auto kern = plan.rows == INTER_ROWS_SHORT
                   ? (sum ? k_inter_local16<INTER_ROWS_SHORT, true> : k_inter_local16<INTER_ROWS_SHORT, false>)
                   : (sum ? k_inter_local16<INTER_ROWS, true> : k_inter_local16<INTER_ROWS, false>);
@@ -847,11 +852,14 @@ int launch_inter_local16(dsa_ctx* ctx, const dsa_db* db, const PackedPlan& plan,
     return DSA_ERR_INVALID_ARG;
   }
   // the attribute belongs to the current device: set it on every launch (cheap)
-  DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  DSA_CUDA_TRY(cudaMemsetAsync(ctx->d_counters, 0, sizeof(uint32_t), ctx->stream));
-  kern<<<grid, NT, smem, ctx->stream>>>(A);
-  ++ctx->launches;
-  cudaError_t err = cudaGetLastError();
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)inter_smem(MAX_ALPHABET + 1, plan.rows));
+  if (err == cudaSuccess) err = cudaMemsetAsync(ctx->d_counters, 0, sizeof(uint32_t), ctx->stream);
+  if (err == cudaSuccess) {
+    kern<<<grid, NT, smem, ctx->stream>>>(A);
+    ++ctx->launches;
+    err = cudaGetLastError();
+  }
   ctx->release(scr, scr_bytes);
   if (err != cudaSuccess) {
     set_error("k_inter_local16 launch: %s", cudaGetErrorString(err));
@@ -891,8 +899,7 @@ int launch_inter_glob16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const 
   A.o_score = out.score; A.o_qend = out.q_end; A.o_tend = out.t_end; A.o_flag = out.flag;
   A.n_out_t = n_targets_out;
   A.status = ctx->d_status;
-  const size_t smem = 2ull * NCOPY * replica_stride(plan.R) + (size_t)plan.rows * NT * sizeof(uint32_t) +
-                      (size_t)RING * 4 * NT * sizeof(uint2);
+  const size_t smem = inter_smem(plan.R, plan.rows);
   const bool sg = mode == DSA_SEMIGLOBAL;
   const bool tb = sg && (fe & DSA_FREE_T_BEGIN), te = sg && (fe & DSA_FREE_T_END);
   auto pick = [&](auto w) {
@@ -910,11 +917,14 @@ int launch_inter_glob16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const 
     set_error("strip height %d has no kernel", plan.rows);
     return DSA_ERR_INVALID_ARG;
   }
-  DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  DSA_CUDA_TRY(cudaMemsetAsync(ctx->d_counters, 0, sizeof(uint32_t), ctx->stream));
-  kern<<<grid, NT, smem, ctx->stream>>>(A, G);
-  ++ctx->launches;
-  cudaError_t err = cudaGetLastError();
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)inter_smem(MAX_ALPHABET + 1, plan.rows));
+  if (err == cudaSuccess) err = cudaMemsetAsync(ctx->d_counters, 0, sizeof(uint32_t), ctx->stream);
+  if (err == cudaSuccess) {
+    kern<<<grid, NT, smem, ctx->stream>>>(A, G);
+    ++ctx->launches;
+    err = cudaGetLastError();
+  }
   ctx->release(scr, scr_bytes);
   if (err != cudaSuccess) {
     set_error("k_inter_glob16 launch: %s", cudaGetErrorString(err));

@@ -346,14 +346,14 @@ extern "C" int dsa_score_pairs_noalloc(const uint8_t* d_q_codes, const uint64_t*
   // lanes a pair as it takes to keep them busy (8 when pairs abound: the fewer
   // lanes, the fewer steps a pair spends filling its wavefront)
   const bool local = mode == DSA_LOCAL;
-  const size_t smem = pair_wave_table_bytes(alphabet_size) +
-                      (size_t)WAVE_WARPS * pair_wave_warp_bytes(alphabet_size, local);
+  const size_t smem = pair_wave_smem(alphabet_size, local);
   const bool small = smem <= 50 * 1024;
   auto kern = local ? (small ? k_noalloc_wave<true, 4> : k_noalloc_wave<true, 2>)
                     : (small ? k_noalloc_wave<false, 4> : k_noalloc_wave<false, 2>);
   int sms = 0, per_sm = 0;
   DSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)pair_wave_smem(MAX_ALPHABET, local)));
   DSA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WAVE_WARPS * 32, smem));
   const uint64_t resident = (uint64_t)std::max(1, per_sm) * sms * WAVE_WARPS;   // warps
   NoallocArgs N{d_q_codes, d_q_offsets, n_queries, d_t_codes, d_t_offsets, n_targets, d_pairs, n_pairs,

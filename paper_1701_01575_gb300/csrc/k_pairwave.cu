@@ -134,7 +134,7 @@ int launch_pair_wave(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int
   K.n_items = (uint32_t)items;
   K.T = 32767 - std::max(0, smax);
   K.out = out;
-  const size_t smem = pair_wave_table_bytes(A) + (size_t)WAVE_WARPS * pair_wave_warp_bytes(A, local);
+  const size_t smem = pair_wave_smem(A, local);
   // small alphabets: registers bound the warps per SM (4 CTAs); larger ones:
   // the profiles do (2 CTAs of 4 x 28 KB for proteins)
   auto kern = pair_wave_wide(A) ? (lsum    ? k_pair_wave<WAVE_LOCAL_SUM, true, 4>
@@ -143,7 +143,8 @@ int launch_pair_wave(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int
                                 : (lsum    ? k_pair_wave<WAVE_LOCAL_SUM, false, 2>
                                    : local ? k_pair_wave<WAVE_LOCAL, false, 2>
                                            : k_pair_wave<WAVE_GLOBAL, false, 2>);
-  DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)pair_wave_smem(MAX_ALPHABET, local)));
   int per_sm = 0;
   DSA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WAVE_WARPS * 32, smem));
   const uint64_t grid = std::min<uint64_t>((items + WAVE_WARPS - 1) / WAVE_WARPS,

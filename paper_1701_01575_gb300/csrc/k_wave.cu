@@ -680,8 +680,11 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
     return DSA_ERR_INVALID_ARG;
   }
   const int halves = dual ? 2 : 1;   // targets per lane group
-  const size_t smem = (size_t)(A + 1) * (dual ? 32 * rows : rows / 4 * PLANE) + (size_t)rows * NT * 4;
-  DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  auto smem_of = [&](int letters) {
+    return (size_t)(letters + 1) * (dual ? 32 * rows : rows / 4 * PLANE) + (size_t)rows * NT * 4;
+  };
+  const size_t smem = smem_of(A);
+  DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(MAX_ALPHABET)));
   int per_sm = 0;
   DSA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
   const uint32_t ctas = (uint32_t)std::max(1, per_sm) * ctx->sm_count;

@@ -113,6 +113,10 @@ __host__ __device__ inline uint32_t pair_wave_warp_bytes(int A, bool local) {
   const int R = A <= WAVE_WIDE_ALPHABET ? 20 : 16;
   return (uint32_t)(A + 1) * wave_residue(R) + (local ? 2u * R * 32u * 2u : 0u);
 }
+// of a CTA's warps, and the most any alphabet takes
+__host__ __device__ inline uint32_t pair_wave_smem(int A, bool local) {
+  return pair_wave_table_bytes(A) + (uint32_t)WAVE_WARPS * pair_wave_warp_bytes(A, local);
+}
 // offset of the parked columns behind the profile
 __host__ __device__ inline uint32_t pair_wave_park_offset(int A) {
   return (uint32_t)(A + 1) * wave_residue(A <= WAVE_WIDE_ALPHABET ? 20 : 16);
