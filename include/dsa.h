@@ -317,8 +317,9 @@ int dsa_server_destroy(dsa_server* srv);
  * inside the library (one per device that loads the library, held until the
  * process exits).  `max_t_len`, an upper bound on every pair's t_len, must
  * be at most 32768; larger values return DSA_ERR_INVALID_ARG.  The first
- * call on each device looks up that array's device address (with the device
- * current); make that first call before any stream capture.  Every call
+ * call on each device, in whatever mode, looks up that array's device address
+ * and loads the kernels of every mode (with the device current); make that
+ * first call before any stream capture.  Every call
  * shares the array and no part of it needs to start at zero (each pair
  * writes its boundary row before reading it), so calls whose kernels overlap
  * on the GPU race on it: order them on one stream or synchronize between

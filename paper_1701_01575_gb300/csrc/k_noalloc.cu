@@ -278,11 +278,26 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) k_noalloc_pairs(
 }
 
 // Device address of g_noalloc_scratch per device, looked up once per device
-// (with that device current) on the first call made on it.  The address
-// belongs to the device's primary context: it does not survive a
-// cudaDeviceReset of that device (the header says so).
+// (with that device current) on the first call made on it, which also loads every
+// kernel a later call may take: a kernel is otherwise loaded, into device memory,
+// by the first call in its mode.  The address belongs to the device's primary
+// context: it does not survive a cudaDeviceReset of that device (the header says
+// so).
 std::mutex g_noalloc_mu;
 void* g_noalloc_ptr[64] = {};
+
+using WaveKernel = void (*)(const NoallocArgs);
+// by mode and by whether 4 CTAs' profiles fit an SM
+constexpr WaveKernel WAVE_KERNELS[2][2] = {{k_noalloc_wave<false, 2>, k_noalloc_wave<false, 4>},
+                                           {k_noalloc_wave<true, 2>, k_noalloc_wave<true, 4>}};
+cudaError_t load_kernels() {
+  cudaFuncAttributes a;
+  cudaError_t err = cudaFuncGetAttributes(&a, k_noalloc_pairs);
+  for (const auto& of_mode : WAVE_KERNELS)
+    for (const WaveKernel k : of_mode)
+      if (err == cudaSuccess) err = cudaFuncGetAttributes(&a, k);
+  return err;
+}
 
 }  // namespace
 }  // namespace dsa
@@ -327,6 +342,7 @@ extern "C" int dsa_score_pairs_noalloc(const uint8_t* d_q_codes, const uint64_t*
         set_error("cudaGetSymbolAddress(g_noalloc_scratch) failed: %s", cudaGetErrorString(err));
         return DSA_ERR_CUDA;
       }
+      DSA_CUDA_TRY(load_kernels());
       g_noalloc_ptr[dev] = p;
     }
     scratch = g_noalloc_ptr[dev];
@@ -347,9 +363,7 @@ extern "C" int dsa_score_pairs_noalloc(const uint8_t* d_q_codes, const uint64_t*
   // lanes, the fewer steps a pair spends filling its wavefront)
   const bool local = mode == DSA_LOCAL;
   const size_t smem = pair_wave_smem(alphabet_size, local);
-  const bool small = smem <= 50 * 1024;
-  auto kern = local ? (small ? k_noalloc_wave<true, 4> : k_noalloc_wave<true, 2>)
-                    : (small ? k_noalloc_wave<false, 4> : k_noalloc_wave<false, 2>);
+  const WaveKernel kern = WAVE_KERNELS[local][smem <= 50 * 1024];
   int sms = 0, per_sm = 0;
   DSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   DSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
