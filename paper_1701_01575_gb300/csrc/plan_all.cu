@@ -225,6 +225,23 @@ bool wave_dual(const dsa_db* qs, const Validated& v, bool local, uint32_t max_n,
   return 2ull * qs->max_len * 10 > sum * 12;
 }
 
+// Work on the side stream, joined to the context's stream on every way out of a
+// call: the buffers it uses are given back in the order of the context's stream,
+// so a call that fails after the fork (an allocation past the budget) must not
+// leave it running beside them.
+struct SideJoin {
+  dsa_ctx* ctx;
+  bool open = false;
+  int close() {
+    if (!open) return DSA_OK;
+    open = false;
+    DSA_CUDA_TRY(cudaEventRecord(ctx->join_ev, ctx->side));
+    DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->stream, ctx->join_ev, 0));
+    return DSA_OK;
+  }
+  ~SideJoin() { close(); }
+};
+
 // Packed score pass (int16x2).  Targets of groups longer than `long_thr` go
 // to the wavefront kernel, the rest to the inter-sequence kernel; with both,
 // the wavefronts run on the side stream.  The results do not depend on
@@ -334,10 +351,12 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
   // two kernels write disjoint targets' results
   cudaStream_t ls = ctx->stream;
   DevBuf d_pmeta, d_pbase, d_pns, d_pprof, d_long, d_litems;
+  SideJoin join{ctx};   // before the buffers above and the caller's scores are given back
   if (n_long && inter) {
     ls = ctx->side;
     DSA_CUDA_TRY(cudaEventRecord(ctx->fork_ev, ctx->stream));
     DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0));
+    join.open = true;
   }
   if (wave) {
     bool dual = wave_dual(qs, v, local, db->h_glen[0], o, e);
@@ -388,7 +407,6 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
     DSA_TRY(launch_intra_glob16(ctx, ls, db, qs, ppl, xw, mode, fe, o, e, v.smax, v.smin, out, nt));
     phase_end(res, PH_INTRA, ls);
   }
-  if (n_long && inter) DSA_CUDA_TRY(cudaEventRecord(ctx->join_ev, ctx->side));
   if (inter) {
     DevBuf d_smeta, d_sbase, d_sns, d_sprof, d_items;
     DSA_TRY(upload(ctx, d_smeta, smeta));
@@ -412,8 +430,7 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
       DSA_TRY(launch_inter_glob16(ctx, db, qs, spl, iw, mode, fe, o, e, v.smax, v.smin, sum, out, nt));
     phase_end(res, PH_INTER);
   }
-  if (n_long && inter) DSA_CUDA_TRY(cudaStreamWaitEvent(ctx->stream, ctx->join_ev, 0));
-  return DSA_OK;
+  return join.close();
 }
 
 // Targets longer than this go to the wavefronts when nothing is tuned or
