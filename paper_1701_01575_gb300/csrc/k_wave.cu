@@ -94,9 +94,9 @@ struct WaveArgs {
   uint32_t pad_word;               // profile word (DUAL: 4 bytes) of strips past a unit's end
   const Segment* segs;
   uint32_t n_segs, n_items;
-  uint32_t* counter;
+  unsigned long long* counter;     // CTAs started << 32 | items taken
   uint2* scratch;
-  uint64_t warp_cols;              // boundary cells per warp
+  const uint64_t* slot;            // first boundary cell of the k-th CTA to start
   Scores out;
   uint32_t n_out_t;
 };
@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
   constexpr int MIN_SLOTS = DUAL ? 16 : 8;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ Segment s_seg;
-  __shared__ uint32_t s_tile;
+  __shared__ uint32_t s_tile, s_row;
+  __shared__ uint64_t s_slot;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // parked columns: local [half][8 rows of 16 bits][thread], others packed
   // [row][thread]
@@ -126,13 +127,14 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
   const bool qb_free = sg && (A.fe & DSA_FREE_Q_BEGIN), qe_free = sg && (A.fe & DSA_FREE_Q_END);
   const bool tb_free = sg && (A.fe & DSA_FREE_T_BEGIN), te_free = sg && (A.fe & DSA_FREE_T_END);
   auto row0 = [&](int j) { return (j == 0 || tb_free) ? 0 : -(o + (j - 1) * e); };
-  uint2* const scr_warp = A.scratch + (uint64_t)(blockIdx.x * NW + warp) * A.warp_cols;
   uint32_t held = NONE;               // first strip and group size of the profile in place
 
-  for (;;) {
+  for (bool first = true;; first = false) {
     __syncthreads();
     if (tid == 0) {
-      const uint32_t item = atomicAdd(A.counter, 1u);
+      const unsigned long long got = atomicAdd(A.counter, first ? (1ull << 32) + 1 : 1ull);
+      const uint32_t item = (uint32_t)got;
+      if (first) s_slot = A.slot[got >> 32];
       if (item >= A.n_items) {
         s_tile = NONE;
       } else {
@@ -144,6 +146,8 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
         }
         s_seg = A.segs[lo];
         s_tile = item - s_seg.item0;
+        // its longest target
+        s_row = A.tlen[A.perm[s_seg.first + s_tile * (s_seg.warps * 32 / s_seg.G) * (DUAL ? 2 : 1)]];
       }
     }
     __syncthreads();
@@ -177,7 +181,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
       nmin = min(nmin, __shfl_xor_sync(FULL, nmin, w));
     }
     const uint32_t sh = 8u * (uint32_t)((uintptr_t)(t - k) & 3), sh2 = 8u * (uint32_t)((uintptr_t)(t2 - k) & 3);
-    uint2* const scr = scr_warp + (uint64_t)(lane / G) * nmax;
+    uint2* const scr = A.scratch + s_slot + (uint64_t)(warp * (32 / G) + lane / G) * s_row;
     const int steps = nmax + G - 1;
     const int nb = ((int)ns + G - 1) / G;
 
@@ -705,7 +709,6 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   const uint64_t limit = strip_cols / slots * 3 / 5;
   std::vector<Segment> segs;
   size_t n_first = 0;
-  uint64_t cols = 0;   // boundary cells of a warp
   std::vector<uint32_t> next(ns.size(), 0);   // the unit's targets dealt so far
   for (int most = 32; most >= FEW_LANES; most /= 2) {
     for (uint32_t u = 0; u < ns.size(); ++u) {
@@ -725,7 +728,6 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
       while (G < 32 && (uint32_t)G < ns[u] && (G < most || n_targets / halves * ns.size() * G < slots)) G *= 2;
       segs.push_back({u, first, count, 0, G, NW});
       n_first += most == 32;
-      if (ns[u] > (uint32_t)G) cols = std::max<uint64_t>(cols, 32ull / G * db->h_len[db->h_perm[first]]);
     }
   }
   auto items_of = [&](size_t from, size_t to, int warps) {
@@ -752,6 +754,32 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   }
   const unsigned grid = std::min<uint32_t>(items, ctas);
 
+  // Boundary rows: an item takes a row of its longest target per lane group with
+  // a target, none if its unit fits one band.  The k-th CTA to start takes its
+  // first item in the same step, so never one before item k: its slot holds the
+  // largest of the items from there on.  (Slots of every warp by the longest
+  // target of all: one query of 2,000 against 100 targets of a million took 3.2
+  // GB, now 0.4.)
+  auto boundary = [&](const Segment& s, uint32_t tile) -> uint64_t {
+    if (ns[s.unit] <= (uint32_t)s.G) return 0;
+    const uint32_t per = s.warps * 32 / s.G * halves, at = tile * per;
+    return (uint64_t)((std::min(per, s.count - at) + halves - 1) / halves) * db->h_len[db->h_perm[s.first + at]];
+  };
+  std::vector<uint64_t> slot(grid, 0);
+  uint64_t largest = 0;
+  for (uint32_t k = (uint32_t)segs.size(), end = items; k-- > 0; end = segs[k].item0) {
+    const Segment& s = segs[k];   // needs fall along a segment
+    if (end > grid) largest = std::max(largest, boundary(s, std::max(s.item0, grid) - s.item0));
+    for (uint32_t x = std::min(end, grid); x-- > s.item0;) slot[x] = largest = std::max(largest, boundary(s, x - s.item0));
+  }
+  uint64_t b_scr = 0;
+  for (uint64_t& s : slot) {
+    const uint64_t cells = s;
+    s = b_scr;
+    b_scr += cells;
+  }
+  b_scr *= sizeof(uint2);
+
   WaveArgs W{};
   W.tcodes = db->d_codes; W.toff = db->d_off; W.tlen = db->d_len; W.perm = db->d_perm;
   W.qlen = qs->d_len;
@@ -775,17 +803,19 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   const int pw = local ? P.none : P.pad_row;
   W.pad_word = dual ? (uint32_t)pw * 0x01010101u : form == LOCAL_WRAP ? (uint32_t)(pw & 0xFFFF) * 0x10001u : ((uint32_t)pw << 16) + (uint32_t)pw;
 
-  // one upload: segments, strip records, each unit's first strip and strip count
+  // one upload: segments, strip records, each unit's first strip and strip
+  // count, the CTAs' slots
   const size_t b_seg = (segs.size() * sizeof(Segment) + 15) & ~(size_t)15;
   const size_t b_meta = (meta.size() * sizeof(StripMeta) + 15) & ~(size_t)15;
   const size_t b_u = (ns.size() * 4 + 15) & ~(size_t)15;
-  std::vector<uint8_t> host(b_seg + b_meta + 2 * b_u);
+  const size_t b_slot = (grid * 8 + 15) & ~(size_t)15;
+  std::vector<uint8_t> host(b_seg + b_meta + 2 * b_u + b_slot);
   memcpy(host.data(), segs.data(), segs.size() * sizeof(Segment));
   memcpy(host.data() + b_seg, meta.data(), meta.size() * sizeof(StripMeta));
   memcpy(host.data() + b_seg + b_meta, sbase.data(), sbase.size() * 4);
   memcpy(host.data() + b_seg + b_meta + b_u, ns.data(), ns.size() * 4);
+  memcpy(host.data() + b_seg + b_meta + 2 * b_u, slot.data(), grid * 8);
   const size_t b_prof = ((size_t)P.n_strips * (A + 1) * rows * (dual ? 1 : 4) + 15) & ~(size_t)15;
-  const size_t b_scr = (size_t)grid * NW * cols * sizeof(uint2);
   void* buf = nullptr;
   const size_t b_all = host.size() + b_prof + b_scr + 16;
   DSA_TRY(ctx->alloc(&buf, b_all, stream));
@@ -797,13 +827,13 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   W.nstrips = reinterpret_cast<const uint32_t*>(d + b_seg + b_meta + b_u);
   W.prof = P.prof = reinterpret_cast<uint32_t*>(d + host.size());
   W.scratch = reinterpret_cast<uint2*>(d + host.size() + b_prof);
-  W.warp_cols = cols;
+  W.slot = reinterpret_cast<const uint64_t*>(d + b_seg + b_meta + 2 * b_u);
   W.n_segs = (uint32_t)segs.size();
   W.n_items = items;
-  W.counter = ctx->d_counters + 2;
+  W.counter = reinterpret_cast<unsigned long long*>(ctx->d_counters + 4);
   W.out = out;
   W.n_out_t = db->n;
-  if (err == cudaSuccess) err = cudaMemsetAsync(W.counter, 0, sizeof(uint32_t), stream);
+  if (err == cudaSuccess) err = cudaMemsetAsync(W.counter, 0, sizeof(*W.counter), stream);
   if (err == cudaSuccess) {
     const uint64_t words = (uint64_t)P.n_strips * (A + 1) * rows;
     k_wave_profile<<<(unsigned)std::min<uint64_t>((words + 255) / 256, (uint64_t)ctx->sm_count * 8), 256, 0,

@@ -97,8 +97,10 @@ size_t dsa_server::estimate(const std::vector<Req*>& batch) const {
     const uint64_t nt = db->n;
     const uint64_t glen = db->max_len;
     bytes += nq * nt * 13;                                           // dense scores
-    // boundary rows of the packed kernel: grid = min(items, 2 CTAs per SM),
-    // items = units (<= query pairs) x blocks of 8 groups
+    // boundary rows of the inter-sequence kernel: grid = min(items, 2 CTAs per
+    // SM), items = units (<= query pairs) x blocks of 8 groups.  The wavefronts
+    // take no more: a row per unit and target (or two targets), and at most
+    // 2 x 8 x 32 lanes' groups per SM
     const uint64_t blocks = (db->n_groups + dsa::INTER_WARPS - 1) / dsa::INTER_WARPS;
     const uint64_t grid = std::min<uint64_t>((nq + 1) / 2 * blocks, (uint64_t)sm_count * 2);
     bytes += grid * dsa::INTER_WARPS * 32 * glen * 8;

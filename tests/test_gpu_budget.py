@@ -46,3 +46,38 @@ def test_call_refused_beside_running_wavefronts(monkeypatch):
             ctx.align(d, q, S, 11, 1, top_k=40)
         assert err.value.code == dsa.ERR_OVER_BUDGET and ctx.mem_in_use() == held
     ctx.sync()
+
+
+@pytest.mark.parametrize("lens,budget", [([60_000] * 100, 80), ([300_000] + [200] * 3000, 200)])
+def test_boundary_rows_follow_the_targets(lens, budget, monkeypatch):
+    """Wavefronts of several bands: a few long targets, and one very long one
+    among many short, take about a boundary row per target, not one of the
+    longest for every warp of the chip."""
+    monkeypatch.setenv("DSA_AUTOTUNE", "off")
+    monkeypatch.setenv("DSA_LONG_THRESHOLD", "0")
+    rng = np.random.default_rng(7300 + budget)
+    bg = W.protein_background()
+    qs = W._make_set(rng, np.array([2000]), bg)
+    db = W._make_set(rng, np.array(lens), bg)
+    S = W.blosum62()
+    h = _hits(dsa.Context(0, mem_budget=budget * MB), db, qs, S, 11, 1, 24)
+    assert_same((h["score"].reshape(1, -1), h["q_end"].reshape(1, -1), h["t_end"].reshape(1, -1)),
+                oracle_all(qs, db, S, 11, 1), f"budget {budget} MB")
+
+
+@pytest.mark.parametrize("mode", [dsa.LOCAL, dsa.GLOBAL, dsa.SEMIGLOBAL])
+def test_more_items_than_slots(mode, monkeypatch):
+    """Units of several bands whose items outnumber the resident CTAs, long
+    targets in every unit: each CTA's boundary rows hold whatever it is dealt."""
+    monkeypatch.setenv("DSA_AUTOTUNE", "off")
+    rng = np.random.default_rng(7400 + mode)
+    bg = W.protein_background()
+    qs = W._make_set(rng, rng.integers(400, 1000, 24), bg)
+    db = W._make_set(rng, np.concatenate([rng.integers(2000, 5000, 200), rng.integers(20, 700, 8000)]), bg)
+    S = W.blosum62()
+    ctx = dsa.Context(0)
+    got = []
+    for thr in ("0", "1000000"):
+        monkeypatch.setenv("DSA_LONG_THRESHOLD", thr)
+        got.append(_hits(ctx, db, qs, S, 11, 1, 24, mode=mode))
+    assert (got[0] == got[1]).all()
