@@ -461,6 +461,37 @@ uint32_t model_threshold(const dsa_db* db, const dsa_db* qs, const Validated& v,
   return left * 4 < db->n_res ? 0 : t;
 }
 
+// A threshold whose inter-sequence boundary rows (8 bytes per thread and column
+// of its longest target) fit: past PLAIN_THRESHOLD columns they may take half of
+// what the context can still allocate, so that a long threshold, faster where
+// targets abound, is no reason to refuse a call (contigs of up to a million
+// residues would take 600 GB; 4,096 columns take at most 2.6).
+constexpr uint32_t PLAIN_THRESHOLD = 4096;
+uint32_t fit_threshold(dsa_ctx* ctx, const dsa_db* db, uint32_t nq, uint32_t thr) {
+  uint32_t g = 0;
+  while (g < db->n_groups && db->h_glen[g] > thr) ++g;
+  if (g == db->n_groups || db->h_glen[g] <= PLAIN_THRESHOLD) return thr;
+  const uint64_t blocks = (db->n_groups - g + INTER_WARPS - 1) / INTER_WARPS;
+  const uint64_t ctas = std::min<uint64_t>((nq + 1ull) / 2 * blocks, (uint64_t)inter_blocks_per_sm() * ctx->sm_count);
+  uint64_t room = 0;
+  {
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    if (ctx->budget) room = ctx->budget > ctx->in_use ? ctx->budget - ctx->in_use : 0;
+  }
+  if (!ctx->budget) {   // free memory, and what the pool keeps mapped for itself
+    size_t free = 0, total = 0;
+    uint64_t held = 0, used = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess ||
+        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+      cudaGetLastError();
+    room = free + (held > used ? held - used : 0);
+  }
+  const uint64_t fits = room / 2 / (ctas * INTER_WARPS * 32 * sizeof(uint2));
+  if (db->h_glen[g] <= fits) return thr;
+  return (uint32_t)std::max<uint64_t>(PLAIN_THRESHOLD, fits);
+}
+
 // Strip rows forced by DSA_INTER_ROWS (0: let the tuner choose).
 int forced_rows() {
   if (const char* env = getenv("DSA_INTER_ROWS")) {
@@ -485,7 +516,8 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   const char* mode_env = getenv("DSA_AUTOTUNE");
   const std::string tmode = mode_env ? mode_env : "cache";
   const int rows_default = rows_forced ? rows_forced : INTER_ROWS;
-  const uint32_t thr_default = thr_env ? thr_forced : model_threshold(db, qs, v, local, o, e);
+  auto fit = [&](uint32_t thr) { return fit_threshold(ctx, db, qs->n, thr); };
+  const uint32_t thr_default = thr_env ? thr_forced : fit(model_threshold(db, qs, v, local, o, e));
   if (tmode == "off" || (rows_forced && thr_env))
     return run(res, thr_default, rows_default);
   // workload shape key: GPU, driver, mode, alphabet, and log2 bins of the
@@ -512,7 +544,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
     auto it_r = t.cache.find(key_rows);
     auto it_t = t.cache.find(key_thr);
     if (tmode != "retune" && it_r != t.cache.end() && it_t != t.cache.end())
-      return run(res, thr_env ? thr_forced : it_t->second,
+      return run(res, thr_env ? thr_forced : fit(it_t->second),
                  rows_forced ? rows_forced : (int)it_r->second);
   }
   if (!ctx->tune)   // contexts that must not spend calls on tuning (serving workers)
@@ -572,6 +604,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
           continue;
         }
         last_g = g;
+        if (fit(thr) != thr) break;
         const double ms = measure(thr, best_rows);
         if (ms < 0.97 * best_ms) {
           best_ms = ms;

@@ -81,3 +81,18 @@ def test_more_items_than_slots(mode, monkeypatch):
         monkeypatch.setenv("DSA_LONG_THRESHOLD", thr)
         got.append(_hits(ctx, db, qs, S, 11, 1, 24, mode=mode))
     assert (got[0] == got[1]).all()
+
+
+def test_threshold_fits_the_budget(monkeypatch):
+    """Many short queries against long targets, where the model would keep
+    targets of some 13,000 residues on the inter-sequence kernel: 8 GB of
+    boundary rows, which a small budget does not hold."""
+    monkeypatch.setenv("DSA_AUTOTUNE", "off")
+    monkeypatch.delenv("DSA_LONG_THRESHOLD", raising=False)
+    rng = np.random.default_rng(7500)
+    bg = np.full(4, 0.25)
+    qs = W._make_set(rng, np.full(512, 60), bg)
+    db = W._make_set(rng, rng.integers(2000, 20_000, 1500), bg)
+    S = W.dna_matrix(2, -3)
+    got = [_hits(dsa.Context(0, mem_budget=b), db, qs, S, 5, 2, 4, top_k=5) for b in (3 << 30, 0)]
+    assert (got[0] == got[1]).all()
