@@ -41,6 +41,14 @@
 // Lanes start one after another: before a target's first column they hold the
 // padding residue, under which a strip's column-0 state is a fixed point.
 //
+// Boundary rows.  Lane 0 reads the band above one column ahead of its use.  A
+// global step of 8 or 16 rows is shorter than that load takes, and the compiler
+// waits for it in every step (776 of 1,440 cycles, long scoreboard), so there
+// lanes 0 to 3 load the next block's four columns a block ahead and hand them
+// over by two shuffles a step: 24 queries of 175 against 20,000 targets, global,
+// 12.2 -> 6.3 ms, 7 of 90-1,100 against 50,000 with 16 rows forced 19.6 -> 6.9.
+// Steps of 24 rows and local ones are long enough (0 to 7% slower that way).
+//
 // End cells.  Local: a column maximum above the best of the strip's query so
 // far (as known to the lane: shared along the query's lanes every 32 steps)
 // parks the column in shared memory; per band the lanes of a query are
@@ -110,6 +118,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
   constexpr uint32_t BIAS2 = 0x80008000u;
   constexpr int RS = DUAL ? 32 * R : R / 4 * PLANE;   // profile bytes per residue
   constexpr int MIN_SLOTS = DUAL ? 16 : 8;
+  constexpr bool BLOCK_IN = !LOCAL && R < 24;         // see "Boundary rows"
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ Segment s_seg;
   __shared__ uint32_t s_tile, s_row;
@@ -280,8 +289,9 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
       };
       if (LOCAL) set_thr();
       const bool hand = b + 1 < nb && k == G - 1;   // the band's bottom row is read again
-      uint2 in = make_uint2(0, 0);
-      if (b > 0 && k == 0 && n > 0) in = scr[0];
+      uint2 in = make_uint2(0, 0), in_nxt = in;
+      if (b > 0 && k < (BLOCK_IN ? min(4, n) : min(1, n))) in_nxt = scr[k];
+      if (!BLOCK_IN) in = in_nxt;
 
       // residues of 4 steps, one block ahead: two aligned words, or (edge) the
       // four bytes with the padding residue outside the target
@@ -302,6 +312,10 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
       for (int s0 = 0; s0 < steps; s0 += 4) {
         const uint32_t r4 = edge_at(s0) ? nxt.x : __funnelshift_r(nxt.x, nxt.y, sh);
         nxt = fetch(s0 + 4, t, n);
+        if (BLOCK_IN) {
+          in = in_nxt;
+          if (b > 0 && k < 4 && s0 + 4 + k < n) in_nxt = scr[s0 + 4 + k];
+        }
         uint32_t r4b = 0;
         if (DUAL) {
           r4b = edge_at(s0) ? nxt2.x : __funnelshift_r(nxt2.x, nxt2.y, sh2);
@@ -328,7 +342,14 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
           ++j;
           uint32_t upH = __shfl_up_sync(FULL, sendH, 1);
           uint32_t upF = __shfl_up_sync(FULL, sendF, 1);
-          if (b > 0 && k == 0) {
+          if (BLOCK_IN) {
+            if (b > 0) {
+              const int from = (lane & ~(G - 1)) + y;
+              const uint32_t h = __shfl_sync(FULL, in.x, from), f = __shfl_sync(FULL, in.y, from);
+              upH = k == 0 ? h : upH;
+              upF = k == 0 ? f : upF;
+            }
+          } else if (b > 0 && k == 0) {
             upH = in.x;
             upF = in.y;
             if (j < n) in = scr[j];
