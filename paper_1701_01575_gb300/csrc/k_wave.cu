@@ -109,6 +109,9 @@ struct WaveArgs {
   uint32_t n_out_t;
 };
 
+// Cells of a boundary row: whole 128-byte lines, none shared by two lane groups.
+__host__ __device__ inline uint32_t boundary_row(uint32_t n) { return (n + 15) & ~15u; }
+
 template <int FORM, int R, bool DUAL>
 __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
   static_assert(!DUAL || FORM != LOCAL_WRAP, "two targets a lane: summed forms");
@@ -121,7 +124,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
   constexpr bool BLOCK_IN = !LOCAL && R < 24;         // see "Boundary rows"
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ Segment s_seg;
-  __shared__ uint32_t s_tile, s_row;
+  __shared__ uint32_t s_tile;
   __shared__ uint64_t s_slot;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // parked columns: local [half][8 rows of 16 bits][thread], others packed
@@ -136,6 +139,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
   const bool qb_free = sg && (A.fe & DSA_FREE_Q_BEGIN), qe_free = sg && (A.fe & DSA_FREE_Q_END);
   const bool tb_free = sg && (A.fe & DSA_FREE_T_BEGIN), te_free = sg && (A.fe & DSA_FREE_T_END);
   auto row0 = [&](int j) { return (j == 0 || tb_free) ? 0 : -(o + (j - 1) * e); };
+  uint2* scr_cta = nullptr;           // the CTA's boundary rows (two targets a lane: no registers left)
   uint32_t held = NONE;               // first strip and group size of the profile in place
 
   for (bool first = true;; first = false) {
@@ -155,15 +159,17 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
         }
         s_seg = A.segs[lo];
         s_tile = item - s_seg.item0;
-        // its longest target
-        s_row = A.tlen[A.perm[s_seg.first + s_tile * (s_seg.warps * 32 / s_seg.G) * (DUAL ? 2 : 1)]];
       }
     }
     __syncthreads();
     if (s_tile == NONE) break;
+    if (first) scr_cta = A.scratch + s_slot;
     const int G = s_seg.G, k = lane & (G - 1);
     const uint32_t ns = A.nstrips[s_seg.unit], sb = A.sbase[s_seg.unit];
-    const uint32_t in_seg = (s_tile * (s_seg.warps * 32 / G) + warp * (32 / G) + lane / G) * (DUAL ? 2 : 1);
+    const uint32_t tile0 = s_tile * (s_seg.warps * 32 / G), group = warp * (32 / G) + lane / G;
+    const uint32_t in_seg = (tile0 + group) * (DUAL ? 2 : 1);
+    // boundary rows are as long as the item's longest target, its first
+    const uint32_t row = (int)ns > G ? boundary_row(A.tlen[A.perm[s_seg.first + tile0 * (DUAL ? 2 : 1)]]) : 0;
     // the halves' targets: the same, or (DUAL) neighbours, the longer one first
     const bool valid = in_seg < s_seg.count && warp < s_seg.warps;
     const bool valid2 = DUAL ? valid && in_seg + 1 < s_seg.count : valid;
@@ -190,7 +196,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
       nmin = min(nmin, __shfl_xor_sync(FULL, nmin, w));
     }
     const uint32_t sh = 8u * (uint32_t)((uintptr_t)(t - k) & 3), sh2 = 8u * (uint32_t)((uintptr_t)(t2 - k) & 3);
-    uint2* const scr = A.scratch + s_slot + (uint64_t)(warp * (32 / G) + lane / G) * s_row;
+    uint2* const scr = (DUAL ? A.scratch + s_slot : scr_cta) + (uint64_t)group * row;
     const int steps = nmax + G - 1;
     const int nb = ((int)ns + G - 1) / G;
 
@@ -784,7 +790,8 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   auto boundary = [&](const Segment& s, uint32_t tile) -> uint64_t {
     if (ns[s.unit] <= (uint32_t)s.G) return 0;
     const uint32_t per = s.warps * 32 / s.G * halves, at = tile * per;
-    return (uint64_t)((std::min(per, s.count - at) + halves - 1) / halves) * db->h_len[db->h_perm[s.first + at]];
+    return (uint64_t)((std::min(per, s.count - at) + halves - 1) / halves) *
+           boundary_row(db->h_len[db->h_perm[s.first + at]]);
   };
   std::vector<uint64_t> slot(grid, 0);
   uint64_t largest = 0;
