@@ -288,6 +288,20 @@ int launch_intra_glob16(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, con
 // stay inside its 16-bit range.  dual (wave_dual_takes): both halves of a unit
 // follow one stream, against two targets; residues: those of the targets.
 constexpr uint32_t WAVE_LONG_TARGET = 2048;   // longer targets take up to 32 lanes
+constexpr int WAVE_FEW_LANES = 8;             // lanes per target where targets abound
+// Lanes per target of a unit of `strips` strips: as many as it has strips, up to
+// `most`; launches of fewer lane groups than the chip has room for take more.
+inline int wave_lanes(uint64_t strips, int most, uint64_t groups, uint64_t slots) {
+  int G = 4;
+  while (G < 32 && (uint64_t)G < strips && (G < most || groups * G < slots)) G *= 2;
+  return G;
+}
+// Targets longer than this take up to `most` lanes, not half as many: with that
+// half their chain, columns times bands, would pass `limit`.
+inline uint64_t wave_longest(uint64_t strips, int most, uint64_t limit) {
+  const uint64_t bands = (strips + most / 2 - 1) / (most / 2);
+  return limit / bands < WAVE_LONG_TARGET ? limit / bands : WAVE_LONG_TARGET;
+}
 int sum_bias(bool local, int o, int e, int smin);
 bool sum_fits(bool local, int64_t m, int64_t n, int o, int e, int smax, int smin);
 bool wave_takes(bool local, uint32_t max_m, uint32_t max_n, int o, int e, int smax, int smin);

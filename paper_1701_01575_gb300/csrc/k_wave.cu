@@ -74,7 +74,6 @@ namespace {
 
 constexpr int NW = 8;              // warps per CTA
 constexpr int NT = NW * 32;
-constexpr int FEW_LANES = 8;       // lanes per target where targets abound
 constexpr int PLANE = 512;         // bytes of one row quad of 32 strips
 constexpr int MIN_WARPS = 2;       // busy warps per CTA of spread launches and longest targets
 enum Form { LOCAL_SUM = 0, LOCAL_WRAP = 1, GLOBAL_SUM = 2 };
@@ -737,13 +736,12 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   std::vector<Segment> segs;
   size_t n_first = 0;
   std::vector<uint32_t> next(ns.size(), 0);   // the unit's targets dealt so far
-  for (int most = 32; most >= FEW_LANES; most /= 2) {
+  for (int most = 32; most >= WAVE_FEW_LANES; most /= 2) {
     for (uint32_t u = 0; u < ns.size(); ++u) {
       // targets whose chain on half the lanes is too long
       uint32_t end = n_targets;
-      if (most > FEW_LANES) {
-        const uint64_t bands = (ns[u] + most / 2 - 1) / (most / 2);
-        const uint64_t longest = std::min<uint64_t>(limit / bands, WAVE_LONG_TARGET);
+      if (most > WAVE_FEW_LANES) {
+        const uint64_t longest = wave_longest(ns[u], most, limit);
         end = (uint32_t)(std::partition_point(db->h_perm.begin() + next[u], db->h_perm.begin() + n_targets,
                                               [&](uint32_t t) { return db->h_len[t] > longest; }) -
                          db->h_perm.begin());
@@ -751,8 +749,7 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
       const uint32_t first = next[u], count = end - first;
       if (count == 0) continue;
       next[u] = end;
-      int G = 4;
-      while (G < 32 && (uint32_t)G < ns[u] && (G < most || n_targets / halves * ns.size() * G < slots)) G *= 2;
+      const int G = wave_lanes(ns[u], most, n_targets / halves * ns.size(), slots);
       segs.push_back({u, first, count, 0, G, NW});
       n_first += most == 32;
     }

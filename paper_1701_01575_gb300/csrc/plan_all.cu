@@ -193,22 +193,61 @@ Streams build_streams(const dsa_db* qs, const std::vector<uint32_t>& qorder, uin
   return S;
 }
 
+// Cycles of the wavefronts over the first n_groups groups of the database on
+// strips of R rows: the work, every unit's strips in whole bands of the lanes that
+// each target takes, at 4 warps a scheduler; or the longest target's chain, its
+// columns times the unit's bands, where its warp has 1.5 others beside it.  A
+// warp's step takes about 11 cycles a row and 45 (global 8 and 66) for the
+// hand-over.  Against the times of 134 searches of 1 to 100 queries of 32 to 2,300
+// and 300 to 150,000 targets up to 100,000, the height of the smaller estimate is
+// 0.3% slower than the better one on average; strips alone, without their bands,
+// chose up to 53% wrong (one query of 1,000 against 4,000 targets up to 9,000, two
+// bands either way: 24 rows 12.6 ms, 16 rows 8.8, the kernel before 11.2).
+double wave_cycles(const dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, uint32_t n_groups,
+                   uint64_t residues, uint32_t R, bool dual, bool local) {
+  const uint64_t slots = 512ull * ctx->sm_count, halves = dual ? 2 : 1, longest = db->h_glen[0];
+  uint64_t strips = 0;
+  for (uint32_t m : qs->h_len) strips += (m + R - 1) / R;
+  const uint64_t most_q = (qs->max_len + R - 1) / R;
+  // the streams that packed_score builds
+  const uint64_t lane = std::max(most_q, 32 * (strips / 2 * residues / slots / (2 * longest)));
+  uint64_t K = std::min<uint64_t>(qs->n, (strips + lane - 1) / lane);
+  const uint64_t units = dual ? K : (K + 1) / 2;
+  if (!dual) K = 2 * units;
+  const uint64_t ns = std::max(most_q, (strips + K - 1) / K);
+  const uint64_t limit = ns * units * residues / halves / slots * 3 / 5;
+  double work = 0;
+  uint32_t g = 0;
+  for (int most = 32; most >= WAVE_FEW_LANES; most /= 2) {
+    const uint64_t past = most > WAVE_FEW_LANES ? wave_longest(ns, most, limit) : 0;
+    const uint64_t G = wave_lanes(ns, most, (uint64_t)n_groups * GROUP / halves * units, slots);
+    uint64_t cols = 0;
+    for (; g < n_groups && db->h_glen[g] > past; ++g) cols += (uint64_t)db->h_glen[g] * GROUP;
+    work += (double)cols * (double)((ns + G - 1) / G * G);
+  }
+  work *= (double)units / (double)(halves * 32 * 4 * ctx->sm_count) * (dual ? 1.17 : 1.0);
+  const double chain = 2.5 * (double)((ns + 31) / 32) * (double)longest;
+  return std::max(work, chain) * (local ? 11 * R + 45 : 8 * R + 66);
+}
+
 // Strip rows of the wavefront search: 24 spread a step's hand-over over more
-// rows, 16 pad short queries less.  Cost per query: strips times (rows of
-// about 11 cycles and a hand-over of about 45).  A search whose queries fill one
-// band (32 lanes) at 8 rows, and whose lanes fill the chip three times at most,
-// lasts about as long as its longest target, so it takes the shortest steps:
+// rows, 16 pad short queries and fill some bands better.  A search whose queries
+// fill one band (32 lanes) at 8 rows, and whose lanes fill the chip three times at
+// most, lasts about as long as its longest target, so it takes the shortest steps:
 // 128 residues against 2,000 targets 0.53 ms (16 rows 0.75, 24 rows 1.01),
 // against 12,000 0.91 (1.14, 1.56).  Past one band they lose, 300 residues 1.24
 // (0.86, 1.01), and with more lanes too, 16 queries against 2,000 1.48 (1.19,
 // 1.18).
-int wave_rows(const dsa_ctx* ctx, const dsa_db* qs, uint32_t n_targets, bool dual) {
+int wave_rows(const dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, uint32_t n_targets, uint64_t residues,
+              bool dual, bool local) {
   auto strips = [&](uint32_t R) {
     uint64_t c = 0;
     for (uint32_t m : qs->h_len) c += (m + R - 1) / R;
     return c;
   };
-  auto cost = [&](uint32_t R) { return strips(R) * (R * 11 + 45); };
+  auto cost = [&](uint32_t R) {
+    return wave_cycles(ctx, db, qs, (n_targets + GROUP - 1) / GROUP, residues, R, dual, local);
+  };
   const uint64_t lanes = dual ? strips(8) : std::max<uint64_t>((qs->max_len + 7) / 8, (strips(8) + 1) / 2);
   if (lanes <= 32 && lanes * n_targets / (dual ? 2 : 1) <= 3ull * 512 * ctx->sm_count) return 8;
   return cost(16) < cost(24) ? 16 : 24;
@@ -360,7 +399,7 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
   }
   if (wave) {
     bool dual = wave_dual(qs, v, local, db->h_glen[0], o, e);
-    int wr = wave_rows(ctx, qs, n_long, dual);
+    int wr = wave_rows(ctx, db, qs, n_long, long_res, dual, local);
     // two targets a lane halve the work but not the longest target's chain: not
     // where the work, as strip columns per lane of the chip, is the shorter (one
     // query of 300 residues against 2,000 targets, global, 0.70 and 0.96 ms, of
@@ -369,7 +408,7 @@ int packed_score(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs,
       const uint64_t steps = (uint64_t)((qs->max_len + wr - 1) / wr) * long_res / (ctx->sm_count * 512ull);
       if (steps * 4 < 3ull * db->h_glen[0]) {
         dual = false;
-        wr = wave_rows(ctx, qs, n_long, dual);
+        wr = wave_rows(ctx, db, qs, n_long, long_res, dual, local);
       }
     }
     // longer streams waste fewer lanes and balance the halves better, until the
