@@ -410,9 +410,13 @@ int align_impl(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const dsa_pair*
   pp.hp_ready = all;
   if (!all) {
     const bool wave = pairs_take_wave(mode, o, e, v, n_pairs, local16, packed_ok);
-    const PairPlanParams P{qs->n, db->n, w16, o, e, local16, packed_ok, wave, v.smax, v.smin, pair_wave_wide(A),
-                           n_pairs >= 32768};
+    PairPlanParams P{qs->n, db->n, w16, o, e, local16, packed_ok, wave, v.smax, v.smin, pair_wave_wide(A),
+                           n_pairs >= 32768, mode == DSA_LOCAL};
     DSA_TRY(pairs_classify(ctx, db, qs, P, pp));
+    if (pairs_thread_form(ctx, mode, o, e, matrix, A, w16, qs->max_len, pp)) {
+      P.wave = false;
+      DSA_TRY(pairs_classify(ctx, db, qs, P, pp));
+    }
   }
   // int32 range: (m + n) * max|value step| must stay far from 2^31
   const uint32_t max_m = qs->max_len;

@@ -606,6 +606,14 @@ __host__ __device__ inline int pair_wave_class(uint64_t m, bool wide, bool dense
   // several bands of 768 or 1,024 rows, whichever computes fewer rows
   return (m + 767) / 768 * 12 < (m + 1023) / 1024 * 16 ? 14 : 15;
 }
+// Lanes and rows per block of a class.
+struct WaveClass { int G, R; };
+__host__ __device__ constexpr WaveClass wave_class(int c) {
+  constexpr WaveClass C[WAVE_CLASSES] = {{4, 8},   {2, 16},  {2, 20},  {4, 12},  {4, 16}, {4, 20},
+                                         {8, 12},  {8, 16},  {8, 20},  {16, 12}, {16, 16}, {16, 20},
+                                         {32, 12}, {32, 16}, {32, 12}, {32, 16}};
+  return C[c];
+}
 int launch_pair_wave(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const int8_t* d_matrix, int A,
                      int o, int e, int mode, uint32_t fe, int smax, int smin, const dsa_pair* d_pairs,
                      const uint32_t* d_order, const uint64_t* class_n, uint32_t max_n, Scores out);
@@ -620,6 +628,7 @@ struct PairPlanParams {
   bool wave;            // packed pairs take the wavefront kernel
   int32_t smax, smin;
   bool wide, dense;     // see pair_wave_class
+  bool local;
 };
 struct PairPlanStats {   // field order is used by the kernels' atomics
   uint64_t cells;        // cells of all valid pairs
@@ -630,6 +639,8 @@ struct PairPlanStats {   // field order is used by the kernels' atomics
   uint32_t max_t_len;    // longest window of a valid pair
   uint32_t pad;
   uint64_t cls[32];      // wave: packed pairs of each class
+  uint64_t cols16;       // columns of the packed pairs
+  uint64_t wave_cost;    // wave: what they take on the wavefronts (pairs_thread_form)
 };
 // A valid pair of m x n takes the packed kernel the call chose.
 bool pair_packed(const PairPlanParams& P, uint64_t m, uint64_t n);

@@ -66,6 +66,20 @@ int set_device(dsa_ctx* ctx) {
   return DSA_OK;
 }
 
+uint64_t memory_room(dsa_ctx* ctx) {
+  if (ctx->budget) {
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    return ctx->budget > ctx->in_use ? ctx->budget - ctx->in_use : 0;
+  }
+  size_t free = 0, total = 0;
+  uint64_t held = 0, used = 0;
+  if (cudaMemGetInfo(&free, &total) != cudaSuccess ||
+      cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+      cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+    cudaGetLastError();
+  return free + (held > used ? held - used : 0);
+}
+
 int check_matrix(const int8_t* matrix, int A, int o, int e, Validated* v) {
   if (!matrix) { set_error("matrix is NULL"); return DSA_ERR_INVALID_ARG; }
   if (o < 0 || e < 0 || e > o) {

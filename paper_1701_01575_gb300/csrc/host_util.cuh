@@ -49,6 +49,9 @@ int upload(dsa_ctx* ctx, DevBuf& buf, const std::vector<T>& v) {
 }
 
 int set_device(dsa_ctx* ctx);
+// Bytes the context can still allocate: the rest of its budget, or free memory and
+// what its pool keeps mapped.
+uint64_t memory_room(dsa_ctx* ctx);
 
 struct Validated {
   int smax = 0, smin = 0;
@@ -92,6 +95,10 @@ struct PairPass {
 bool pairs_take_wave(int mode, int o, int e, const Validated& v, uint64_t n_pairs, bool local16,
                      bool packed_ok);
 bool pair_wave_wide(int A);   // its blocks may have 20 rows
+// Classified for the wavefronts, the call's pairs are faster on the byte form of
+// the per-thread kernel.
+bool pairs_thread_form(dsa_ctx* ctx, int mode, int o, int e, const int8_t* matrix, int A, int64_t w16, uint32_t max_m,
+                       const PairPass& pp);
 // Upload (unless on the device), range-check and classify the pairs.
 int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairPlanParams& P,
                    PairPass& pp);

@@ -20,16 +20,6 @@
 namespace dsa {
 namespace {
 
-// The classes, ascending by the rows they hold in one band; the last two take
-// longer queries in several bands.
-struct WaveClass { int G, R; };
-constexpr WaveClass wave_class(int c) {
-  constexpr WaveClass C[WAVE_CLASSES] = {{4, 8},   {2, 16},  {2, 20},  {4, 12},  {4, 16}, {4, 20},
-                                         {8, 12},  {8, 16},  {8, 20},  {16, 12}, {16, 16}, {16, 20},
-                                         {32, 12}, {32, 16}, {32, 12}, {32, 16}};
-  return C[c];
-}
-
 struct WaveRange { uint32_t first, n, item0; int G, R; };   // sorted pairs and bundles of a class
 struct WaveKernelArgs {
   WaveParams W;

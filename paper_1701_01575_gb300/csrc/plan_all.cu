@@ -512,21 +512,7 @@ uint32_t fit_threshold(dsa_ctx* ctx, const dsa_db* db, uint32_t nq, uint32_t thr
   if (g == db->n_groups || db->h_glen[g] <= PLAIN_THRESHOLD) return thr;
   const uint64_t blocks = (db->n_groups - g + INTER_WARPS - 1) / INTER_WARPS;
   const uint64_t ctas = std::min<uint64_t>((nq + 1ull) / 2 * blocks, (uint64_t)inter_blocks_per_sm() * ctx->sm_count);
-  uint64_t room = 0;
-  {
-    std::lock_guard<std::mutex> lk(ctx->mu);
-    if (ctx->budget) room = ctx->budget > ctx->in_use ? ctx->budget - ctx->in_use : 0;
-  }
-  if (!ctx->budget) {   // free memory, and what the pool keeps mapped for itself
-    size_t free = 0, total = 0;
-    uint64_t held = 0, used = 0;
-    if (cudaMemGetInfo(&free, &total) != cudaSuccess ||
-        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
-        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
-      cudaGetLastError();
-    room = free + (held > used ? held - used : 0);
-  }
-  const uint64_t fits = room / 2 / (ctas * INTER_WARPS * 32 * sizeof(uint2));
+  const uint64_t fits = memory_room(ctx) / 2 / (ctas * INTER_WARPS * 32 * sizeof(uint2));
   if (db->h_glen[g] <= fits) return thr;
   return (uint32_t)std::max<uint64_t>(PLAIN_THRESHOLD, fits);
 }

@@ -51,9 +51,8 @@ int PairPass::need_hp(dsa_ctx* ctx) {
 // wavefront against per-thread form (ms): 150 bp in 500, semi-global, 1,000
 // pairs 0.15 / 1.12, 40,000 0.60 / 1.55, 300,000 3.87 / 5.21, 1,000,000 12.8 /
 // 16.5; local 1,000,000 15.4 / 18.8; 75 bp in 200, semi-global, 1,000,000 2.75 /
-// 3.92; 101 bp in 300, local, 1,000,000 8.25 / 7.98 (a third of its rows are
-// padding), the only shape measured that loses.  So the per-thread form is
-// left with scorings past the byte tables.
+// 3.92.  The per-thread form is left with scorings past the byte tables, and with
+// the calls that pairs_thread_form finds.
 bool pairs_take_wave(int mode, int o, int e, const Validated& v, uint64_t n_pairs, bool local16,
                      bool packed_ok) {
   if (!packed_ok || (mode == DSA_LOCAL && !local16) || n_pairs > UINT32_MAX) return false;
@@ -61,6 +60,35 @@ bool pairs_take_wave(int mode, int o, int e, const Validated& v, uint64_t n_pair
   const char* tune = getenv("DSA_AUTOTUNE");
   if (getenv("DSA_PAIRS_ROWS") || (tune && std::string(tune) == "retune")) return false;
   return pair_wave_tables_ok(mode == DSA_LOCAL, o, e, v.smax, v.smin);
+}
+
+// The per-thread form's boundary rows, 8 bytes per thread and column of the longest
+// window (the wavefronts need none), take at most half of the memory left.
+static bool thread_form_fits(dsa_ctx* ctx, const PairPass& pp) {
+  const uint64_t threads = std::min<uint64_t>((pp.n_pairs / 2 + 127) / 128 * 128, 512ull * ctx->sm_count);
+  const uint64_t bytes = threads * pp.pst.max_t_len * sizeof(uint2);
+  return (!ctx->budget && bytes <= 1ull << 30) || bytes <= memory_room(ctx) / 2;   // asking takes 30 us
+}
+
+// The wavefronts pad a query to its class's rows, and its window by the columns
+// that fill and drain them.  Where many pairs fill the chip and much is padding,
+// the per-thread form, whose strips of 16 or 20 rows pad less, is the faster one;
+// only its byte form is (letters of two bits).  Wavefronts and per-thread form (ms
+// a call): 1,000,000 local reads of 97 bp in 300 8.5 / 8.0, in 110 4.1 / 3.4, of 112
+// in 300 8.6 / 8.7; 500,000 of 161 in 400 9.6 / 8.5 (semi-global 7.6 / 7.5), of 193
+// in 210 7.2 / 5.5 (5.5 / 4.8); 300,000 of 321 in 340 11.7 / 8.4 (8.8 / 7.3);
+// 100,000 of 101 in 300 1.05 / 1.20.  In 10^-14 s a column, a pair takes 20 m + 300
+// (local 23 m + 290) per thread, and a call of n pairs 18,000 / n more for its last
+// ones; where the estimates of 66 shapes choose the slower form it is within 1%.
+bool pairs_thread_form(dsa_ctx* ctx, int mode, int o, int e, const int8_t* matrix, int A, int64_t w16, uint32_t max_m,
+                       const PairPass& pp) {
+  const PairPlanStats& st = pp.pst;
+  if (!pp.plan.wave || st.n_other || st.cells16 == 0 || A > 4 || !s_plus_o_fits_int8(matrix, A, o)) return false;
+  const bool local = mode == DSA_LOCAL;
+  // its range rule, for the longest pair
+  if (!local && !((int64_t)(max_m + (uint64_t)st.max_t_len) * w16 + o < 12000 && o + e < 4096)) return false;
+  const double threads = (local ? 23.0 : 20.0) * (double)st.cells16 + (local ? 290.0 : 300.0) * (double)st.cols16;
+  return threads * (1.0 + 18000.0 / (double)pp.n_pairs) < (double)st.wave_cost && thread_form_fits(ctx, pp);
 }
 
 int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairPlanParams& P,
@@ -71,7 +99,7 @@ int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairP
   pp.plan = P;
   if (pp.flags & DSA_PAIRS_ON_DEVICE) {
     pp.d_pairs = pp.pairs;
-  } else {
+  } else if (!pp.d_pairs) {
     DSA_TRY(upload(ctx, pp.d_pairs_buf, pp.pairs, n_pairs));
     pp.d_pairs = pp.d_pairs_buf.as<dsa_pair>();
   }
