@@ -56,9 +56,7 @@ int PairPass::need_hp(dsa_ctx* ctx) {
 bool pairs_take_wave(int mode, int o, int e, const Validated& v, uint64_t n_pairs, bool local16,
                      bool packed_ok) {
   if (!packed_ok || (mode == DSA_LOCAL && !local16) || n_pairs > UINT32_MAX) return false;
-  // DSA_PAIRS_ROWS fixes a variant of the per-thread form, and re-tuning times it
-  const char* tune = getenv("DSA_AUTOTUNE");
-  if (getenv("DSA_PAIRS_ROWS") || (tune && std::string(tune) == "retune")) return false;
+  if (getenv("DSA_PAIRS_ROWS")) return false;   // fixes a variant of the per-thread form
   return pair_wave_tables_ok(mode == DSA_LOCAL, o, e, v.smax, v.smin);
 }
 
@@ -68,6 +66,16 @@ static bool thread_form_fits(dsa_ctx* ctx, const PairPass& pp) {
   const uint64_t threads = std::min<uint64_t>((pp.n_pairs / 2 + 127) / 128 * 128, 512ull * ctx->sm_count);
   const uint64_t bytes = threads * pp.pst.max_t_len * sizeof(uint2);
   return (!ctx->budget && bytes <= 1ull << 30) || bytes <= memory_room(ctx) / 2;   // asking takes 30 us
+}
+
+// The byte form of the per-thread kernel holds every pair of a call that is
+// classified for the wavefronts (its range rule for the longest pair).
+static bool thread_form_holds(int mode, int o, int e, const int8_t* matrix, int A, int64_t w16, uint32_t max_m,
+                              const PairPass& pp) {
+  const PairPlanStats& st = pp.pst;
+  if (!pp.plan.wave || st.n_other || st.cells16 == 0 || A > 4 || !s_plus_o_fits_int8(matrix, A, o)) return false;
+  return mode == DSA_LOCAL ||
+         ((int64_t)(max_m + (uint64_t)st.max_t_len) * w16 + o < 12000 && o + e < 4096);
 }
 
 // The wavefronts pad a query to its class's rows, and its window by the columns
@@ -83,10 +91,8 @@ static bool thread_form_fits(dsa_ctx* ctx, const PairPass& pp) {
 bool pairs_thread_form(dsa_ctx* ctx, int mode, int o, int e, const int8_t* matrix, int A, int64_t w16, uint32_t max_m,
                        const PairPass& pp) {
   const PairPlanStats& st = pp.pst;
-  if (!pp.plan.wave || st.n_other || st.cells16 == 0 || A > 4 || !s_plus_o_fits_int8(matrix, A, o)) return false;
+  if (!thread_form_holds(mode, o, e, matrix, A, w16, max_m, pp)) return false;
   const bool local = mode == DSA_LOCAL;
-  // its range rule, for the longest pair
-  if (!local && !((int64_t)(max_m + (uint64_t)st.max_t_len) * w16 + o < 12000 && o + e < 4096)) return false;
   const double threads = (local ? 23.0 : 20.0) * (double)st.cells16 + (local ? 290.0 : 300.0) * (double)st.cols16;
   return threads * (1.0 + 18000.0 / (double)pp.n_pairs) < (double)st.wave_cost && thread_form_fits(ctx, pp);
 }
@@ -123,6 +129,77 @@ int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairP
   }
   return DSA_OK;
 }
+
+namespace {
+
+// Jobs of the per-thread form, planned on the device: stable sort by (query
+// length, window length), jobs from the runs of equal query length.
+int plan_jobs16(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, PairPass& pp, DevBuf& d_pj, uint32_t* n_pj,
+                uint32_t* max_n) {
+  DevBuf d_key2, d_idx2;
+  DSA_TRY(d_key2.alloc(ctx, pp.n_pairs * sizeof(uint64_t)));
+  DSA_TRY(d_idx2.alloc(ctx, pp.n_pairs * sizeof(uint32_t)));
+  DSA_TRY(d_pj.alloc(ctx, pp.pst.n_jobs * sizeof(Pair16Job)));
+  uint64_t* kk = pp.d_key.as<uint64_t>();
+  uint32_t* vv = pp.d_idx.as<uint32_t>();
+  DSA_TRY(launch_pair_sort(ctx, kk, vv, d_key2.as<uint64_t>(), d_idx2.as<uint32_t>(), pp.n_pairs, qs->max_len,
+                           pp.pst.max_t_len));
+  DSA_TRY(launch_pair_build_jobs(ctx, kk, vv, pp.n_pairs, pp.d_hist.as<uint64_t>(), pp.d_jcnt.as<uint64_t>(),
+                                 pp.L, pp.d_pairs, qs, db, d_pj.as<Pair16Job>()));
+  *n_pj = (uint32_t)pp.pst.n_jobs;
+  *max_n = std::max<uint32_t>(1, pp.pst.max_t_len);
+  return DSA_OK;
+}
+
+// Kernel variant of the byte form (16-row strips at 4 blocks per SM, or the wide
+// 20-row strips at 3): DSA_PAIRS_ROWS, else the autotuner, per workload shape
+// (mode, alphabet, and log2 bins of the job count, the longest query and the
+// longest window), timing both on the first call.
+template <class Launch>
+int rows_of_byte_form(dsa_ctx* ctx, const dsa_db* qs, int mode, int A, bool bytes, uint32_t n_pj, uint32_t max_n,
+                      Launch launch, int* rows) {
+  *rows = 16;
+  const int wide = pairs16_wide_rows();
+  const char* rows_env = getenv("DSA_PAIRS_ROWS");
+  const char* tune_env = getenv("DSA_AUTOTUNE");
+  if (rows_env) {
+    if (bytes && atoi(rows_env) == wide) *rows = wide;
+    return DSA_OK;
+  }
+  if (!bytes || !ctx->tune || (tune_env && std::string(tune_env) == "off")) return DSA_OK;
+  char k[160];
+  snprintf(k, sizeof k, "|pairs|%s|A%d|j%d|m%d|n%d|rows",
+           mode == DSA_LOCAL ? "local" : (mode == DSA_GLOBAL ? "global" : "semi"), A, tuner_bin(n_pj),
+           tuner_bin(qs->max_len), tuner_bin(max_n));
+  const std::string key = tuner_shape_prefix(ctx) + k;
+  uint32_t cached = 0;
+  if (tuner_get(key, &cached)) {
+    *rows = (int)cached == wide ? wide : 16;
+    return DSA_OK;
+  }
+  cudaEvent_t ev[3];
+  for (auto& x : ev) DSA_CUDA_TRY(cudaEventCreate(&x));
+  int trc = DSA_OK;
+  if (cudaEventRecord(ev[0], ctx->stream) != cudaSuccess || (trc = launch(16)) ||
+      cudaEventRecord(ev[1], ctx->stream) != cudaSuccess || (trc = launch(wide)) ||
+      cudaEventRecord(ev[2], ctx->stream) != cudaSuccess || cudaEventSynchronize(ev[2]) != cudaSuccess)
+    trc = trc ? trc : DSA_ERR_CUDA;
+  float t16 = 0.f, tw = 0.f;
+  if (!trc) {
+    cudaEventElapsedTime(&t16, ev[0], ev[1]);
+    cudaEventElapsedTime(&tw, ev[1], ev[2]);
+  }
+  for (auto& x : ev) cudaEventDestroy(x);
+  if (trc) {
+    set_error("pairs autotune: %s", cudaGetErrorString(cudaGetLastError()));
+    return trc;
+  }
+  *rows = tw < 0.97f * t16 ? wide : 16;   // a switch needs a 3% gain
+  tuner_put(key, (uint32_t)*rows);
+  return DSA_OK;
+}
+
+}  // namespace
 
 int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, PairPass& pp,
                 int mode, uint32_t fe, const int8_t* matrix, const int8_t* d_mat, int A, int o,
@@ -297,13 +374,13 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
     // (kernel, mode, and log2 bins of the pair count, the longest query and
     // the longest window) and keeps the faster (a switch needs 3%).
     int bps = l16 ? 2 : 4;
+    const bool few = l16 && bands / 2 <= (mode == DSA_LOCAL ? LONG_MANY_BANDS : LONG_FEW_BANDS) *
+                                             (uint64_t)ctx->sm_count;
     const char* bps_env = getenv("DSA_LONG_BLOCKS");
     const char* tune_env = getenv("DSA_AUTOTUNE");
     if (bps_env) {
       bps = std::min(4, std::max(1, atoi(bps_env)));
-    } else if (l16 && !(tune_env && std::string(tune_env) == "retune") &&
-               bands / 2 <= (mode == DSA_LOCAL ? LONG_MANY_BANDS : LONG_FEW_BANDS) *
-                                (uint64_t)ctx->sm_count) {
+    } else if (few && !(tune_env && std::string(tune_env) == "retune")) {
       bps = 1;
     } else if (ctx->tune && !(tune_env && std::string(tune_env) == "off")) {
       uint32_t mmax = 0, nmax = 0;
@@ -341,6 +418,7 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
         bps = t2 < 0.97f * t4 ? 2 : 4;
         tuner_put(key, (uint32_t)bps);
       }
+      if (few) bps = 1;   // re-tuning, which times the others for calls of more bands
     }
     phase_begin(res, PH_INTRA);
     if ((rc = run_long(bps))) return (rc);
@@ -353,6 +431,26 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
     DevBuf d_pj;
     uint32_t n_pj = 0, max_n = 1;
     if (wave) {
+      // re-tuning times the per-thread form's variants, although this call takes
+      // the wavefronts: calls of the same bins with other pairs may take it
+      if (const char* tune = getenv("DSA_AUTOTUNE");
+          tune && std::string(tune) == "retune" && thread_form_holds(mode, o, e, matrix, A, w16, qs->max_len, pp) &&
+          thread_form_fits(ctx, pp)) {
+        PairPass again;
+        again.pairs = d_pairs;
+        again.n_pairs = n_pairs;
+        again.flags = pp.flags | DSA_PAIRS_ON_DEVICE;
+        PairPlanParams P = pp.plan;
+        P.wave = false;
+        int rows = 16;
+        if ((rc = pairs_classify(ctx, db, qs, P, again)) ||
+            (rc = plan_jobs16(ctx, db, qs, again, d_pj, &n_pj, &max_n)) ||
+            (rc = rows_of_byte_form(ctx, qs, mode, A, true, n_pj, max_n, [&](int r) {
+               return launch_pairs16(ctx, db, qs, d_mat, A, o, e, mode, fe, v.smax, true, r, d_pj.as<Pair16Job>(),
+                                     n_pj, max_n, sc);
+             }, &rows)))
+          return rc;
+      }
       // stable sort by (class, window length); pairs of other paths last
       DevBuf d_key2, d_idx2;
       if ((rc = d_key2.alloc(ctx, n_pairs * sizeof(uint64_t))) ||
@@ -369,23 +467,7 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
         return (rc);
       phase_end(res, PH_INTER);
     } else if (dev_plan) {
-      // device planner: stable sort by (query length, window length), jobs
-      // from the runs of equal query length
-      DevBuf d_key2, d_idx2;
-      if ((rc = d_key2.alloc(ctx, n_pairs * sizeof(uint64_t))) ||
-          (rc = d_idx2.alloc(ctx, n_pairs * sizeof(uint32_t))) ||
-          (rc = d_pj.alloc(ctx, pp.pst.n_jobs * sizeof(Pair16Job))))
-        return (rc);
-      uint64_t* kk = pp.d_key.as<uint64_t>();
-      uint32_t* vv = pp.d_idx.as<uint32_t>();
-      if ((rc = launch_pair_sort(ctx, kk, vv, d_key2.as<uint64_t>(), d_idx2.as<uint32_t>(), n_pairs,
-                                 qs->max_len, pp.pst.max_t_len)) ||
-          (rc = launch_pair_build_jobs(ctx, kk, vv, n_pairs, pp.d_hist.as<uint64_t>(),
-                                       pp.d_jcnt.as<uint64_t>(), pp.L, d_pairs, qs, db,
-                                       d_pj.as<Pair16Job>())))
-        return (rc);
-      n_pj = (uint32_t)pp.pst.n_jobs;
-      max_n = std::max<uint32_t>(1, pp.pst.max_t_len);
+      if ((rc = plan_jobs16(ctx, db, qs, pp, d_pj, &n_pj, &max_n))) return (rc);
     } else {
       // order by (query length, window length); two pairs of equal query length per thread
       const unsigned T = host_threads(p16.size(), 1u << 16);
@@ -453,48 +535,8 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
       return launch_pairs16(ctx, db, qs, d_mat, A, o, e, mode, fe, v.smax, bytes, rows,
                             d_pj.as<Pair16Job>(), n_pj, max_n, sc);
     };
-    // kernel variant of the byte form (16-row strips at 4 blocks per SM, or
-    // the wide 20-row strips at 3): DSA_PAIRS_ROWS, else the autotuner, per
-    // workload shape (mode, alphabet, and log2 bins of the job count, the
-    // longest query and the longest window), timing both on the first call
     int rows = 16;
-    const int wide = pairs16_wide_rows();
-    const char* rows_env = getenv("DSA_PAIRS_ROWS");
-    const char* tune_env = getenv("DSA_AUTOTUNE");
-    if (rows_env) {
-      rows = bytes && atoi(rows_env) == wide ? wide : 16;
-    } else if (bytes && ctx->tune && !(tune_env && std::string(tune_env) == "off")) {
-      char k[160];
-      snprintf(k, sizeof k, "|pairs|%s|A%d|j%d|m%d|n%d|rows",
-               mode == DSA_LOCAL ? "local" : (mode == DSA_GLOBAL ? "global" : "semi"), A,
-               tuner_bin(n_pj), tuner_bin(qs->max_len), tuner_bin(max_n));
-      const std::string key = tuner_shape_prefix(ctx) + k;
-      uint32_t cached = 0;
-      if (tuner_get(key, &cached)) {
-        rows = (int)cached == wide ? wide : 16;
-      } else {
-        cudaEvent_t ev[3];
-        for (auto& x : ev) DSA_CUDA_TRY(cudaEventCreate(&x));
-        int trc = DSA_OK;
-        if (cudaEventRecord(ev[0], ctx->stream) != cudaSuccess || (trc = launch(16)) ||
-            cudaEventRecord(ev[1], ctx->stream) != cudaSuccess || (trc = launch(wide)) ||
-            cudaEventRecord(ev[2], ctx->stream) != cudaSuccess ||
-            cudaEventSynchronize(ev[2]) != cudaSuccess)
-          trc = trc ? trc : DSA_ERR_CUDA;
-        float t16 = 0.f, tw = 0.f;
-        if (!trc) {
-          cudaEventElapsedTime(&t16, ev[0], ev[1]);
-          cudaEventElapsedTime(&tw, ev[1], ev[2]);
-        }
-        for (auto& x : ev) cudaEventDestroy(x);
-        if (trc) {
-          set_error("pairs autotune: %s", cudaGetErrorString(cudaGetLastError()));
-          return trc;
-        }
-        rows = tw < 0.97f * t16 ? wide : 16;   // a switch needs a 3% gain
-        tuner_put(key, (uint32_t)rows);
-      }
-    }
+    if ((rc = rows_of_byte_form(ctx, qs, mode, A, bytes, n_pj, max_n, launch, &rows))) return (rc);
     phase_begin(res, PH_INTER);
     if ((rc = launch(rows))) return (rc);
     phase_end(res, PH_INTER);

@@ -1,7 +1,7 @@
 """Which packed form a call's explicit pairs take, and that its results are the
 oracle's: reads whose wavefront class is a quarter padding go to the per-thread
-form (its row tuner then leaves an entry in the cache file), others stay on the
-wavefronts."""
+form (its row tuner then leaves an entry in the cache file), others stay on
+the wavefronts, under DSA_AUTOTUNE=retune too."""
 import json
 
 import numpy as np
@@ -54,3 +54,29 @@ def test_form_and_results(ctx, mode, fe, m, window, n, per_thread, tmp_path, mon
     assert_same((h["score"], h["q_end"], h["t_end"]), want, f"m={m} mode={mode}")
     keys = json.loads(cache.read_text()) if cache.exists() else {}
     assert any("|pairs|" in k for k in keys) == per_thread
+
+
+@pytest.mark.parametrize("mode", [dsa.LOCAL, dsa.GLOBAL])
+def test_retuning_keeps_the_form(ctx, mode, tmp_path, monkeypatch):
+    """Protein pairs past the per-thread form's narrow range: on the wavefronts
+    under DSA_AUTOTUNE=retune as without it, none in int32."""
+    monkeypatch.setenv("DSA_AUTOTUNE_CACHE", str(tmp_path / "tune.json"))
+    monkeypatch.delenv("DSA_PAIRS_ROWS", raising=False)
+    rng = np.random.default_rng(7800 + mode)
+    bg = W.protein_background()
+    qs = W._make_set(rng, rng.integers(50, 1200, 60), bg)
+    db = W._make_set(rng, rng.integers(50, 1200, 90), bg)
+    pairs = np.zeros(500, W.PAIR_DTYPE)
+    pairs["query_id"], pairs["target_id"] = rng.integers(0, qs.n, 500), rng.integers(0, db.n, 500)
+    pairs["t_len"] = db.lengths[pairs["target_id"]]
+    S = W.blosum62()
+    d, q = ctx.load_set(db, 24), ctx.load_set(qs, 24)
+    launches, hits = [], []
+    for tune in ("off", "retune"):
+        monkeypatch.setenv("DSA_AUTOTUNE", tune)
+        before = ctx.kernel_launches()
+        r = ctx.align(d, q, S, 11, 1, mode=mode, pairs=pairs)
+        hits.append(r.hits().copy())
+        launches.append(ctx.kernel_launches() - before)
+        assert r.phase_cells()["int32"] == 0 and r.phase_cells()["inter16"] > 0
+    assert (hits[0] == hits[1]).all() and launches[0] == launches[1]
