@@ -411,10 +411,11 @@ int align_impl(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const dsa_pair*
   if (!all) {
     const bool wave = pairs_take_wave(mode, o, e, v, n_pairs, local16, packed_ok);
     PairPlanParams P{qs->n, db->n, w16, o, e, local16, packed_ok, wave, v.smax, v.smin, pair_wave_wide(A),
-                           n_pairs >= 32768, mode == DSA_LOCAL};
+                           n_pairs >= 32768, false, {}, {}, 0, 0, 0};
+    pairs_compare_forms(&P, n_pairs, mode, o, matrix, A);
     DSA_TRY(pairs_classify(ctx, db, qs, P, pp));
     if (pairs_thread_form(ctx, mode, o, e, matrix, A, w16, qs->max_len, pp)) {
-      P.wave = false;
+      P.wave = P.compare = false;
       DSA_TRY(pairs_classify(ctx, db, qs, P, pp));
     }
   }

@@ -628,8 +628,14 @@ struct PairPlanParams {
   bool wave;            // packed pairs take the wavefront kernel
   int32_t smax, smin;
   bool wide, dense;     // see pair_wave_class
-  bool local;
+  // the per-thread form may be the faster one: by class, what a column costs on
+  // the wavefronts, and how many columns filling and draining them stand for; what
+  // a column costs there per query row, strip of 16 rows and at all
+  bool compare;
+  uint32_t unit[WAVE_CLASSES], fill[WAVE_CLASSES];
+  uint32_t t_row, t_strip, t_col;
 };
+constexpr uint32_t THREAD_FILL = 9;   // its columns of fill
 struct PairPlanStats {   // field order is used by the kernels' atomics
   uint64_t cells;        // cells of all valid pairs
   uint64_t cells16;      // cells of the packed pairs
@@ -639,8 +645,7 @@ struct PairPlanStats {   // field order is used by the kernels' atomics
   uint32_t max_t_len;    // longest window of a valid pair
   uint32_t pad;
   uint64_t cls[32];      // wave: packed pairs of each class
-  uint64_t cols16;       // columns of the packed pairs
-  uint64_t wave_cost;    // wave: what they take on the wavefronts (pairs_thread_form)
+  uint64_t wave_cost, thread_cost;   // compare: of the packed pairs
 };
 // A valid pair of m x n takes the packed kernel the call chose.
 bool pair_packed(const PairPlanParams& P, uint64_t m, uint64_t n);

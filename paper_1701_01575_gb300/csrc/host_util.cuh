@@ -95,8 +95,10 @@ struct PairPass {
 bool pairs_take_wave(int mode, int o, int e, const Validated& v, uint64_t n_pairs, bool local16,
                      bool packed_ok);
 bool pair_wave_wide(int A);   // its blocks may have 20 rows
-// Classified for the wavefronts, the call's pairs are faster on the byte form of
-// the per-thread kernel.
+// The byte form of the per-thread kernel may be the faster one for a call that
+// takes the wavefronts: sets what the classification compares.
+void pairs_compare_forms(PairPlanParams* P, uint64_t n_pairs, int mode, int o, const int8_t* matrix, int A);
+// Classified so, the call's pairs are faster there.
 bool pairs_thread_form(dsa_ctx* ctx, int mode, int o, int e, const int8_t* matrix, int A, int64_t w16, uint32_t max_m,
                        const PairPass& pp);
 // Upload (unless on the device), range-check and classify the pairs.

@@ -35,14 +35,6 @@ __host__ __device__ inline bool takes_packed(const PairPlanParams& P, uint64_t m
   return (int64_t)(m + n) * P.w16 + P.o < 12000 && P.o + P.e < 4096;
 }
 
-// A pair on the wavefronts, in 10^-14 s of the whole chip: 2 G blocks of R rows
-// and a hand-over per column; filling, draining and the window's edges as columns.
-__device__ __forceinline__ uint64_t wave_pair_cost(int cls, uint64_t m, uint64_t n, bool local) {
-  const WaveClass c = wave_class(cls);
-  const uint64_t band = 2 * c.G * c.R, bands = (m + band - 1) / band;
-  return bands * (n + 16 + (local ? 7 : 5) * c.G) * (2 * c.G * (local ? 14 * c.R + 80 : 12 * c.R + 57));
-}
-
 // One pass over the pairs: range check (smallest bad index), the class of
 // every pair, the sort key (m << 32 | t_len) of every packed pair, the number
 // of packed pairs of every query length, and the call's totals.  Wavefront
@@ -55,7 +47,7 @@ __global__ void __launch_bounds__(PLAN_T) k_pair_classify(
   __shared__ uint64_t red[6][PLAN_T / 32];
   __shared__ uint32_t redm[PLAN_T / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  uint64_t cells = 0, c16 = 0, n_other = 0, bad = UINT64_MAX, cols = 0, cost = 0;
+  uint64_t cells = 0, c16 = 0, n_other = 0, bad = UINT64_MAX, thread = 0, wave = 0;
   uint32_t max_t = 0;
   const uint64_t stride = (uint64_t)gridDim.x * PLAN_T;
   // whole warps iterate together (warp-aggregated histogram updates)
@@ -79,8 +71,11 @@ __global__ void __launch_bounds__(PLAN_T) k_pair_classify(
           key[k] = ((uint64_t)hm << 32) | p.t_len;
           idx[k] = (uint32_t)k;
           c16 += c;
-          cols += p.t_len;
-          if (P.wave) cost += wave_pair_cost((int)hm, m, p.t_len, P.local);
+          if (P.compare) {
+            const uint64_t bands = m <= 1024 ? 1 : hm == 14 ? (m + 767) / 768 : (m + 1023) / 1024;
+            wave += bands * (p.t_len + P.fill[hm]) * P.unit[hm];
+            thread += (uint64_t)(p.t_len + THREAD_FILL) * (m * P.t_row + (m + 15) / 16 * P.t_strip + P.t_col);
+          }
         } else {
           ++n_other;
           if (P.wave) {
@@ -97,13 +92,13 @@ __global__ void __launch_bounds__(PLAN_T) k_pair_classify(
   cells = warp_sum(cells);
   c16 = warp_sum(c16);
   n_other = warp_sum(n_other);
-  cols = warp_sum(cols);
-  cost = warp_sum(cost);
+  thread = warp_sum(thread);
+  wave = warp_sum(wave);
   max_t = warp_max(max_t);
   for (int s = 16; s > 0; s >>= 1) bad = min(bad, __shfl_xor_sync(FULL, bad, s));
   if (lane == 0) {
     red[0][w] = cells; red[1][w] = c16; red[2][w] = n_other; red[3][w] = bad; redm[w] = max_t;
-    red[4][w] = cols; red[5][w] = cost;
+    red[4][w] = thread; red[5][w] = wave;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -119,7 +114,7 @@ __global__ void __launch_bounds__(PLAN_T) k_pair_classify(
     if (red[2][0]) atomicAdd(s + 2, (unsigned long long)red[2][0]);
     if (red[3][0] != UINT64_MAX) atomicMin(s + 3, (unsigned long long)red[3][0]);
     if (redm[0]) atomicMax(&st->max_t_len, redm[0]);
-    if (red[4][0]) atomicAdd(reinterpret_cast<unsigned long long*>(&st->cols16), (unsigned long long)red[4][0]);
+    if (red[4][0]) atomicAdd(reinterpret_cast<unsigned long long*>(&st->thread_cost), (unsigned long long)red[4][0]);
     if (red[5][0]) atomicAdd(reinterpret_cast<unsigned long long*>(&st->wave_cost), (unsigned long long)red[5][0]);
   }
 }

@@ -85,16 +85,30 @@ static bool thread_form_holds(int mode, int o, int e, const int8_t* matrix, int 
 // a call): 1,000,000 local reads of 97 bp in 300 8.5 / 8.0, in 110 4.1 / 3.4, of 112
 // in 300 8.6 / 8.7; 500,000 of 161 in 400 9.6 / 8.5 (semi-global 7.6 / 7.5), of 193
 // in 210 7.2 / 5.5 (5.5 / 4.8); 300,000 of 321 in 340 11.7 / 8.4 (8.8 / 7.3);
-// 100,000 of 101 in 300 1.05 / 1.20.  In 10^-14 s a column, a pair takes 20 m + 300
-// (local 23 m + 290) per thread, and a call of n pairs 18,000 / n more for its last
-// ones; where the estimates of 66 shapes choose the slower form it is within 1%.
+// 100,000 of 101 in 300 1.05 / 1.20; 1,000,000 of 36 in 100 1.80 / 1.53, of 50
+// 1.85 / 2.12.  The estimates (10^-15 s a column of the whole chip, fitted to 90
+// such calls): wavefronts 2 G blocks of R rows and a hand-over; per-thread form rows,
+// strips and a constant, and 18,000 / n more for the last of n pairs.
+// Calls of fewer pairs leave most of its threads without one.
+constexpr uint64_t THREAD_FORM_PAIRS = 65536;
+void pairs_compare_forms(PairPlanParams* P, uint64_t n_pairs, int mode, int o, const int8_t* matrix, int A) {
+  P->compare = P->wave && n_pairs >= THREAD_FORM_PAIRS && A <= 4 && s_plus_o_fits_int8(matrix, A, o);
+  const bool local = mode == DSA_LOCAL;
+  for (int c = 0; c < WAVE_CLASSES; ++c) {
+    const WaveClass w = wave_class(c);
+    P->unit[c] = (uint32_t)(20 * w.G * (local ? 14 * w.R + 80 : 12 * w.R + 57));
+    P->fill[c] = (uint32_t)(16 + (local ? 7 : 5) * w.G);
+  }
+  P->t_row = local ? 168 : 141;
+  P->t_strip = local ? 830 : 750;
+  P->t_col = local ? 2700 : 3350;
+}
 bool pairs_thread_form(dsa_ctx* ctx, int mode, int o, int e, const int8_t* matrix, int A, int64_t w16, uint32_t max_m,
                        const PairPass& pp) {
   const PairPlanStats& st = pp.pst;
-  if (!thread_form_holds(mode, o, e, matrix, A, w16, max_m, pp)) return false;
-  const bool local = mode == DSA_LOCAL;
-  const double threads = (local ? 23.0 : 20.0) * (double)st.cells16 + (local ? 290.0 : 300.0) * (double)st.cols16;
-  return threads * (1.0 + 18000.0 / (double)pp.n_pairs) < (double)st.wave_cost && thread_form_fits(ctx, pp);
+  if (!pp.plan.compare || !thread_form_holds(mode, o, e, matrix, A, w16, max_m, pp)) return false;
+  return (double)st.thread_cost * (1.0 + 18000.0 / (double)pp.n_pairs) < (double)st.wave_cost &&
+         thread_form_fits(ctx, pp);
 }
 
 int pairs_classify(dsa_ctx* ctx, const dsa_db* db, const dsa_db* qs, const PairPlanParams& P,
@@ -441,7 +455,7 @@ int score_pairs(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db* qs, 
         again.n_pairs = n_pairs;
         again.flags = pp.flags | DSA_PAIRS_ON_DEVICE;
         PairPlanParams P = pp.plan;
-        P.wave = false;
+        P.wave = P.compare = false;
         int rows = 16;
         if ((rc = pairs_classify(ctx, db, qs, P, again)) ||
             (rc = plan_jobs16(ctx, db, qs, again, d_pj, &n_pj, &max_n)) ||
