@@ -512,7 +512,9 @@ uint32_t fit_threshold(dsa_ctx* ctx, const dsa_db* db, uint32_t nq, uint32_t thr
   if (g == db->n_groups || db->h_glen[g] <= PLAIN_THRESHOLD) return thr;
   const uint64_t blocks = (db->n_groups - g + INTER_WARPS - 1) / INTER_WARPS;
   const uint64_t ctas = std::min<uint64_t>((nq + 1ull) / 2 * blocks, (uint64_t)inter_blocks_per_sm() * ctx->sm_count);
-  const uint64_t fits = memory_room(ctx) / 2 / (ctas * INTER_WARPS * 32 * sizeof(uint2));
+  const uint64_t column = ctas * INTER_WARPS * 32 * sizeof(uint2);
+  if (!ctx->budget && column * db->h_glen[g] <= 4ull << 30) return thr;   // asking takes 30 us
+  const uint64_t fits = memory_room(ctx) / 2 / column;
   if (db->h_glen[g] <= fits) return thr;
   return (uint32_t)std::max<uint64_t>(PLAIN_THRESHOLD, fits);
 }
