@@ -590,37 +590,48 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
     const auto k = std::make_pair(groups_over(thr), rows);
     auto it = timed.find(k);
     if (it != timed.end()) return it->second;
-    float ms = 0.f;
-    if (rc == DSA_OK && cudaEventRecord(ev0, ctx->stream) != cudaSuccess) rc = DSA_ERR_CUDA;
-    if (rc == DSA_OK) rc = run(nullptr, thr, rows);
-    if (rc == DSA_OK && cudaEventRecord(ev1, ctx->stream) != cudaSuccess) rc = DSA_ERR_CUDA;
-    if (rc == DSA_OK && cudaEventSynchronize(ev1) != cudaSuccess) rc = DSA_ERR_CUDA;
-    if (rc == DSA_OK) cudaEventElapsedTime(&ms, ev0, ev1);
-    timed[k] = ms;
-    return ms;
-  };
-  // 1. the kernel variant (strip rows) at the default threshold; a switch
-  //    from the default needs a gain of at least 3% (single timings)
-  int best_rows = rows_default;
-  double best_ms = measure(thr_default, best_rows);
-  if (!rows_forced && groups_over(thr_default) < db->n_groups)
-    for (int rows : {INTER_ROWS_SHORT}) {
-      const double ms = measure(thr_default, rows);
-      if (ms < 0.97 * best_ms) { best_ms = ms; best_rows = rows; }
+    float best_ms = 0.f;
+    for (int pass = 0; pass < 2 && rc == DSA_OK && (pass == 0 || best_ms < 50.f); ++pass) {
+      float ms = 0.f;   // short passes twice: one alone is off by more than 3% at times
+      if (cudaEventRecord(ev0, ctx->stream) != cudaSuccess) rc = DSA_ERR_CUDA;
+      if (rc == DSA_OK) rc = run(nullptr, thr, rows);
+      if (rc == DSA_OK && cudaEventRecord(ev1, ctx->stream) != cudaSuccess) rc = DSA_ERR_CUDA;
+      if (rc == DSA_OK && cudaEventSynchronize(ev1) != cudaSuccess) rc = DSA_ERR_CUDA;
+      if (rc == DSA_OK) cudaEventElapsedTime(&ms, ev0, ev1);
+      best_ms = pass ? std::min(best_ms, ms) : ms;
     }
-  // 2. the long-target threshold: every target on the wavefronts, then a local
-  //    search from the default by factors of 4 in each direction while it
-  //    improves; thresholds that move the same groups as the last one are skipped
+    timed[k] = best_ms;
+    return best_ms;
+  };
+  // 1. the kernel variant (strip rows) at the default threshold, or, where that
+  //    leaves the inter-sequence kernel no group, at the plain one (8 queries of 32
+  //    against 150,000 targets: 4.5 ms on the wavefronts, 3.8 on 20-row strips); a
+  //    switch from the default needs a gain of at least 3%.  An untimed pass comes
+  //    before them: a shape's first one also maps its scratch and loads its kernels,
+  //    and whatever was timed second had won by that.
+  int best_rows = rows_default;
   uint32_t best = thr_default;
+  rc = run(nullptr, thr_default, best_rows);
+  double best_ms = measure(thr_default, best_rows);
+  const uint32_t thr_inter =
+      thr_env || groups_over(thr_default) < db->n_groups ? thr_default : fit(PLAIN_THRESHOLD);
+  if (!rows_forced && groups_over(thr_inter) < db->n_groups) {
+    const double ms = measure(thr_inter, INTER_ROWS_SHORT);
+    if (ms < 0.97 * best_ms) { best_ms = ms; best = thr_inter; best_rows = INTER_ROWS_SHORT; }
+  }
+  // 2. the long-target threshold: every target on the wavefronts, then a local
+  //    search from the best so far by factors of 4 in each direction while it
+  //    improves; thresholds that move the same groups as the last one are skipped
   if (!thr_env) {
-    if (thr_default) {
+    if (best) {
       const double ms = measure(0, best_rows);
       if (ms < 0.97 * best_ms) { best_ms = ms; best = 0; }
     }
-    const uint64_t start = std::max<uint32_t>(thr_default, 1024);
+    const uint32_t from = best ? best : thr_default;
+    const uint64_t start = std::max<uint32_t>(from, 1024);
     for (int dir = -1; dir <= 1 && rc == DSA_OK; dir += 2) {
       uint64_t cur = start;
-      uint32_t last_g = groups_over(thr_default);
+      uint32_t last_g = groups_over(from);
       for (int step = 0; step < 12 && rc == DSA_OK; ++step) {
         const uint64_t nx = dir < 0 ? cur / 4 : cur * 4;
         const uint32_t thr = (dir > 0 && nx >= db->max_len) ? UINT32_MAX : (uint32_t)nx;
