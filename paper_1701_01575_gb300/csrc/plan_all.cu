@@ -26,8 +26,8 @@ namespace {
 // results): the strip height of the inter-sequence kernel (28 rows, or 20
 // rows, which wastes fewer padding rows on short queries), and which
 // targets go to the wavefront kernel (long) and which to the inter-sequence
-// kernel.  For a workload shape (GPU, driver, mode, alphabet,
-// and log2 bins of the query count, query residues, longest query, target
+// kernel.  For a workload shape (GPU, driver, kernel form, mode, alphabet,
+// how far the queries fill their strips, and log2 bins of the query count, query residues, longest query, target
 // count, database residues and longest target) the first call times each
 // strip height at the modelled threshold (a switch needs a 3% gain), then
 // every target on the wavefronts, then a local search of thresholds lower and
@@ -547,9 +547,11 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   const uint32_t thr_default = thr_env ? thr_forced : fit(model_threshold(db, qs, v, local, o, e));
   if (tmode == "off" || (rows_forced && thr_env))
     return run(res, thr_default, rows_default);
-  // workload shape key: GPU, driver, mode, alphabet, and log2 bins of the
-  // query count, query residues, longest query, target count, database
-  // residues and longest target
+  // workload shape key: GPU, driver, the form of the wavefronts (summed, two
+  // targets a lane, wrapping, or k_intra.cu's kernel) and, in eighths, how much of
+  // the inter-sequence kernel's 28-row and the wavefronts' 16-row strips the
+  // queries fill, mode, alphabet, and log2 bins of the query count, query
+  // residues, longest query, target count, database residues and longest target
   uint64_t qres = 0;
   uint32_t qmax = 0;
   for (uint32_t x : qs->h_len) { qres += x; qmax = std::max(qmax, x); }
@@ -557,9 +559,19 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   DSA_CUDA_TRY(cudaGetDeviceProperties(&prop, ctx->device));
   int drv = 0;
   cudaDriverGetVersion(&drv);
+  const uint32_t longest = db->h_glen[0];
+  const char form = wave_dual(qs, v, local, longest, o, e)                          ? 'd'
+                    : sum_fits(local, qs->max_len, longest, o, e, v.smax, v.smin)   ? 's'
+                    : wave_takes(local, qs->max_len, longest, o, e, v.smax, v.smin) ? 'w'
+                                                                                    : 'i';
+  auto eighths = [&](uint32_t R) {
+    uint64_t rows = 0;
+    for (uint32_t m : qs->h_len) rows += (m + R - 1) / R * R;
+    return (unsigned)std::min<uint64_t>(99, 8 * rows / qres);
+  };
   char key[512];
-  snprintf(key, sizeof key, "%s|sm%d|drv%d|wave|%s|A%d|q%d|qr%d|qm%d|t%d|tr%d|L%d", prop.name,
-           ctx->sm_count, drv, local ? "local" : (mode == DSA_GLOBAL ? "global" : "semi"), A,
+  snprintf(key, sizeof key, "%s|sm%d|drv%d|wave %c%u.%u|%s|A%d|q%d|qr%d|qm%d|t%d|tr%d|L%d", prop.name,
+           ctx->sm_count, drv, form, eighths(INTER_ROWS), eighths(16), local ? "local" : (mode == DSA_GLOBAL ? "global" : "semi"), A,
            ilog2_bin(qs->n), ilog2_bin(qres), ilog2_bin(qmax), ilog2_bin(db->n),
            ilog2_bin(db->n_res), ilog2_bin(db->max_len));
   const std::string key_thr = std::string(key) + "|thr", key_rows = std::string(key) + "|rows";
