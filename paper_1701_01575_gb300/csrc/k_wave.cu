@@ -42,12 +42,13 @@
 // padding residue, under which a strip's column-0 state is a fixed point.
 //
 // Boundary rows.  Lane 0 reads the band above one column ahead of its use.  A
-// global step of 8 or 16 rows is shorter than that load takes, and the compiler
+// global step of 16 rows is shorter than that load takes, and the compiler
 // waits for it in every step (776 of 1,440 cycles, long scoreboard), so there
 // lanes 0 to 3 load the next block's four columns a block ahead and hand them
 // over by two shuffles a step: 24 queries of 175 against 20,000 targets, global,
 // 12.2 -> 6.3 ms, 7 of 90-1,100 against 50,000 with 16 rows forced 19.6 -> 6.9.
-// Steps of 24 rows and local ones are long enough (0 to 7% slower that way).
+// Steps of 24 rows and local ones are long enough (0 to 7% slower that way), and
+// 8 rows are for searches of one band (6% slower).
 //
 // End cells.  Local: a column maximum above the best of the strip's query so
 // far (as known to the lane: shared along the query's lanes every 32 steps)
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(NT, 2) k_wave(const WaveArgs A) {
   constexpr uint32_t BIAS2 = 0x80008000u;
   constexpr int RS = DUAL ? 32 * R : R / 4 * PLANE;   // profile bytes per residue
   constexpr int MIN_SLOTS = DUAL ? 16 : 8;
-  constexpr bool BLOCK_IN = !LOCAL && R < 24;         // see "Boundary rows"
+  constexpr bool BLOCK_IN = !LOCAL && R == 16;        // see "Boundary rows"
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ Segment s_seg;
   __shared__ uint32_t s_tile;
