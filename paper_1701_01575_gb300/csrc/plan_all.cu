@@ -29,9 +29,9 @@ namespace {
 // kernel.  For a workload shape (GPU, driver, kernel form, mode, alphabet,
 // how far the queries fill their strips, and log2 bins of the query count, query residues, longest query, target
 // count, database residues and longest target) the first call times each
-// strip height at the modelled threshold (a switch needs a 3% gain), then
+// strip height at the modelled threshold (a switch needs a 2% gain), then
 // every target on the wavefronts, then a local search of thresholds lower and
-// higher by factors of 4 while it keeps improving by 3% or more -- and keeps
+// higher by factors of 4 while it keeps improving by 2% or more -- and keeps
 // both in a JSON cache file.  DSA_AUTOTUNE=off (28 rows, the model) | cache
 // (default: tune on a miss) | retune (always tune); DSA_AUTOTUNE_CACHE names
 // the file (default $XDG_CACHE_HOME/dsa/autotune.json or
@@ -618,7 +618,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   // 1. the kernel variant (strip rows) at the default threshold, or, where that
   //    leaves the inter-sequence kernel no group, at the plain one (8 queries of 32
   //    against 150,000 targets: 4.5 ms on the wavefronts, 3.8 on 20-row strips); a
-  //    switch from the default needs a gain of at least 3%.  An untimed pass comes
+  //    switch from the default needs a gain of at least 2%.  An untimed pass comes
   //    before them: a shape's first one also maps its scratch and loads its kernels,
   //    and whatever was timed second had won by that.
   int best_rows = rows_default;
@@ -629,7 +629,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
       thr_env || groups_over(thr_default) < db->n_groups ? thr_default : fit(PLAIN_THRESHOLD);
   if (!rows_forced && groups_over(thr_inter) < db->n_groups) {
     const double ms = measure(thr_inter, INTER_ROWS_SHORT);
-    if (ms < 0.97 * best_ms) { best_ms = ms; best = thr_inter; best_rows = INTER_ROWS_SHORT; }
+    if (ms < 0.98 * best_ms) { best_ms = ms; best = thr_inter; best_rows = INTER_ROWS_SHORT; }
   }
   // 2. the long-target threshold: every target on the wavefronts, then a local
   //    search from the best so far by factors of 4 in each direction while it
@@ -637,7 +637,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   if (!thr_env) {
     if (best) {
       const double ms = measure(0, best_rows);
-      if (ms < 0.97 * best_ms) { best_ms = ms; best = 0; }
+      if (ms < 0.98 * best_ms) { best_ms = ms; best = 0; }
     }
     const uint32_t from = best ? best : thr_default;
     const uint64_t start = std::max<uint32_t>(from, 1024);
@@ -656,7 +656,7 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
         last_g = g;
         if (fit(thr) != thr) break;
         const double ms = measure(thr, best_rows);
-        if (ms < 0.97 * best_ms) {
+        if (ms < 0.98 * best_ms) {
           best_ms = ms;
           best = thr;
         } else {
