@@ -1,7 +1,8 @@
 // Packed int16x2 kernel for explicit short pairs of the map phase (Sec. II.B.1,
 // any of the three algorithms of Sec. II.C.2) whose scoring the byte tables of
-// the pair wavefronts (pairwave.cuh), faster at every size measured, do not
-// hold: one thread aligns two pairs at once, one in each 16-bit half of every
+// the pair wavefronts (pairwave.cuh) do not hold, and for large calls of pairs
+// that those would mostly pad (pairs_thread_form in plan_pairs.cu, byte form
+// only): one thread aligns two pairs at once, one in each 16-bit half of every
 // DP register.  The two pairs of a thread have the same query length
 // (pairs are sorted by query length, then window length), so the strips and
 // the row of the query's last residue line up in both halves.

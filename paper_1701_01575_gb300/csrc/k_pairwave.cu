@@ -5,7 +5,8 @@
 // size and the rows per block, so that a query wastes at most a third of its
 // rows, and the groups of a warp hold pairs of nearly equal work.  Persistent
 // warps pop bundles of 32 / G pairs, the costliest class and the longest
-// windows first.
+// windows first.  Large calls of pairs that the classes mostly pad take the
+// per-thread form (pairs_thread_form).
 //
 // Bound by the ALU pipe and, at the end of a call, by the longest pair's
 // chain.  Measured against the forms it replaces (whole call): 20,000 protein

@@ -57,7 +57,8 @@
 // merges with the earlier bands' result.  Global and semi-global: as in the
 // inter-sequence kernel (column n parked, row m tracked).
 //
-// Bound by the ALU pipe; 128 registers keep 16 warps per SM.  Measured (whole
+// Bound by the ALU pipe; 128 registers keep 16 warps per SM (the local summed form
+// on strips of 24 rows spills 12 bytes, 20 with two targets a lane).  Measured (whole
 // score pass, before: the inter-sequence kernel with the longest targets on
 // the wavefronts of k_intra.cu): 7 queries of 90-1,100 against 50,011 targets,
 // global, 16.1 -> 7.5 ms (7,200 GCUPS); 5 of 60-700 against 60,000, local, 17.1

@@ -29,6 +29,8 @@ namespace dsa {
 //   5.7          14.9  16.7  15.0  13.4         13.0  21.5  16.1  16.2
 //   8.0          26.2  27.9  31.1  24.5         23.8  36.0  35.4  27.9
 //   16           47.9  30.8  52.9  39.2         43.6  41.4  59.2  44.9
+// (At 1.2 bands one block and two are the same launch, fewer blocks than SMs: those
+// columns differ by their runs alone.)
 constexpr uint64_t LONG_FEW_BANDS = 4, LONG_MANY_BANDS = 9;
 
 int PairPass::need_hp(dsa_ctx* ctx) {
