@@ -602,9 +602,13 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
     const auto k = std::make_pair(groups_over(thr), rows);
     auto it = timed.find(k);
     if (it != timed.end()) return it->second;
+    // Short passes run twice, one alone being off by more than 3% at times; the first
+    // of a shape also when it is longer, because it maps scratch and loads kernels,
+    // and whatever was timed second had won by that.
+    const float twice = timed.empty() ? 500.f : 50.f;
     float best_ms = 0.f;
-    for (int pass = 0; pass < 2 && rc == DSA_OK && (pass == 0 || best_ms < 50.f); ++pass) {
-      float ms = 0.f;   // short passes twice: one alone is off by more than 3% at times
+    for (int pass = 0; pass < 2 && rc == DSA_OK && (pass == 0 || best_ms < twice); ++pass) {
+      float ms = 0.f;
       if (cudaEventRecord(ev0, ctx->stream) != cudaSuccess) rc = DSA_ERR_CUDA;
       if (rc == DSA_OK) rc = run(nullptr, thr, rows);
       if (rc == DSA_OK && cudaEventRecord(ev1, ctx->stream) != cudaSuccess) rc = DSA_ERR_CUDA;
@@ -618,12 +622,9 @@ int run_packed_tuned(dsa_ctx* ctx, dsa_res* res, const dsa_db* db, const dsa_db*
   // 1. the kernel variant (strip rows) at the default threshold, or, where that
   //    leaves the inter-sequence kernel no group, at the plain one (8 queries of 32
   //    against 150,000 targets: 4.5 ms on the wavefronts, 3.8 on 20-row strips); a
-  //    switch from the default needs a gain of at least 2%.  An untimed pass comes
-  //    before them: a shape's first one also maps its scratch and loads its kernels,
-  //    and whatever was timed second had won by that.
+  //    switch from the default needs a gain of at least 2%
   int best_rows = rows_default;
   uint32_t best = thr_default;
-  rc = run(nullptr, thr_default, best_rows);
   double best_ms = measure(thr_default, best_rows);
   const uint32_t thr_inter =
       thr_env || groups_over(thr_default) < db->n_groups ? thr_default : fit(PLAIN_THRESHOLD);
