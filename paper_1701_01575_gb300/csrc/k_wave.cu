@@ -844,7 +844,8 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   memcpy(host.data() + b_seg + b_meta + 2 * b_u, slot.data(), grid * 8);
   const size_t b_prof = ((size_t)P.n_strips * (A + 1) * rows * (dual ? 1 : 4) + 15) & ~(size_t)15;
   void* buf = nullptr;
-  const size_t b_all = host.size() + b_prof + b_scr + 16;
+  const size_t at_scr = (host.size() + b_prof + 127) & ~(size_t)127;
+  const size_t b_all = at_scr + b_scr + 16;
   DSA_TRY(ctx->alloc(&buf, b_all, stream));
   uint8_t* d = static_cast<uint8_t*>(buf);
   cudaError_t err = cudaMemcpyAsync(d, host.data(), host.size(), cudaMemcpyHostToDevice, stream);
@@ -853,7 +854,7 @@ int launch_wave_search(dsa_ctx* ctx, cudaStream_t stream, const dsa_db* db, cons
   W.sbase = reinterpret_cast<const uint32_t*>(d + b_seg + b_meta);
   W.nstrips = reinterpret_cast<const uint32_t*>(d + b_seg + b_meta + b_u);
   W.prof = P.prof = reinterpret_cast<uint32_t*>(d + host.size());
-  W.scratch = reinterpret_cast<uint2*>(d + host.size() + b_prof);
+  W.scratch = reinterpret_cast<uint2*>(d + at_scr);
   W.slot = reinterpret_cast<const uint64_t*>(d + b_seg + b_meta + 2 * b_u);
   W.n_segs = (uint32_t)segs.size();
   W.n_items = items;
